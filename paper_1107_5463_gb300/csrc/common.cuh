@@ -62,6 +62,28 @@ struct Partial {
     double f[4];
 };
 
+// Division of n < 2^31 by a divisor fixed for a launch: a multiply-high and a
+// shift in place of the some 20 instructions of a 32-bit division (and 70 of a
+// 64-bit one).  With 2^(s-1) < d <= 2^s and m = ceil(2^(31+s) / d) < 2^32 the
+// error m d - 2^(31+s) is below 2^s, so n m >> (31 + s) is exact for n < 2^31.
+struct FastDiv {
+    uint32_t d, m, s;
+    __host__ __device__ uint32_t div(uint32_t n) const
+    {
+        return (uint32_t)(((uint64_t)n * m) >> (31 + s));
+    }
+};
+
+__host__ inline FastDiv make_fast_div(uint32_t d)
+{
+    FastDiv f;
+    f.d = d;
+    f.s = 0;
+    while (((uint64_t)1 << f.s) < d) ++f.s;
+    f.m = (uint32_t)((((uint64_t)1 << (31 + f.s)) + d - 1) / d);
+    return f;
+}
+
 // Fold one value across a warp (any type with operator+).
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v)

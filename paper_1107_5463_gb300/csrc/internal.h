@@ -63,6 +63,8 @@ struct sl_lattice {
     // views into the device buffer
     void* spins[2];          // per colour
     void* bonds[2][3];       // per colour, per direction (null for uniform J)
+    void* buf;               // the device buffer the views lie in
+    size_t buf_bytes;
     void* staging;           // natural-order staging area
     size_t staging_bytes;
     spinmc::Ctrl* ctrl;

@@ -244,37 +244,72 @@ __global__ void bits_init_kernel(uint32_t* s0, uint32_t* s1, long long nwords, u
 
 // natural +-1 bytes -> bit words: word (row r, w) of colour c holds natural
 // sites r L + 64 w + 2 b + p, p = (y + z + c) & 1
-__global__ void bits_scatter_kernel(uint32_t* s0, uint32_t* s1, const int8_t* nat, long long nwords,
-                                    int L, int WW, int par)
+// Natural order <-> colour words, bound by the natural array's bytes.  The
+// gather gives 16 natural bytes to a thread (8 bits of each colour's word,
+// four threads share a word), the scatter 64 (one word of each colour).  One
+// thread per natural byte with two 64-bit divisions took 503 us for 1.3e8
+// sites (0.27 TB/s).
+struct BitLay {
+    uint32_t *s0, *s1;
+    int8_t* nat;
+    uint32_t nwords;  // words per colour
+    FastDiv WW, L;    // words per row, lattice side
+    int par;          // parity of the first plane's global index
+};
+
+// colour of the even-x sites of the row that holds word w
+__device__ __forceinline__ int even_colour(const BitLay& a, uint32_t w)
 {
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < 2 * nwords;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(q / nwords);
-        const long long wi = q % nwords;
-        const long long r = wi / WW;
-        const int w = (int)(wi % WW);
-        const int y = (int)(r % L), z = (int)(r / L);
-        const int p = (y + z + c + par) & 1;
-        const long long base = r * L + 64LL * w + p;
-        uint32_t word = 0;
-        for (int b = 0; b < 32; ++b)
-            if (nat[base + 2 * b] < 0) word |= 1u << b;
-        (c ? s1 : s0)[wi] = word;
+    const uint32_t row = a.WW.div(w);  // z L + y; L is even, so row and y agree mod 2
+    return (int)((row + a.L.div(row) + (uint32_t)a.par) & 1u);
+}
+
+// bits 0-3 of b -> bytes +1 (0) / -1 (1)
+__device__ __forceinline__ uint32_t nibble_signs(uint32_t b)
+{
+    return 0x01010101u ^ ((((b & 0xFu) * 0x00204081u) & 0x01010101u) * 0xFEu);
+}
+
+// sign bits of four bytes -> bits 0-3
+__device__ __forceinline__ uint32_t signs_nibble(uint32_t v)
+{
+    return (((v >> 7) & 0x01010101u) * 0x10204080u) >> 28;
+}
+
+__global__ void __launch_bounds__(256) bits_gather_kernel(const BitLay a)
+{
+    const uint32_t items = 4 * a.nwords;  // H <= 2e9: below 2^28
+    for (uint32_t it = blockIdx.x * blockDim.x + threadIdx.x; it < items;
+         it += gridDim.x * blockDim.x) {
+        const uint32_t w = it >> 2, sub = 8 * (it & 3);
+        const int ce = even_colour(a, w);
+        const uint32_t ev = (ce ? a.s1 : a.s0)[w] >> sub;
+        const uint32_t ov = (ce ? a.s0 : a.s1)[w] >> sub;
+        const uint32_t e0 = nibble_signs(ev), e1 = nibble_signs(ev >> 4);
+        const uint32_t o0 = nibble_signs(ov), o1 = nibble_signs(ov >> 4);
+        *reinterpret_cast<uint4*>(a.nat + 16 * (size_t)it) =
+            make_uint4(__byte_perm(e0, o0, 0x5140), __byte_perm(e0, o0, 0x7362),
+                       __byte_perm(e1, o1, 0x5140), __byte_perm(e1, o1, 0x7362));
     }
 }
 
-__global__ void bits_gather_kernel(const uint32_t* s0, const uint32_t* s1, int8_t* nat, long long N,
-                                   int L, int par)
+__global__ void __launch_bounds__(256) bits_scatter_kernel(const BitLay a)
 {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % L);
-        const long long r = i / L;
-        const int y = (int)(r % L), z = (int)(r / L);
-        const int c = (x + y + z + par) & 1;
-        const long long j = i >> 1;  // = r W + (x >> 1)
-        const uint32_t word = (c ? s1 : s0)[j >> 5];
-        nat[i] = ((word >> (j & 31)) & 1u) ? (int8_t)-1 : (int8_t)1;
+    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < a.nwords;
+         w += gridDim.x * blockDim.x) {
+        const int ce = even_colour(a, w);
+        const uint4* n = reinterpret_cast<const uint4*>(a.nat + 64 * (size_t)w);
+        uint32_t ev = 0, ov = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint4 v = n[q];
+            ev |= (signs_nibble(__byte_perm(v.x, v.y, 0x6420)) |
+                   signs_nibble(__byte_perm(v.z, v.w, 0x6420)) << 4) << (8 * q);
+            ov |= (signs_nibble(__byte_perm(v.x, v.y, 0x7531)) |
+                   signs_nibble(__byte_perm(v.z, v.w, 0x7531)) << 4) << (8 * q);
+        }
+        (ce ? a.s1 : a.s0)[w] = ev;
+        (ce ? a.s0 : a.s1)[w] = ov;
     }
 }
 
@@ -367,18 +402,28 @@ cudaError_t ising_bits_init(const sl_lattice* h, cudaStream_t s)
     return cudaGetLastError();
 }
 
+static BitLay bits_layout(const sl_lattice* h, const int8_t* nat)
+{
+    BitLay a;
+    a.s0 = (uint32_t*)h->spins[0];
+    a.s1 = (uint32_t*)h->spins[1];
+    a.nat = const_cast<int8_t*>(nat);
+    a.nwords = (uint32_t)(h->H / 32);
+    a.WW = make_fast_div((uint32_t)(h->W / 32));
+    a.L = make_fast_div((uint32_t)h->L);
+    a.par = h->z0 & 1;
+    return a;
+}
+
 cudaError_t ising_bits_scatter(const sl_lattice* h, const int8_t* nat, cudaStream_t s)
 {
-    const long long nwords = h->H / 32;
-    bits_scatter_kernel<<<grid_for(2 * nwords, 256), 256, 0, s>>>(
-        (uint32_t*)h->spins[0], (uint32_t*)h->spins[1], nat, nwords, h->L, h->W / 32, h->z0 & 1);
+    bits_scatter_kernel<<<grid_for(h->H / 32, 256), 256, 0, s>>>(bits_layout(h, nat));
     return cudaGetLastError();
 }
 
 cudaError_t ising_bits_gather(const sl_lattice* h, int8_t* nat, cudaStream_t s)
 {
-    bits_gather_kernel<<<grid_for(h->N, 256), 256, 0, s>>>(
-        (const uint32_t*)h->spins[0], (const uint32_t*)h->spins[1], nat, h->N, h->L, h->z0 & 1);
+    bits_gather_kernel<<<grid_for(h->H / 8, 256), 256, 0, s>>>(bits_layout(h, nat));
     return cudaGetLastError();
 }
 

@@ -3,6 +3,8 @@
 // sweep scheduling (plain launches or replays of a captured CUDA graph), and
 // measurement / state transfer.  Every compute step runs in the kernels of
 // the per-model .cu files.
+#include <cuda.h>  // types only; the one driver function is looked up at run time
+
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -270,6 +272,37 @@ size_t nat_bytes(const sl_lattice* h)
     return (size_t)h->N * (h->n == 1 ? 1 : (h->n == 2 ? 4 : 12));
 }
 
+// Whether the layout kernels may work on the caller's natural-order array in
+// place of the staging area (saving a copy of the whole array): 16-byte
+// aligned memory of the lattice's own device, every byte of it inside one
+// allocation (what the copy would have checked), and no part of the lattice's
+// own buffer.  Anything else goes through the staging area.
+bool nat_in_place(const sl_lattice* h, const void* p, size_t bytes)
+{
+    using RangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const RangeFn range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 3020, cudaEnableDefault,
+                                             &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return (RangeFn)f;
+    }();
+    cudaPointerAttributes at;
+    if ((uintptr_t)p % 16 || !range) return false;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const uintptr_t lo = (uintptr_t)p, hi = lo + bytes;
+    return at.type == cudaMemoryTypeDevice && at.device == h->device &&
+           range(&base, &size, (CUdeviceptr)lo) == CUDA_SUCCESS && hi <= base + size &&
+           (hi <= (uintptr_t)h->buf || lo >= (uintptr_t)h->buf + h->buf_bytes);
+}
+
 }  // namespace
 }  // namespace spinmc
 
@@ -366,6 +399,8 @@ int create_lattice(int d, int L, int n, int j_layout, int storage, double J, con
             h->bonds[c][mu] =
                 (j_layout == SL_J_BONDS && mu < d) ? (void*)(base + y.off_bonds[c][mu]) : nullptr;
     }
+    h->buf = dev_buf;
+    h->buf_bytes = y.total;
     h->staging = base + y.off_staging;
     h->staging_bytes = y.staging;
     h->ctrl = (Ctrl*)(base + y.off_ctrl);
@@ -545,12 +580,14 @@ int sl_measure(sl_lattice* h, double* energy, double* magnetisation)
 int sl_get_spins(sl_lattice* h, void* dst)
 {
     if (!h || !dst) return fail(SL_EINVAL, "NULL argument");
+    const bool direct = nat_in_place(h, dst, nat_bytes(h));
+    void* nat = direct ? dst : h->staging;
     cudaError_t e = cudaErrorInvalidValue;
-    if (h->storage == SL_STORE_I8) e = ising_i8_gather(h, (int8_t*)h->staging, h->stream);
-    else if (h->storage == SL_STORE_BITS) e = ising_bits_gather(h, (int8_t*)h->staging, h->stream);
-    else if (h->n > 1) e = on_layout(h, (float*)h->staging, 1, h->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(dst, h->staging, nat_bytes(h), cudaMemcpyDefault, h->stream);
+    if (h->storage == SL_STORE_I8) e = ising_i8_gather(h, (int8_t*)nat, h->stream);
+    else if (h->storage == SL_STORE_BITS) e = ising_bits_gather(h, (int8_t*)nat, h->stream);
+    else if (h->n > 1) e = on_layout(h, (float*)nat, 1, h->stream);
+    if (e == cudaSuccess && !direct)
+        e = cudaMemcpyAsync(dst, nat, nat_bytes(h), cudaMemcpyDefault, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "sl_get_spins");
     return sync_and_check(h);
 }
@@ -558,12 +595,15 @@ int sl_get_spins(sl_lattice* h, void* dst)
 int sl_set_spins(sl_lattice* h, const void* src)
 {
     if (!h || !src) return fail(SL_EINVAL, "NULL argument");
-    cudaError_t e = cudaMemcpyAsync(h->staging, src, nat_bytes(h), cudaMemcpyDefault, h->stream);
+    const bool direct = nat_in_place(h, src, nat_bytes(h));
+    void* nat = direct ? const_cast<void*>(src) : h->staging;
+    cudaError_t e = cudaSuccess;
+    if (!direct) e = cudaMemcpyAsync(nat, src, nat_bytes(h), cudaMemcpyDefault, h->stream);
     if (e == cudaSuccess) {
-        if (h->storage == SL_STORE_I8) e = ising_i8_scatter(h, (const int8_t*)h->staging, h->stream);
+        if (h->storage == SL_STORE_I8) e = ising_i8_scatter(h, (const int8_t*)nat, h->stream);
         else if (h->storage == SL_STORE_BITS)
-            e = ising_bits_scatter(h, (const int8_t*)h->staging, h->stream);
-        else if (h->n > 1) e = on_layout(h, (float*)h->staging, 0, h->stream);
+            e = ising_bits_scatter(h, (const int8_t*)nat, h->stream);
+        else if (h->n > 1) e = on_layout(h, (float*)nat, 0, h->stream);
         else e = cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return cuda_fail(e, "sl_set_spins");
