@@ -148,6 +148,7 @@ extern "C" int sl_autotune(sl_lattice* h, double beta, int trial_sweeps, const c
         (kc == 0 || kc == 2 || (kc == 3 && h->n == 3) || (kc == 4 && h->n == 3 && h->d == 3))) {
         h->rows = r;
         h->blocks_per_sm = c;
+        h->shape_tuned = 1;
         if (kc) h->kernel = kc;
         forget_graphs(h);
         return report();
@@ -211,6 +212,7 @@ extern "C" int sl_autotune(sl_lattice* h, double beta, int trial_sweeps, const c
     // put the state back whatever happened
     h->rows = best_r;
     h->blocks_per_sm = best_c;
+    h->shape_tuned = 1;
     h->kernel = best_k;
     cudaError_t e2 = cudaMemcpyAsync(h->spins[0], keep, colour_bytes, cudaMemcpyDeviceToDevice, s);
     if (e2 == cudaSuccess)

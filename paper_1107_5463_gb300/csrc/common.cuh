@@ -42,6 +42,43 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const RoundKeys& rk)
     return c;
 }
 
+// Philox4x32-10 of counters (g, t, replica, w) that differ only in g: what the
+// first two rounds make of the other three words is worked out once (2 of the
+// 20 wide multiplies, and the XORs around them).
+struct PhiloxGroups {
+    uint32_t z1, x2, z2, w2;
+};
+
+__device__ __forceinline__ PhiloxGroups philox_groups(uint32_t t, uint32_t replica, uint32_t w,
+                                                      const RoundKeys& rk)
+{
+    const uint64_t p = (uint64_t)replica * 0xCD9E8D57u;
+    const uint32_t x1 = (uint32_t)(p >> 32) ^ t ^ rk.k0[0];
+    const uint64_t q = (uint64_t)x1 * 0xD2511F53u;
+    PhiloxGroups c;
+    c.z1 = w ^ rk.k1[0];
+    c.x2 = (uint32_t)p ^ rk.k0[1];
+    c.z2 = (uint32_t)(q >> 32) ^ rk.k1[1];
+    c.w2 = (uint32_t)q;
+    return c;
+}
+
+__device__ __forceinline__ uint4 philox_at(const PhiloxGroups& pg, uint32_t g, const RoundKeys& rk)
+{
+    const uint64_t p0 = (uint64_t)g * 0xD2511F53u;
+    const uint32_t z1 = (uint32_t)(p0 >> 32) ^ pg.z1;
+    const uint64_t p1 = (uint64_t)z1 * 0xCD9E8D57u;
+    uint4 c = make_uint4((uint32_t)(p1 >> 32) ^ pg.x2, (uint32_t)p1, (uint32_t)p0 ^ pg.z2, pg.w2);
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+        const uint64_t a = (uint64_t)c.x * 0xD2511F53u;
+        const uint64_t b = (uint64_t)c.z * 0xCD9E8D57u;
+        c = make_uint4((uint32_t)(b >> 32) ^ c.y ^ rk.k0[r], (uint32_t)b,
+                       (uint32_t)(a >> 32) ^ c.w ^ rk.k1[r], (uint32_t)a);
+    }
+    return c;
+}
+
 enum Purpose : uint32_t { kSweep = 0, kInit = 1, kCoupling = 2, kExchange = 3 };
 
 // Device control block: one per lattice, inside the caller's buffer.
@@ -65,22 +102,24 @@ struct Partial {
 // Division of n < 2^31 by a divisor fixed for a launch: a multiply-high and a
 // shift in place of the some 20 instructions of a 32-bit division (and 70 of a
 // 64-bit one).  With 2^(s-1) < d <= 2^s and m = ceil(2^(31+s) / d) < 2^32 the
-// error m d - 2^(31+s) is below 2^s, so n m >> (31 + s) is exact for n < 2^31.
+// error m d - 2^(31+s) is below 2^s, so n m >> (31 + s) is exact for n < 2^31;
+// the shift beyond the high word is kept (d = 1, whose s = 0, is let through).
 struct FastDiv {
     uint32_t d, m, s;
-    __host__ __device__ uint32_t div(uint32_t n) const
+    __device__ __forceinline__ uint32_t div(uint32_t n) const
     {
-        return (uint32_t)(((uint64_t)n * m) >> (31 + s));
+        return d == 1u ? n : __umulhi(n, m) >> s;
     }
 };
 
 __host__ inline FastDiv make_fast_div(uint32_t d)
 {
     FastDiv f;
+    int s = 0;
+    while (((uint64_t)1 << s) < d) ++s;
     f.d = d;
-    f.s = 0;
-    while (((uint64_t)1 << f.s) < d) ++f.s;
-    f.m = (uint32_t)((((uint64_t)1 << (31 + f.s)) + d - 1) / d);
+    f.m = (uint32_t)((((uint64_t)1 << (31 + s)) + d - 1) / d);
+    f.s = (uint32_t)(s > 0 ? s - 1 : 0);
     return f;
 }
 

@@ -13,6 +13,9 @@
 namespace spinmc {
 
 constexpr int kMaxBlocks = 4096;     // upper bound on any measuring grid
+// Byte-Ising kernels leave at most this many block partials; the space of the
+// others holds the resident sweeps' control area (ising_res.cu)
+constexpr int kI8Blocks = kMaxBlocks / 2;
 constexpr size_t kAlign = 256;
 
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -74,6 +77,7 @@ struct sl_lattice {
     // options
     int renorm_every, fast_math, kernel, rows, use_graph;
     int blocks_per_sm;       // cap of the streaming kernels' grids per SM (0 = none)
+    int shape_tuned;         // rows and blocks_per_sm come from sl_autotune, not from the user
     int update;              // SL_UPDATE_METROPOLIS, _HEATBATH or _SW
     int multihit, tile;      // k-fold multi-hit sweeps in tiles of side `tile` (0 = off)
     // cached graphs of kGraphSweeps sweeps and of one sweep
@@ -123,6 +127,12 @@ cudaError_t ising_i8_pass(const sl_lattice* h, const SweepParams& p, int c, cuda
 cudaError_t ising_i8_measure(const sl_lattice* h, cudaStream_t s);
 // measurement that also closes a sweep (series entry, sweep counter + 1)
 cudaError_t ising_i8_measure_advance(const sl_lattice* h, cudaStream_t s);
+
+// ---- Ising int8, lattices resident in shared memory (ising_res.cu) ----
+bool i8_resident_ok(const sl_lattice* h);
+cudaError_t i8_resident_sweeps(const sl_lattice* h, const SweepParams& p, int64_t count,
+                               cudaStream_t s);
+cudaError_t i8_resident_clear(const sl_lattice* h, cudaStream_t s);  // once, at creation
 
 // ---- Ising multi-hit sweeps in big tiles (ising_tile.cu) ----
 bool tile_size_ok(int d, int L, int T);

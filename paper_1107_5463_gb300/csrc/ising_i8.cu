@@ -16,9 +16,13 @@
 // the move is accepted iff g >= q(u), which equals u <= T[g] for g < ncmp and
 // "always" for the classes with dE <= 0 (thresholds are non-decreasing in g).
 //
-// Two kernels compute the same decisions bit for bit:
+// Three kernels here compute the same decisions bit for bit (a fourth,
+// ising_res.cu, keeps lattices that fit in shared memory):
 //   i8_generic  one thread per Philox group of 4 sites, scalar, any even L and
-//               any couplings; also the standalone measurement;
+//               any couplings, slabs of short rows;
+//   i8_flat     one thread per Philox group, a word of four bytes at a time
+//               where W % 4 == 0, any even L, uniform coupling, whole lattices;
+//               also the standalone measurement;
 //   i8_stream   one thread per 16-byte column chunk marching through R rows
 //               with a rolling window of the other colour's rows in registers,
 //               128-bit loads and stores, SIMD-within-a-word neighbour
@@ -30,7 +34,7 @@
 // global plane offset to every Philox group (gofs colour entries) and its
 // parity to every colour, so each site makes the decisions it makes in the
 // whole lattice.
-#include "internal.h"
+#include "ising_group.cuh"
 
 namespace spinmc {
 namespace {
@@ -165,6 +169,73 @@ __global__ void __launch_bounds__(256) i8_generic(const I8Args a)
     finish_pass(a.ctrl, a.partials, mine, [&](const Partial& tot) { i8_finish(a, tot); });
 }
 
+// --------------------------------------------------------------- flat ----
+//
+// Row lengths the streaming kernel cannot take (W no multiple of 16) and the
+// standalone measurement.  A thread takes one Philox group at a time:
+// neighbour words from L1 / L2, the counts and decisions of four sites in one
+// word (ising_group.cuh), two multiply-highs for the position.  Bound by
+// issue.  UPD = false measures without moves.
+
+template <int D, bool ALIGNED, bool HB, bool UPD, bool MEAS>
+__global__ void __launch_bounds__(256) i8_flat(const I8Args a, const FastDiv Wd, const FastDiv Ld)
+{
+    __shared__ long long red[32];
+    __shared__ uint32_t s_hb[16];
+    if (HB && UPD) {
+        if (threadIdx.x < 13) s_hb[threadIdx.x] = a.tab.hb[threadIdx.x];
+        __syncthreads();
+    }
+    GroupGeo e;
+    e.W = a.W;
+    e.L = a.L;
+    e.P = D == 3 ? a.L * a.W : a.W;
+    e.H = (int)a.H;
+    const PhiloxGroups pg =
+        philox_groups((uint32_t)a.ctrl->t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
+    const GroupSign sg = group_sign<D>(a.tab);
+    const uint8_t* o = reinterpret_cast<const uint8_t*>(a.oth);
+    const int ngroups = (int)((a.H + 3) >> 2);
+    GroupCounts m = {0u, 0u, 0u, 0u};
+    uint32_t nsite = 0;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < ngroups; q += gridDim.x * blockDim.x) {
+        const GroupPos g = group_at<D, ALIGNED>(4 * q, e, Wd, Ld, a.c);
+        uint32_t nw[2 * D];
+        group_neighbours<D, ALIGNED>(o, g, e, 0, nw, [&](int l, bool up) {
+            int z = up ? l + e.P : l - e.P;
+            if (z < 0) z += e.H;
+            if (z >= e.H) z -= e.H;
+            // (entries past the lattice's last, whose results are masked, stay inside)
+            if (!ALIGNED && z >= e.H) z -= e.H;
+            return ALIGNED ? *reinterpret_cast<const uint32_t*>(o + z) : (uint32_t)o[z];
+        });
+        const uint32_t cur = nw[0];
+        const uint32_t av = *reinterpret_cast<const uint32_t*>(a.own + g.l);
+        const uint32_t valid = ALIGNED || g.l + 4 <= e.H
+                                   ? 0x01010101u
+                                   : 0x01010101u & ((1u << (8 * (e.H - g.l))) - 1u);
+        if (UPD) {
+            const uint4 rnd = philox_at(pg, (uint32_t)q, a.rk);
+            *reinterpret_cast<uint32_t*>(a.own + g.l) =
+                group_update<D, HB, MEAS>(av, nw, cur, rnd, a.tab, sg, s_hb, valid, m);
+        } else {
+            m.na += group_unsatisfied<D>(av, nw, valid);
+            m.down = __dp4a(av, valid, __dp4a(cur, valid, m.down));
+        }
+        if (MEAS) nsite += __popc(valid);
+    }
+    if (!MEAS) return;
+    long long bond = 2LL * D * nsite - 2LL * unsatisfied_after<D>(m);
+    if (UPD && a.tab.sigma_neg && !HB) bond = -bond;
+    const long long b = block_sum(bond, red);
+    const long long dn = block_sum((long long)m.down, red);
+    if (threadIdx.x == 0) {
+        Partial* acc = a.partials + kMaxBlocks;
+        atomicAdd(reinterpret_cast<unsigned long long*>(&acc->i0), (unsigned long long)b);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&acc->i1), (unsigned long long)dn);
+    }
+}
+
 // ---------------------------------------------------------- streaming ----
 
 __device__ __forceinline__ uint4 ld_rows(const int8_t* p)
@@ -195,20 +266,6 @@ __device__ __forceinline__ uint4 shift_row(uint4 v, uint32_t edge, int p)
 __device__ __forceinline__ uint32_t w_of(const uint4& v, int k)
 {
     return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w;
-}
-
-// Per byte: 0x80 minus the number of thresholds below u, i.e. 0x80 - q(u)
-// for the four sites of one Philox block (byte b <- output b).
-template <int NCMP>
-__device__ __forceinline__ uint32_t q_bias(const uint4& r, const IsingTable& tab)
-{
-    uint32_t acc = 0x80808080u;
-    const uint32_t u[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-        for (int k = 0; k < NCMP; ++k) acc -= (u[b] > tab.thr[k]) ? (1u << (8 * b)) : 0u;
-    return acc;
 }
 
 // MEAS: the measuring (colour-1) pass; the other pass is compiled without the
@@ -677,8 +734,38 @@ int pick_rows(const sl_lattice* h)
     return R;
 }
 
+__global__ void i8_finish_kernel(const I8Args a);
+
+// whole lattices with a uniform coupling (SL_OPT_KERNEL 1 asks for i8_generic)
+bool flat_ok(const sl_lattice* h)
+{
+    return !h->slab && h->j_layout == SL_J_UNIFORM && h->kernel != 1;
+}
+
+template <int D, bool ALIGNED>
+cudaError_t launch_flat(const sl_lattice* h, const I8Args& a, cudaStream_t s)
+{
+    const FastDiv Wd = make_fast_div((uint32_t)h->W), Ld = make_fast_div((uint32_t)h->L);
+    const int grid = grid_for((h->H + 3) >> 2, 256);
+    if (!a.update) i8_flat<D, ALIGNED, false, false, true><<<grid, 256, 0, s>>>(a, Wd, Ld);
+    else if (a.tab.heatbath && a.measure)
+        i8_flat<D, ALIGNED, true, true, true><<<grid, 256, 0, s>>>(a, Wd, Ld);
+    else if (a.tab.heatbath) i8_flat<D, ALIGNED, true, true, false><<<grid, 256, 0, s>>>(a, Wd, Ld);
+    else if (a.measure) i8_flat<D, ALIGNED, false, true, true><<<grid, 256, 0, s>>>(a, Wd, Ld);
+    else i8_flat<D, ALIGNED, false, true, false><<<grid, 256, 0, s>>>(a, Wd, Ld);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || !a.measure) return e;
+    i8_finish_kernel<<<1, 1, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_pass(const sl_lattice* h, I8Args a, cudaStream_t s, bool stream)
 {
+    if (!stream && flat_ok(h)) {
+        if (h->d == 2)
+            return h->W % 4 == 0 ? launch_flat<2, true>(h, a, s) : launch_flat<2, false>(h, a, s);
+        return h->W % 4 == 0 ? launch_flat<3, true>(h, a, s) : launch_flat<3, false>(h, a, s);
+    }
     if (stream) {
         a.R = pick_rows(h);
         const long long items = (long long)(h->W / 16) * (h->d == 3 ? h->L : 1) * (h->Lz / a.R);
@@ -719,7 +806,8 @@ cudaError_t launch_pass(const sl_lattice* h, I8Args a, cudaStream_t s, bool stre
             i8_finish_kernel<<<1, 1, 0, s>>>(a);
         }
     } else {
-        const int grid = grid_for((h->H + 3) >> 2, 256);
+        int grid = grid_for((h->H + 3) >> 2, 256);
+        if (a.measure && grid > kI8Blocks) grid = kI8Blocks;
         if (h->d == 2) i8_generic<2><<<grid, 256, 0, s>>>(a);
         else i8_generic<3><<<grid, 256, 0, s>>>(a);
     }

@@ -890,8 +890,10 @@ cudaError_t ising_sw_sweeps(const sl_lattice* h, const SweepParams& p, int64_t c
         if (e == cudaSuccess) {
             if (h->L % 8 == 0) {
                 const long long items = (long long)h->L * (h->d == 3 ? h->L : 1) * (h->L / 8);
-                if (h->d == 2) sw_measure<2><<<grid_for(items, 256), 256, 0, s>>>(a, h->partials, h->J);
-                else sw_measure<3><<<grid_for(items, 256), 256, 0, s>>>(a, h->partials, h->J);
+                int grid = grid_for(items, 256);
+                if (grid > kI8Blocks) grid = kI8Blocks;
+                if (h->d == 2) sw_measure<2><<<grid, 256, 0, s>>>(a, h->partials, h->J);
+                else sw_measure<3><<<grid, 256, 0, s>>>(a, h->partials, h->J);
                 e = cudaGetLastError();
             } else {
                 e = ising_i8_measure_advance(h, s);

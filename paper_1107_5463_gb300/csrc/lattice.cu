@@ -411,6 +411,7 @@ int create_lattice(int d, int L, int n, int j_layout, int storage, double J, con
     h->kernel = 0;
     h->rows = 0;
     h->blocks_per_sm = 0;
+    h->shape_tuned = 0;
     h->use_graph = 1;
     h->update = 0;
     h->multihit = 0;
@@ -434,6 +435,7 @@ int create_lattice(int d, int L, int n, int j_layout, int storage, double J, con
     e = cudaMemsetAsync(h->ctrl, 0, sizeof(Ctrl), h->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(h->partials + kMaxBlocks, 0, sizeof(Partial), h->stream);
+    if (e == cudaSuccess && storage == SL_STORE_I8) e = i8_resident_clear(h, h->stream);
     if (e == cudaSuccess && storage == SL_STORE_I8) e = ising_i8_init(h, h->stream);
     if (e == cudaSuccess && storage == SL_STORE_BITS) e = ising_bits_init(h, h->stream);
     if (e == cudaSuccess && n > 1) e = on_init(h, h->stream);
@@ -528,7 +530,12 @@ int sl_sweep_series(sl_lattice* h, double beta, int64_t nsweeps, uint64_t seed, 
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "series setup");
     int64_t left = nsweeps;
-    if (h->use_graph && nsweeps >= 2) {
+    if (i8_resident_ok(h)) {
+        e = i8_resident_sweeps(h, p, nsweeps, h->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
+        left = 0;
+    }
+    if (h->use_graph && left >= 2) {
         // whole runs of kGraphSweeps sweeps, then single-sweep replays
         const int st = ensure_graph(h, p);
         if (st != SL_OK) return st;
@@ -673,10 +680,12 @@ int sl_set_option(sl_lattice* h, int option, int64_t value)
         if (value < 0 || (value > 0 && (h->Lz % value != 0)))
             return fail(SL_EINVAL, "rows must be 0 (automatic) or divide the planes held");
         h->rows = (int)value;
+        h->shape_tuned = 0;
         return SL_OK;
     case SL_OPT_BLOCKS_PER_SM:
         if (value < 0 || value > 64) return fail(SL_EINVAL, "blocks_per_sm must be in [0, 64]");
         h->blocks_per_sm = (int)value;
+        h->shape_tuned = 0;
         return SL_OK;
     case SL_OPT_GRAPH:
         if (value != 0 && value != 1) return fail(SL_EINVAL, "graph must be 0 or 1");
