@@ -150,19 +150,54 @@ __device__ __forceinline__ T block_sum(T v, T* scratch)
     return r;
 }
 
+// Block-wide sums of four doubles, valid in thread 0.  FP64 adds run at two
+// lanes per clock and multiprocessor, so a warp's butterfly over each value (20
+// warp adds, 180 for a block of 256 threads with the second stage) took 7 to
+// 12 us of a measuring pass of 1024 blocks.  Here the lanes split the values
+// between them as they fold: after two exchanges each quarter of the warp
+// holds one value, 6 warp adds in all, and one warp folds the warps' sums of
+// all four values together (51 adds for the block).  `scratch` holds 4 doubles
+// per warp; the order of the additions is fixed.
+__device__ __forceinline__ void block_sum4(double (&v)[4], double* scratch)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool up = (lane & 16) != 0, odd = (lane & 8) != 0;
+    // lanes 0-15 keep values 0 and 1, lanes 16-31 values 2 and 3
+    double a = up ? v[2] : v[0], b = up ? v[3] : v[1];
+    a += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], 16);
+    b += __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], 16);
+    double x = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    __syncthreads();
+    if ((lane & 7) == 0) scratch[4 * warp + (lane >> 3)] = x;
+    __syncthreads();
+    if (warp == 0) {
+        // lane (value, slot): the sums of warps slot, slot + 8, ...
+        const int nw = (blockDim.x + 31) >> 5;
+        x = 0.0;
+        for (int w = lane & 7; w < nw; w += 8) x += scratch[4 * w + (lane >> 3)];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = __shfl_sync(0xffffffffu, x, 8 * k);
+    }
+}
+
 // Called by every thread of every block at the end of a measured pass with
 // the block's partial (valid in thread 0).  The last block to arrive adds all
 // partials: thread k takes blocks k, k + blockDim, ... in order and the block
 // tree-sums the threads, a fixed order for a given grid, so FP64 totals are
 // reproducible.  Thread 0 of that block passes the totals to `finish` and
-// resets the arrival count.
-template <typename Finish>
+// resets the arrival count.  FP: the totals are the double members, else the
+// integer ones.
+template <bool FP, typename Finish>
 __device__ __forceinline__ void finish_pass(Ctrl* ctrl, Partial* partials, const Partial& mine,
                                             Finish finish)
 {
     __shared__ bool last;
-    __shared__ long long red_i[32];
-    __shared__ double red_f[32];
+    __shared__ long long red_i[FP ? 1 : 32];
+    __shared__ double red_f[FP ? 128 : 1];
     if (threadIdx.x == 0) {
         partials[blockIdx.x] = mine;
         __threadfence();
@@ -176,16 +211,25 @@ __device__ __forceinline__ void finish_pass(Ctrl* ctrl, Partial* partials, const
     double f[4] = {0.0, 0.0, 0.0, 0.0};
     for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
         const Partial* p = partials + b;
-        i0 += __ldcg(&p->i0);
-        i1 += __ldcg(&p->i1);
+        if (FP) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) f[k] += __ldcg(&p->f[k]);
+            for (int k = 0; k < 4; ++k) f[k] += __ldcg(&p->f[k]);
+        } else {
+            i0 += __ldcg(&p->i0);
+            i1 += __ldcg(&p->i1);
+        }
     }
     Partial tot;
-    tot.i0 = block_sum(i0, red_i);
-    tot.i1 = block_sum(i1, red_i);
+    if (FP) {
+        block_sum4(f, red_f);
+    } else {
+        i0 = block_sum(i0, red_i);
+        i1 = block_sum(i1, red_i);
+    }
+    tot.i0 = i0;
+    tot.i1 = i1;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) tot.f[k] = block_sum(f[k], red_f);
+    for (int k = 0; k < 4; ++k) tot.f[k] = f[k];
     if (threadIdx.x == 0) {
         finish(tot);
         ctrl->done = 0;
@@ -201,36 +245,43 @@ __device__ __forceinline__ void finish_pass(Ctrl* ctrl, Partial* partials, const
 // stores before the loads.  Thread k adds blocks k, k + kFinishThreads, ...
 // in order and the block tree-sums the threads: a fixed order for a given
 // grid, so FP64 totals stay reproducible.
-constexpr int kFinishThreads = 512;
+constexpr int kFinishThreads = 256;
+
+// A continuous-spin block's FP32 sums of a measuring pass, added in FP64;
+// scratch holds 4 doubles per warp.
+__device__ __forceinline__ Partial fp_partial(float e, float mx, float my, float mz,
+                                              double* scratch)
+{
+    double v[4] = {(double)e, (double)mx, (double)my, (double)mz};
+    block_sum4(v, scratch);
+    Partial p;
+    p.i0 = p.i1 = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) p.f[k] = v[k];
+    return p;
+}
 
 __device__ __forceinline__ void store_partial(Partial* partials, const Partial& mine)
 {
     if (threadIdx.x == 0) partials[blockIdx.x] = mine;
 }
 
-// Total of the first nblocks partials (FP: also the four double members),
-// valid in thread 0.
-template <bool FP>
+// FP64 totals of the first nblocks partials, valid in thread 0 of a block of
+// kFinishThreads.
 __device__ __forceinline__ Partial sum_partials(const Partial* partials, unsigned nblocks)
 {
-    __shared__ long long red_i[32];
-    __shared__ double red_f[32];
-    long long i0 = 0, i1 = 0;
+    __shared__ double red[4 * (kFinishThreads / 32)];
     double f[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 4
     for (unsigned b = threadIdx.x; b < nblocks; b += blockDim.x) {
-        i0 += partials[b].i0;
-        i1 += partials[b].i1;
-        if (FP) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) f[k] += partials[b].f[k];
-        }
+        for (int k = 0; k < 4; ++k) f[k] += partials[b].f[k];
     }
+    block_sum4(f, red);
     Partial tot;
-    tot.i0 = block_sum(i0, red_i);
-    tot.i1 = block_sum(i1, red_i);
+    tot.i0 = tot.i1 = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) tot.f[k] = FP ? block_sum(f[k], red_f) : 0.0;
+    for (int k = 0; k < 4; ++k) tot.f[k] = f[k];
     return tot;
 }
 

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256) i8_generic(const I8Args a)
     mine.i0 = block_sum(bond, red);
     mine.i1 = block_sum(down, red);
     mine.f[0] = mine.f[1] = mine.f[2] = mine.f[3] = 0.0;
-    finish_pass(a.ctrl, a.partials, mine, [&](const Partial& tot) { i8_finish(a, tot); });
+    finish_pass<false>(a.ctrl, a.partials, mine, [&](const Partial& tot) { i8_finish(a, tot); });
 }
 
 // --------------------------------------------------------------- flat ----
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
         }
         return;
     }
-    finish_pass(a.ctrl, a.partials, mine, [&](const Partial& tot) { i8_finish(a, tot); });
+    finish_pass<false>(a.ctrl, a.partials, mine, [&](const Partial& tot) { i8_finish(a, tot); });
 }
 
 // Closes an i8_stream measuring pass from the totals its blocks added into

@@ -808,7 +808,7 @@ __global__ void __launch_bounds__(256) sw_measure(const SwArgs a, Partial* parti
     mine.i0 = block_sum(bond, red);
     mine.i1 = block_sum(down, red);
     mine.f[0] = mine.f[1] = mine.f[2] = mine.f[3] = 0.0;
-    finish_pass(a.ctrl, partials, mine, [&](const Partial& tot) {
+    finish_pass<false>(a.ctrl, partials, mine, [&](const Partial& tot) {
         Ctrl* C = a.ctrl;
         const double E = -J * (double)tot.i0;
         const double M = (double)(a.N - 2 * tot.i1);

@@ -342,7 +342,7 @@ __device__ __forceinline__ void on_finish(const OnArgs& a, const Partial& tot)
 template <int NC, int D, bool FAST, bool HB>
 __global__ void __launch_bounds__(128) on_generic(const OnArgs a)
 {
-    __shared__ double red[32];
+    __shared__ double red[32];  // 4 per warp
     const unsigned long long t64 = a.ctrl->t;
     const uint32_t t = (uint32_t)t64;
     const bool renorm = NC == 3 && a.update && a.renorm_every > 0 &&
@@ -491,13 +491,8 @@ __global__ void __launch_bounds__(128) on_generic(const OnArgs a)
         }
     }
     if (!a.measure) return;
-    Partial mine;
-    mine.i0 = mine.i1 = 0;
-    mine.f[0] = block_sum((double)pe, red);
-    mine.f[1] = block_sum((double)pmx, red);
-    mine.f[2] = block_sum((double)pmy, red);
-    mine.f[3] = block_sum((double)pmz, red);
-    finish_pass(a.ctrl, a.partials, mine, [&](const Partial& tot) { on_finish(a, tot); });
+    const Partial mine = fp_partial(pe, pmx, pmy, pmz, red);
+    finish_pass<true>(a.ctrl, a.partials, mine, [&](const Partial& tot) { on_finish(a, tot); });
 }
 
 // ------------------------------------------------------------ streaming ----
@@ -534,7 +529,7 @@ __device__ __forceinline__ V3 shfl3_down(V3 v)
 template <int D, bool FAST, bool HB, bool MEAS>
 __global__ void __launch_bounds__(256, D == 2 && !HB ? 4 : 3) heis_stream(const OnArgs a)
 {
-    __shared__ double red[32];
+    __shared__ double red[32];  // 4 per warp
     // Metropolis with accurate functions: the proposal's azimuth from the shared table
     constexpr bool TAB = !FAST && !HB;
     __shared__ float2 tab[TAB ? kTurnTab : 1];
@@ -668,12 +663,7 @@ __global__ void __launch_bounds__(256, D == 2 && !HB ? 4 : 3) heis_stream(const 
         }
     }
     if (!MEAS) return;
-    Partial mine;
-    mine.i0 = mine.i1 = 0;
-    mine.f[0] = block_sum((double)pe, red);
-    mine.f[1] = block_sum((double)pmx, red);
-    mine.f[2] = block_sum((double)pmy, red);
-    mine.f[3] = block_sum((double)pmz, red);
+    const Partial mine = fp_partial(pe, pmx, pmy, pmz, red);
     store_partial(a.partials, mine);
 }
 
@@ -690,7 +680,7 @@ struct P3 {
 template <int D, bool FAST, bool HB, bool MEAS>
 __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
 {
-    __shared__ double red[32];
+    __shared__ double red[32];  // 4 per warp
     // Metropolis with accurate functions: the proposal's azimuth from the shared table
     constexpr bool TAB = !FAST && !HB;
     __shared__ float2 tab[TAB ? kTurnTab : 1];
@@ -862,12 +852,7 @@ __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
         }
     }
     if (!MEAS) return;
-    Partial mine;
-    mine.i0 = mine.i1 = 0;
-    mine.f[0] = block_sum((double)pe, red);
-    mine.f[1] = block_sum((double)pmx, red);
-    mine.f[2] = block_sum((double)pmy, red);
-    mine.f[3] = block_sum((double)pmz, red);
+    const Partial mine = fp_partial(pe, pmx, pmy, pmz, red);
     store_partial(a.partials, mine);
 }
 
@@ -996,7 +981,7 @@ __global__ void __launch_bounds__(kTileThreads, 3) heis_tile3(const OnArgs a)
     extern __shared__ __align__(128) float tile_smem[];
     __shared__ float2 tab[kTurnTab];
     __shared__ __align__(8) unsigned long long bars[kOthStages + kOwnStages];
-    __shared__ double red[32];
+    __shared__ double red[32];  // 4 per warp
     fill_turn_table(tab);
     const unsigned long long t64 = a.ctrl->t;
     const uint32_t t = (uint32_t)t64;
@@ -1159,12 +1144,7 @@ __global__ void __launch_bounds__(kTileThreads, 3) heis_tile3(const OnArgs a)
         return;
     }
     if (!MEAS) return;
-    Partial mine;
-    mine.i0 = mine.i1 = 0;
-    mine.f[0] = block_sum((double)pe, red);
-    mine.f[1] = block_sum((double)pmx, red);
-    mine.f[2] = block_sum((double)pmy, red);
-    mine.f[3] = block_sum((double)pmz, red);
+    const Partial mine = fp_partial(pe, pmx, pmy, pmz, red);
     store_partial(a.partials, mine);
 }
 
@@ -1173,7 +1153,7 @@ __global__ void __launch_bounds__(kTileThreads, 3) heis_tile3(const OnArgs a)
 template <bool FAST, bool HB, bool MEAS>
 __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
 {
-    __shared__ double red[32];
+    __shared__ double red[32];  // 4 per warp
     // Metropolis with accurate functions: sin and cos from the shared table
     constexpr bool TAB = !FAST && !HB;
     __shared__ float2 tab[TAB ? kTurnTab : 1];
@@ -1329,12 +1309,186 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
         }
     }
     if (!MEAS) return;
-    Partial mine;
-    mine.i0 = mine.i1 = 0;
-    mine.f[0] = block_sum((double)pe, red);
-    mine.f[1] = block_sum((double)pmx, red);
-    mine.f[2] = block_sum((double)pmy, red);
-    mine.f[3] = 0.0;
+    const Partial mine = fp_partial(pe, pmx, pmy, 0.f, red);
+    store_partial(a.partials, mine);
+}
+
+// ------------------------------------------------------------- XY, flat ----
+//
+// XY with a uniform coupling on lattices xy_stream cannot take (3D, and rows of
+// other lengths).  on_generic evaluated sin and cos of every neighbour anew
+// (eight evaluations per site in 3D) and a whole Philox call per site: 366
+// instructions per site, 23 us a pass at 3D L = 100.  Here a first kernel
+// writes (cos, sin) of the other colour's angles once per pass into the
+// staging area (8 H bytes, its whole size; idle between calls), and in the
+// second a thread takes the two sites of one Philox call and reads its
+// neighbours' vectors.  Bound by issue.  The arithmetic of a site is that of
+// on_generic, rounding for rounding.
+
+template <bool FAST>
+__global__ void __launch_bounds__(256) xy_vectors(const float* th, float2* cs, uint32_t H)
+{
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < H; j += gridDim.x * blockDim.x) {
+        float s, c;
+        sincos_angle<FAST>(__ldg(th + j), &s, &c);
+        cs[j] = make_float2(c, s);
+    }
+}
+
+// EVEN: W is even, so the two sites of a Philox call are neighbours in a row
+// and every neighbour row is read in aligned pairs.
+template <int D, bool EVEN, bool FAST, bool HB>
+__global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs, const FastDiv Wd,
+                                               const FastDiv Ld)
+{
+    __shared__ double red[32];  // 4 per warp
+    const int L = a.L, W = a.W, H = (int)a.H, P = D == 3 ? L * W : W;
+    const float J = a.J;
+    const PhiloxGroups pg =
+        philox_groups((uint32_t)a.ctrl->t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
+    const int ncalls = (H + 1) / 2;
+    float pe = 0.f, pmx = 0.f, pmy = 0.f;
+    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < ncalls; q += gridDim.x * blockDim.x) {
+        const int j0 = 2 * q;
+        int row = (int)Wd.div((uint32_t)j0);
+        int k = j0 - row * W;
+        int z = D == 3 ? (int)Ld.div((uint32_t)row) : 0;
+        int y = D == 3 ? row - z * L : row;
+        // neighbour vectors of the two sites: -x, +x, -y, +y (, -z, +z)
+        float2 v[2][2 * D], own_col[2];
+        const bool second = EVEN || j0 + 1 < H;
+        if (EVEN) {
+            const int p = (y + z + a.c) & 1;
+            const float4* c4 = reinterpret_cast<const float4*>(cs);
+            auto pair = [&](int j, int dir) {
+                const float4 w = __ldg(c4 + (j >> 1));
+                v[0][dir] = make_float2(w.x, w.y);
+                v[1][dir] = make_float2(w.z, w.w);
+            };
+            const float4 cur = __ldg(c4 + q);
+            own_col[0] = make_float2(cur.x, cur.y);
+            own_col[1] = make_float2(cur.z, cur.w);
+            const float2 edge = __ldg(cs + (p ? (k + 2 == W ? j0 + 2 - W : j0 + 2)
+                                              : (k == 0 ? j0 + W - 1 : j0 - 1)));
+            v[0][0] = p ? own_col[0] : edge;
+            v[0][1] = p ? own_col[1] : own_col[0];
+            v[1][0] = p ? own_col[1] : own_col[0];
+            v[1][1] = p ? edge : own_col[1];
+            if (D == 3) {
+                pair(y == 0 ? j0 + (L - 1) * W : j0 - W, 2);
+                pair(y == L - 1 ? j0 - (L - 1) * W : j0 + W, 3);
+            }
+            pair(j0 < P ? j0 + H - P : j0 - P, 2 * D - 2);
+            pair(j0 + P < H ? j0 + P : j0 + P - H, 2 * D - 1);
+        } else {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int j = b && second ? j0 + 1 : j0;
+                const int p = (y + z + a.c) & 1;
+                own_col[b] = __ldg(cs + j);
+                const float2 e = __ldg(cs + (p ? (k + 1 == W ? j + 1 - W : j + 1)
+                                               : (k == 0 ? j + W - 1 : j - 1)));
+                v[b][0] = p ? own_col[b] : e;
+                v[b][1] = p ? e : own_col[b];
+                if (D == 3) {
+                    v[b][2] = __ldg(cs + (y == 0 ? j + (L - 1) * W : j - W));
+                    v[b][3] = __ldg(cs + (y == L - 1 ? j - (L - 1) * W : j + W));
+                }
+                v[b][2 * D - 2] = __ldg(cs + (j < P ? j + H - P : j - P));
+                v[b][2 * D - 1] = __ldg(cs + (j + P < H ? j + P : j + P - H));
+                if (second && ++k == W) {  // the second site opens the next row
+                    k = 0;
+                    if (++y == L && D == 3) {
+                        y = 0;
+                        ++z;
+                    }
+                }
+            }
+        }
+        float hx[2], hy[2], sx[2], sy[2], th[2];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            hx[b] = __fmul_rn(J, v[b][0].x);
+            hy[b] = __fmul_rn(J, v[b][0].y);
+#pragma unroll
+            for (int d = 1; d < 2 * D; ++d) {
+                hx[b] = __fmaf_rn(J, v[b][d].x, hx[b]);
+                hy[b] = __fmaf_rn(J, v[b][d].y, hy[b]);
+            }
+        }
+        if (EVEN) {
+            const float2 o = *reinterpret_cast<const float2*>(a.own + j0);
+            th[0] = o.x;
+            th[1] = o.y;
+        } else {
+            th[0] = a.own[j0];
+            th[1] = second ? a.own[j0 + 1] : th[0];
+        }
+        bool changed[2] = {false, false};
+        if (HB) {
+            const VonMises m0 = von_mises_setup(hx[0], hy[0], a.beta);
+            const VonMises m1 = von_mises_setup(hx[1], hy[1], a.beta);
+            bool p0 = true, p1 = second;
+            uint32_t acc0 = 0u, acc1 = 0u;
+            for (int at = 0; at < kVonMisesAttempts && (p0 || p1); ++at) {
+                const uint4 rnd = philox4x32_10(
+                    make_uint4((uint32_t)q, (uint32_t)a.ctrl->t, a.replica,
+                               ((uint32_t)at << 16) | (kSweep << 1) | (uint32_t)a.c),
+                    a.rk);
+                if (p0 && von_mises_accept(m0, rnd.x, rnd.y)) {
+                    acc0 = rnd.x;
+                    p0 = false;
+                }
+                if (p1 && von_mises_accept(m1, rnd.z, rnd.w)) {
+                    acc1 = rnd.z;
+                    p1 = false;
+                }
+            }
+            if (!p0) th[0] = von_mises_angle(m0, acc0);
+            if (second && !p1) th[1] = von_mises_angle(m1, acc1);
+            changed[0] = !p0;
+            changed[1] = second && !p1;
+#pragma unroll
+            for (int b = 0; b < 2; ++b) sincos_angle<FAST>(th[b], &sy[b], &sx[b]);
+        } else {
+            const uint4 rnd = philox_at(pg, (uint32_t)q, a.rk);
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const float u = u24(b ? rnd.z : rnd.x), nt = u24(b ? rnd.w : rnd.y);
+                float nx, ny;
+                sincos_angle<FAST>(th[b], &sy[b], &sx[b]);
+                sincos_angle<FAST>(nt, &ny, &nx);
+                const float dE = -__fmaf_rn(__fsub_rn(nx, sx[b]), hx[b],
+                                            __fmul_rn(__fsub_rn(ny, sy[b]), hy[b]));
+                const float w = boltzmann<FAST>(__fmul_rn(-a.beta, dE));
+                if ((dE <= 0.f) | (u < w)) {
+                    th[b] = nt;
+                    sx[b] = nx;
+                    sy[b] = ny;
+                    changed[b] = true;
+                }
+            }
+        }
+        if (EVEN) {
+            if (changed[0] | changed[1])
+                *reinterpret_cast<float2*>(a.own + j0) = make_float2(th[0], th[1]);
+        } else {
+            if (changed[0]) a.own[j0] = th[0];
+            if (second && changed[1]) a.own[j0 + 1] = th[1];
+        }
+        if (a.measure) {
+            pe -= sx[0] * hx[0] + sy[0] * hy[0];
+            pmx += sx[0] + own_col[0].x;
+            pmy += sy[0] + own_col[0].y;
+            if (second) {
+                pe -= sx[1] * hx[1] + sy[1] * hy[1];
+                pmx += sx[1] + own_col[1].x;
+                pmy += sy[1] + own_col[1].y;
+            }
+        }
+    }
+    if (!a.measure) return;
+    const Partial mine = fp_partial(pe, pmx, pmy, 0.f, red);
     store_partial(a.partials, mine);
 }
 
@@ -1343,7 +1497,7 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
 __global__ void __launch_bounds__(kFinishThreads) on_finish_kernel(const OnArgs a,
                                                                    unsigned nblocks)
 {
-    const Partial tot = sum_partials<true>(a.partials, nblocks);
+    const Partial tot = sum_partials(a.partials, nblocks);
     if (threadIdx.x == 0) on_finish(a, tot);
 }
 
@@ -1578,6 +1732,30 @@ int on_rows(const sl_lattice* h, long long cols)
 
 // kernel variant: 0 Metropolis, 1 Metropolis with intrinsics, 2 heat-bath
 // (whose draws and fields use the accurate functions only)
+template <int D, bool EVEN>
+cudaError_t launch_xy_flat(const sl_lattice* h, const OnArgs& a, int var, cudaStream_t s)
+{
+    float2* cs = (float2*)h->staging;
+    const FastDiv Wd = make_fast_div((uint32_t)h->W), Ld = make_fast_div((uint32_t)h->L);
+    const uint32_t H = (uint32_t)h->H;
+    const int gv = grid_for(h->H, 256);
+    int g = grid_for((h->H + 1) / 2, 256);
+    // the measuring pass: no more blocks than are resident at once, so that its
+    // FP64 sums are few
+    if (a.measure && g > 4 * h->sms) g = 4 * h->sms;
+    // (heat-bath angles take the accurate functions whatever SL_OPT_FAST_MATH, as
+    // in the other kernels)
+    if (var == 1) xy_vectors<true><<<gv, 256, 0, s>>>(a.oth, cs, H);
+    else xy_vectors<false><<<gv, 256, 0, s>>>(a.oth, cs, H);
+    if (var == 2) xy_flat<D, EVEN, false, true><<<g, 256, 0, s>>>(a, cs, Wd, Ld);
+    else if (var == 1) xy_flat<D, EVEN, true, false><<<g, 256, 0, s>>>(a, cs, Wd, Ld);
+    else xy_flat<D, EVEN, false, false><<<g, 256, 0, s>>>(a, cs, Wd, Ld);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || !a.measure) return e;
+    on_finish_kernel<<<1, kFinishThreads, 0, s>>>(a, (unsigned)g);
+    return cudaGetLastError();
+}
+
 template <int NC>
 cudaError_t launch_on(const sl_lattice* h, OnArgs a, cudaStream_t s)
 {
@@ -1630,6 +1808,15 @@ cudaError_t launch_on(const sl_lattice* h, OnArgs a, cudaStream_t s)
             on_finish_kernel<<<1, kFinishThreads, 0, s>>>(a, (unsigned)grid);
         }
         return cudaGetLastError();
+    }
+    // XY sweeps with a uniform coupling (SL_OPT_KERNEL 1 asks for on_generic, which
+    // also takes float couplings, Heisenberg spins and the standalone measurement)
+    if (NC == 2 && a.update && h->j_layout == SL_J_UNIFORM && h->kernel != 1) {
+        if (h->d == 2)
+            return h->W % 2 == 0 ? launch_xy_flat<2, true>(h, a, var, s)
+                                 : launch_xy_flat<2, false>(h, a, var, s);
+        return h->W % 2 == 0 ? launch_xy_flat<3, true>(h, a, var, s)
+                             : launch_xy_flat<3, false>(h, a, var, s);
     }
     const long long rows = (long long)h->L * (h->d == 3 ? h->L : 1);
     const long long cap = (long long)h->sms * 8;

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(256) static_measure_kernel(const int8_t* s, lo
     mine.i0 = block_sum(bond, red);
     mine.i1 = block_sum(down, red);
     mine.f[0] = mine.f[1] = mine.f[2] = mine.f[3] = 0.0;
-    finish_pass(&scr->ctrl, scr->partials, mine, [&](const Partial& tot) {
+    finish_pass<false>(&scr->ctrl, scr->partials, mine, [&](const Partial& tot) {
         out[0] = -J * (double)tot.i0;
         out[1] = (double)(N - 2 * tot.i1);
     });
