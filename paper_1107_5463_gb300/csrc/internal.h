@@ -41,6 +41,18 @@ struct SweepParams {
     float beta_f;     // continuous spins
 };
 
+constexpr int kGraphSizes = 6;       // captured runs of 1, 2, 4 .. 32 sweeps
+
+// A run of sweeps captured into a graph with the finishing kernel of every
+// measuring pass on a side branch: it takes 2 us (Ising) to 8 us (FP64 totals)
+// that the next sweep's colour-0 pass need not wait for.  The passes of sweep k
+// read the sweep index as ctrl->t + k; the last finishing kernel advances it.
+struct SweepFork {
+    cudaStream_t side;
+    cudaEvent_t measured, finished;  // a measuring pass / its finishing kernel is done
+    unsigned k, count;               // sweep being captured, sweeps of the run
+};
+
 }  // namespace spinmc
 
 struct sl_lattice {
@@ -63,6 +75,8 @@ struct sl_lattice {
     int64_t sweeps_done;
     cudaStream_t stream;     // the caller's stream
     cudaStream_t cap_stream; // private stream used only to capture graphs
+    spinmc::SweepFork fork_res;   // the side stream and events (created at first use)
+    spinmc::SweepFork* fork;      // set while a forked run is captured, else null
     // views into the device buffer
     void* spins[2];          // per colour
     void* bonds[2][3];       // per colour, per direction (null for uniform J)
@@ -80,9 +94,8 @@ struct sl_lattice {
     int shape_tuned;         // rows and blocks_per_sm come from sl_autotune, not from the user
     int update;              // SL_UPDATE_METROPOLIS, _HEATBATH or _SW
     int multihit, tile;      // k-fold multi-hit sweeps in tiles of side `tile` (0 = off)
-    // cached graphs of kGraphSweeps sweeps and of one sweep
-    cudaGraphExec_t graph, graph1;
-    int graph_sweeps;
+    // cached graphs of 2^i sweeps, captured when a call first needs one
+    cudaGraphExec_t graphs[spinmc::kGraphSizes];
     uint64_t graph_key[4];
     void* owned_buf;
     // update workspace (Swendsen-Wang labels), caller-owned unless ws_owned
@@ -109,8 +122,22 @@ int sweep_params(const sl_lattice* h, double beta, uint64_t seed, SweepParams* p
 cudaError_t set_sweep_index(const sl_lattice* h, int64_t t, cudaStream_t s);
 cudaError_t clear_series(const sl_lattice* h, cudaStream_t s);
 void forget_graphs(sl_lattice* h);
+// forked runs: which sweep's index and how far the finishing kernel advances it;
+// the stream of a finishing kernel; the joins around it (lattice.cu)
+inline unsigned fork_offset(const sl_lattice* h) { return h->fork ? h->fork->k : 0u; }
+inline unsigned fork_advance(const sl_lattice* h)
+{
+    return !h->fork ? 1u : (h->fork->k + 1 == h->fork->count ? h->fork->count : 0u);
+}
+void fork_sweep(const sl_lattice* h, int64_t k);
+cudaError_t fork_join(const sl_lattice* h, cudaStream_t s);           // before a measuring pass
+cudaError_t finish_begin(const sl_lattice* h, cudaStream_t s, cudaStream_t* out);
+cudaError_t finish_end(const sl_lattice* h, cudaStream_t fs);
 // whether a lattice's sweeps run the row-streaming kernels (ising_i8.cu, on_f32.cu)
 bool i8_streams(const sl_lattice* h);
+// whether its measuring passes are closed by a separate kernel
+bool i8_deferred(const sl_lattice* h);
+bool on_deferred(const sl_lattice* h);
 bool on_streams(const sl_lattice* h);
 bool on_tile_ok(const sl_lattice* h);  // the staged 3D Heisenberg kernel applies
 

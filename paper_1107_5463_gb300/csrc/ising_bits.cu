@@ -31,6 +31,8 @@ struct BitArgs {
     IsingTable tab;
     RoundKeys rk;
     Ctrl* ctrl;
+    unsigned toff;     // sweep index of the pass: ctrl->t + toff
+    unsigned tadvance; // added to ctrl->t when the pass is closed
     Partial* partials;
     double J;
     int measure, update;
@@ -50,11 +52,11 @@ __device__ __forceinline__ void bits_finish(const BitArgs& a, const Partial& tot
     C->obs[2] = 0.0;
     C->obs[3] = 0.0;
     if (a.update) {
-        const long long k = (long long)C->t - C->series_base;
+        const long long k = (long long)C->t + a.toff - C->series_base;
         if (C->series_E) C->series_E[k] = E;
         // a slab records its own M (summed over slabs, |M| / N is |m|)
         if (C->series_absm) C->series_absm[k] = a.wrap ? fabs(M) / (double)a.N : M;
-        C->t = C->t + 1;
+        C->t = C->t + a.tadvance;
     }
 }
 
@@ -73,7 +75,7 @@ template <int D, int JNEG, bool MEAS, bool SLAB = false>
 __global__ void __launch_bounds__(128) bits_stream(const BitArgs a)
 {
     __shared__ long long red[32];
-    const uint32_t t = (uint32_t)a.ctrl->t;
+    const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
     const int L = a.L, R = a.R, Lz = SLAB ? a.Lz : a.L;
     const int WW = a.W >> 5;  // words per row
     const long long nseg = Lz / R;
@@ -348,6 +350,8 @@ BitArgs make_args(const sl_lattice* h, int c)
     a.N = h->N;
     a.replica = h->replica;
     a.ctrl = h->ctrl;
+    a.toff = fork_offset(h);
+    a.tadvance = fork_advance(h);
     a.partials = h->partials;
     a.J = h->J;
     a.measure = c == 1;
@@ -383,12 +387,12 @@ cudaError_t launch(const sl_lattice* h, const BitArgs& a, cudaStream_t s)
         else SPINMC_BITS(3, 0);
     }
 #undef SPINMC_BITS
-    if (a.measure) {
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        bits_finish_kernel<<<1, 1, 0, s>>>(a);
-    }
-    return cudaGetLastError();
+    if (!a.measure) return cudaGetLastError();
+    cudaStream_t fs;
+    const cudaError_t e = finish_begin(h, s, &fs);
+    if (e != cudaSuccess) return e;
+    bits_finish_kernel<<<1, 1, 0, fs>>>(a);
+    return finish_end(h, fs);
 }
 
 }  // namespace
@@ -430,14 +434,17 @@ cudaError_t ising_bits_gather(const sl_lattice* h, int8_t* nat, cudaStream_t s)
 cudaError_t ising_bits_sweeps(const sl_lattice* h, const SweepParams& p, int64_t count,
                               cudaStream_t s)
 {
-    for (int64_t k = 0; k < count; ++k)
+    for (int64_t k = 0; k < count; ++k) {
+        fork_sweep(h, k);
         for (int c = 0; c < 2; ++c) {
             BitArgs a = make_args(h, c);
             a.tab = p.tab;
             a.rk = p.rk;
-            const cudaError_t e = launch(h, a, s);
+            cudaError_t e = c == 1 ? fork_join(h, s) : cudaSuccess;
+            if (e == cudaSuccess) e = launch(h, a, s);
             if (e != cudaSuccess) return e;
         }
+    }
     return cudaSuccess;
 }
 

@@ -50,6 +50,8 @@ struct I8Args {
     IsingTable tab;
     RoundKeys rk;
     Ctrl* ctrl;
+    unsigned toff;     // sweep index of the pass: ctrl->t + toff
+    unsigned tadvance; // added to ctrl->t when the pass is closed
     Partial* partials;
     double J;
     int measure;  // accumulate E and M and finish the pass
@@ -72,11 +74,11 @@ __device__ __forceinline__ void i8_finish(const I8Args& a, const Partial& tot)
     C->obs[2] = 0.0;
     C->obs[3] = 0.0;
     if (a.update || a.advance) {
-        const long long k = (long long)C->t - C->series_base;
+        const long long k = (long long)C->t + a.toff - C->series_base;
         if (C->series_E) C->series_E[k] = E;
         // a slab records its own M (summed over slabs, |M| / N is |m|)
         if (C->series_absm) C->series_absm[k] = a.wrap ? fabs(M) / (double)a.N : M;
-        C->t = C->t + 1;
+        C->t = C->t + a.tadvance;
     }
 }
 
@@ -98,7 +100,7 @@ template <int D>
 __global__ void __launch_bounds__(256) i8_generic(const I8Args a)
 {
     __shared__ long long red[32];
-    const uint32_t t = (uint32_t)a.ctrl->t;
+    const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
     const long long ngroups = (a.H + 3) >> 2;
     const int L = a.L;
     long long bond = 0, down = 0;
@@ -192,7 +194,7 @@ __global__ void __launch_bounds__(256) i8_flat(const I8Args a, const FastDiv Wd,
     e.P = D == 3 ? a.L * a.W : a.W;
     e.H = (int)a.H;
     const PhiloxGroups pg =
-        philox_groups((uint32_t)a.ctrl->t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
+        philox_groups((uint32_t)a.ctrl->t + a.toff, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
     const GroupSign sg = group_sign<D>(a.tab);
     const uint8_t* o = reinterpret_cast<const uint8_t*>(a.oth);
     const int ngroups = (int)((a.H + 3) >> 2);
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
         if (threadIdx.x < 13) s_hb[threadIdx.x] = a.tab.hb[threadIdx.x];
         __syncthreads();
     }
-    const uint32_t t = (uint32_t)a.ctrl->t;
+    const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
     const int W = a.W, L = a.L, R = a.R, Lz = SLAB ? a.Lz : a.L;
     const int W16 = W >> 4;
     const long long nseg = Lz / R;
@@ -701,6 +703,8 @@ I8Args make_args(const sl_lattice* h, int c)
     a.N = h->N;
     a.replica = h->replica;
     a.ctrl = h->ctrl;
+    a.toff = fork_offset(h);
+    a.tadvance = fork_advance(h);
     a.partials = h->partials;
     a.J = h->J;
     a.measure = c == 1;
@@ -736,6 +740,15 @@ int pick_rows(const sl_lattice* h)
 
 __global__ void i8_finish_kernel(const I8Args a);
 
+cudaError_t launch_finish(const sl_lattice* h, const I8Args& a, cudaStream_t s)
+{
+    cudaStream_t fs;
+    const cudaError_t e = finish_begin(h, s, &fs);
+    if (e != cudaSuccess) return e;
+    i8_finish_kernel<<<1, 1, 0, fs>>>(a);
+    return finish_end(h, fs);
+}
+
 // whole lattices with a uniform coupling (SL_OPT_KERNEL 1 asks for i8_generic)
 bool flat_ok(const sl_lattice* h)
 {
@@ -753,10 +766,7 @@ cudaError_t launch_flat(const sl_lattice* h, const I8Args& a, cudaStream_t s)
     else if (a.tab.heatbath) i8_flat<D, ALIGNED, true, true, false><<<grid, 256, 0, s>>>(a, Wd, Ld);
     else if (a.measure) i8_flat<D, ALIGNED, false, true, true><<<grid, 256, 0, s>>>(a, Wd, Ld);
     else i8_flat<D, ALIGNED, false, true, false><<<grid, 256, 0, s>>>(a, Wd, Ld);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !a.measure) return e;
-    i8_finish_kernel<<<1, 1, 0, s>>>(a);
-    return cudaGetLastError();
+    return a.measure ? launch_finish(h, a, s) : cudaGetLastError();
 }
 
 cudaError_t launch_pass(const sl_lattice* h, I8Args a, cudaStream_t s, bool stream)
@@ -800,11 +810,7 @@ cudaError_t launch_pass(const sl_lattice* h, I8Args a, cudaStream_t s, bool stre
             else { if (jneg) SPINMC_LAUNCH(3, 0, 1, 0); else SPINMC_LAUNCH(3, 0, 0, 0); }
         }
 #undef SPINMC_LAUNCH
-        if (a.defer) {
-            const cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            i8_finish_kernel<<<1, 1, 0, s>>>(a);
-        }
+        if (a.defer) return launch_finish(h, a, s);
     } else {
         int grid = grid_for((h->H + 3) >> 2, 256);
         if (a.measure && grid > kI8Blocks) grid = kI8Blocks;
@@ -884,11 +890,13 @@ cudaError_t ising_i8_sweeps(const sl_lattice* h, const SweepParams& p, int64_t c
     }
     const bool stream = h->kernel == 2 || (h->kernel == 0 && stream_ok(h));
     for (int64_t k = 0; k < count; ++k) {
+        fork_sweep(h, k);
         for (int c = 0; c < 2; ++c) {
             I8Args a = make_args(h, c);
             a.tab = p.tab;
             a.rk = p.rk;
-            const cudaError_t e = launch_pass(h, a, s, stream);
+            cudaError_t e = c == 1 ? fork_join(h, s) : cudaSuccess;
+            if (e == cudaSuccess) e = launch_pass(h, a, s, stream);
             if (e != cudaSuccess) return e;
         }
     }
@@ -899,6 +907,11 @@ bool i8_streams(const sl_lattice* h)
 {
     return h->multihit == 0 && h->update != SL_UPDATE_SW &&
            (h->kernel == 2 || (h->kernel == 0 && stream_ok(h)));
+}
+
+bool i8_deferred(const sl_lattice* h)
+{
+    return i8_streams(h) || (h->multihit == 0 && h->update != SL_UPDATE_SW && flat_ok(h));
 }
 
 cudaError_t ising_i8_pass(const sl_lattice* h, const SweepParams& p, int c, cudaStream_t s)

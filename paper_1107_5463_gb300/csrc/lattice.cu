@@ -33,8 +33,6 @@ int cuda_fail(cudaError_t e, const char* what)
 
 namespace {
 
-constexpr int kGraphSweeps = 32;  // sweeps in the long graph; a one-sweep graph takes the rest
-
 struct Layout {
     size_t spin_colour;   // bytes of one colour's spins
     size_t bond_array;    // bytes of one (colour, direction) bond array
@@ -197,13 +195,42 @@ int model_sweeps(const sl_lattice* h, const SweepParams& p, int64_t count, cudaS
     return e == cudaSuccess ? SL_OK : cuda_fail(e, "sweep launch");
 }
 
+bool deferred_finish(const sl_lattice* h)
+{
+    if (h->storage == SL_STORE_I8) return i8_deferred(h);
+    return h->storage == SL_STORE_BITS || on_deferred(h);
+}
+
+cudaError_t fork_init(SweepFork* f)
+{
+    if (f->finished) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    if (!f->side) e = cudaStreamCreateWithFlags(&f->side, cudaStreamNonBlocking);
+    if (e == cudaSuccess && !f->measured)
+        e = cudaEventCreateWithFlags(&f->measured, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&f->finished, cudaEventDisableTiming);
+    return e;
+}
+
 // Capture `count` sweeps into an executable graph on the private capture stream.
 int capture_sweeps(sl_lattice* h, const SweepParams& p, int count, cudaGraphExec_t* out)
 {
     *out = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
+    const bool forked = count > 1 && deferred_finish(h);
+    cudaError_t e = forked ? fork_init(&h->fork_res) : cudaSuccess;
+    if (e == cudaSuccess)
+        e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
-    const int st = model_sweeps(h, p, count, h->cap_stream);
+    if (forked) {
+        h->fork = &h->fork_res;
+        h->fork->count = (unsigned)count;
+    }
+    int st = model_sweeps(h, p, count, h->cap_stream);
+    if (forked && st == SL_OK) {
+        e = cudaStreamWaitEvent(h->cap_stream, h->fork->finished, 0);
+        if (e != cudaSuccess) st = cuda_fail(e, "join the finishing kernels");
+    }
+    h->fork = nullptr;
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(h->cap_stream, &g);
     if (st != SL_OK) {
@@ -222,16 +249,17 @@ int capture_sweeps(sl_lattice* h, const SweepParams& p, int count, cudaGraphExec
 
 void drop_graphs(sl_lattice* h)
 {
-    if (h->graph) cudaGraphExecDestroy(h->graph);
-    if (h->graph1) cudaGraphExecDestroy(h->graph1);
-    h->graph = h->graph1 = nullptr;
+    for (cudaGraphExec_t& g : h->graphs) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
 }
 
-// The two graphs of the sweep parameters p (kGraphSweeps sweeps and one
-// sweep), captured again only when p or an option that shapes the launches
-// has changed.  The kernels read the sweep index and the series pointers
-// from the device control block, so one capture serves every later call.
-int ensure_graph(sl_lattice* h, const SweepParams& p)
+// Drop the graphs unless they were captured with the sweep parameters p and the
+// options that shape the launches.  The kernels read the sweep index and the
+// series pointers from the device control block, so a capture serves every
+// later call.
+void check_graph_key(sl_lattice* h, const SweepParams& p)
 {
     uint64_t key[4];
     std::memcpy(&key[0], &p.beta, 8);
@@ -241,17 +269,9 @@ int ensure_graph(sl_lattice* h, const SweepParams& p)
              (uint64_t)h->renorm_every;
     key[3] = ((uint64_t)h->multihit << 16) ^ (uint64_t)h->tile ^
              ((uint64_t)h->blocks_per_sm << 40);
-    if (h->graph && h->graph1 && std::memcmp(key, h->graph_key, sizeof key) == 0) return SL_OK;
+    if (std::memcmp(key, h->graph_key, sizeof key) == 0) return;
     drop_graphs(h);
-    int st = capture_sweeps(h, p, kGraphSweeps, &h->graph);
-    if (st == SL_OK) st = capture_sweeps(h, p, 1, &h->graph1);
-    if (st != SL_OK) {
-        drop_graphs(h);
-        return st;
-    }
-    h->graph_sweeps = kGraphSweeps;
     std::memcpy(h->graph_key, key, sizeof key);
-    return SL_OK;
 }
 
 int sync_and_check(sl_lattice* h)
@@ -416,9 +436,10 @@ int create_lattice(int d, int L, int n, int j_layout, int storage, double J, con
     h->update = 0;
     h->multihit = 0;
     h->tile = 16;
-    h->graph = nullptr;
-    h->graph1 = nullptr;
-    h->graph_sweeps = 0;
+    h->fork_res = SweepFork{};
+    h->fork = nullptr;
+    for (cudaGraphExec_t& g : h->graphs) g = nullptr;
+    std::memset(h->graph_key, 0, sizeof h->graph_key);
     h->next_colour = 0;
     h->ev = nullptr;
     h->owned_buf = owned;
@@ -497,6 +518,34 @@ cudaError_t clear_series(const sl_lattice* h, cudaStream_t s)
 
 void forget_graphs(sl_lattice* h) { drop_graphs(h); }
 
+void fork_sweep(const sl_lattice* h, int64_t k)
+{
+    if (h->fork) h->fork->k = (unsigned)k;
+}
+
+cudaError_t fork_join(const sl_lattice* h, cudaStream_t s)
+{
+    // the previous sweep's finishing kernel has read and cleared the partials
+    return h->fork && h->fork->k > 0 ? cudaStreamWaitEvent(s, h->fork->finished, 0) : cudaSuccess;
+}
+
+cudaError_t finish_begin(const sl_lattice* h, cudaStream_t s, cudaStream_t* out)
+{
+    *out = s;
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || !h->fork) return e;
+    e = cudaEventRecord(h->fork->measured, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(h->fork->side, h->fork->measured, 0);
+    *out = h->fork->side;
+    return e;
+}
+
+cudaError_t finish_end(const sl_lattice* h, cudaStream_t fs)
+{
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess && h->fork ? cudaEventRecord(h->fork->finished, fs) : e;
+}
+
 }  // namespace spinmc
 
 extern "C" {
@@ -536,14 +585,20 @@ int sl_sweep_series(sl_lattice* h, double beta, int64_t nsweeps, uint64_t seed, 
         left = 0;
     }
     if (h->use_graph && left >= 2) {
-        // whole runs of kGraphSweeps sweeps, then single-sweep replays
-        const int st = ensure_graph(h, p);
-        if (st != SL_OK) return st;
+        // runs of 32 sweeps, then one each of the powers of two that make up the
+        // rest: a graph costs a launch, and inside one the finishing kernels run
+        // beside the next sweep
+        check_graph_key(h, p);
         while (left > 0) {
-            const bool big = left >= h->graph_sweeps;
-            e = cudaGraphLaunch(big ? h->graph : h->graph1, h->stream);
+            int i = kGraphSizes - 1;
+            while ((1LL << i) > left) --i;
+            if (!h->graphs[i]) {
+                const int st = capture_sweeps(h, p, 1 << i, &h->graphs[i]);
+                if (st != SL_OK) return st;
+            }
+            e = cudaGraphLaunch(h->graphs[i], h->stream);
             if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
-            left -= big ? h->graph_sweeps : 1;
+            left -= 1LL << i;
         }
     }
     if (left > 0) {
@@ -754,6 +809,9 @@ void sl_destroy(sl_lattice* h)
     drop_graphs(h);
     if (h->ev) cudaEventDestroy(h->ev);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
+    if (h->fork_res.side) cudaStreamDestroy(h->fork_res.side);
+    if (h->fork_res.measured) cudaEventDestroy(h->fork_res.measured);
+    if (h->fork_res.finished) cudaEventDestroy(h->fork_res.finished);
     if (h->owned_buf) cudaFree(h->owned_buf);
     if (h->ws_owned) cudaFree(h->ws_owned);
     delete h;

@@ -48,6 +48,8 @@ struct OnArgs {
     float beta;
     float J;
     Ctrl* ctrl;
+    unsigned toff;     // sweep index of the pass: ctrl->t + toff
+    unsigned tadvance; // added to ctrl->t when the pass is closed
     Partial* partials;
     int measure, update;
     int renorm_every;  // Heisenberg: normalise each updated spin when (t+1) % renorm_every == 0
@@ -329,11 +331,11 @@ __device__ __forceinline__ void on_finish(const OnArgs& a, const Partial& tot)
     C->obs[2] = tot.f[2];
     C->obs[3] = tot.f[3];
     if (a.update) {
-        const long long k = (long long)C->t - C->series_base;
+        const long long k = (long long)C->t + a.toff - C->series_base;
         const double m = sqrt(tot.f[1] * tot.f[1] + tot.f[2] * tot.f[2] + tot.f[3] * tot.f[3]);
         if (C->series_E) C->series_E[k] = tot.f[0];
         if (C->series_absm) C->series_absm[k] = m / (double)a.N;
-        C->t = C->t + 1;
+        C->t = C->t + a.tadvance;
     }
 }
 
@@ -343,7 +345,7 @@ template <int NC, int D, bool FAST, bool HB>
 __global__ void __launch_bounds__(128) on_generic(const OnArgs a)
 {
     __shared__ double red[32];  // 4 per warp
-    const unsigned long long t64 = a.ctrl->t;
+    const unsigned long long t64 = a.ctrl->t + a.toff;
     const uint32_t t = (uint32_t)t64;
     const bool renorm = NC == 3 && a.update && a.renorm_every > 0 &&
                         (t64 + 1) % (unsigned long long)a.renorm_every == 0;
@@ -534,7 +536,7 @@ __global__ void __launch_bounds__(256, D == 2 && !HB ? 4 : 3) heis_stream(const 
     constexpr bool TAB = !FAST && !HB;
     __shared__ float2 tab[TAB ? kTurnTab : 1];
     if (TAB) fill_turn_table(tab);
-    const unsigned long long t64 = a.ctrl->t;
+    const unsigned long long t64 = a.ctrl->t + a.toff;
     const uint32_t t = (uint32_t)t64;
     const bool renorm = a.update && a.renorm_every > 0 &&
                         (t64 + 1) % (unsigned long long)a.renorm_every == 0;
@@ -685,7 +687,7 @@ __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
     constexpr bool TAB = !FAST && !HB;
     __shared__ float2 tab[TAB ? kTurnTab : 1];
     if (TAB) fill_turn_table(tab);
-    const unsigned long long t64 = a.ctrl->t;
+    const unsigned long long t64 = a.ctrl->t + a.toff;
     const uint32_t t = (uint32_t)t64;
     const bool renorm = a.update && a.renorm_every > 0 &&
                         (t64 + 1) % (unsigned long long)a.renorm_every == 0;
@@ -983,7 +985,7 @@ __global__ void __launch_bounds__(kTileThreads, 3) heis_tile3(const OnArgs a)
     __shared__ __align__(8) unsigned long long bars[kOthStages + kOwnStages];
     __shared__ double red[32];  // 4 per warp
     fill_turn_table(tab);
-    const unsigned long long t64 = a.ctrl->t;
+    const unsigned long long t64 = a.ctrl->t + a.toff;
     const uint32_t t = (uint32_t)t64;
     const bool renorm = a.update && a.renorm_every > 0 &&
                         (t64 + 1) % (unsigned long long)a.renorm_every == 0;
@@ -1169,7 +1171,7 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
         sc(th.y, &r.s1, &r.c1);
         return r;
     };
-    const uint32_t t = (uint32_t)a.ctrl->t;
+    const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
     const int L = a.L, W = a.W, R = a.R;
     const int WP = W / 2;
     const int lane = threadIdx.x & 31;
@@ -1345,7 +1347,7 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
     const int L = a.L, W = a.W, H = (int)a.H, P = D == 3 ? L * W : W;
     const float J = a.J;
     const PhiloxGroups pg =
-        philox_groups((uint32_t)a.ctrl->t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
+        philox_groups((uint32_t)a.ctrl->t + a.toff, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
     const int ncalls = (H + 1) / 2;
     float pe = 0.f, pmx = 0.f, pmy = 0.f;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < ncalls; q += gridDim.x * blockDim.x) {
@@ -1432,7 +1434,7 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
             uint32_t acc0 = 0u, acc1 = 0u;
             for (int at = 0; at < kVonMisesAttempts && (p0 || p1); ++at) {
                 const uint4 rnd = philox4x32_10(
-                    make_uint4((uint32_t)q, (uint32_t)a.ctrl->t, a.replica,
+                    make_uint4((uint32_t)q, (uint32_t)a.ctrl->t + a.toff, a.replica,
                                ((uint32_t)at << 16) | (kSweep << 1) | (uint32_t)a.c),
                     a.rk);
                 if (p0 && von_mises_accept(m0, rnd.x, rnd.y)) {
@@ -1639,6 +1641,8 @@ OnArgs make_args(const sl_lattice* h, int c)
     a.replica = h->replica;
     a.J = (float)h->J;
     a.ctrl = h->ctrl;
+    a.toff = fork_offset(h);
+    a.tadvance = fork_advance(h);
     a.partials = h->partials;
     a.measure = c == 1;
     a.update = 1;
@@ -1655,6 +1659,15 @@ bool tile_ok(const sl_lattice* h)
     return h->n == 3 && h->d == 3 && h->bonds[0][0] == nullptr && !h->slab &&
            (W == 32 || W == 64 || W == 128 || W == 256) && h->update == SL_UPDATE_METROPOLIS &&
            !h->fast_math;
+}
+
+cudaError_t launch_finish(const sl_lattice* h, const OnArgs& a, unsigned nblocks, cudaStream_t s)
+{
+    cudaStream_t fs;
+    const cudaError_t e = finish_begin(h, s, &fs);
+    if (e != cudaSuccess) return e;
+    on_finish_kernel<<<1, kFinishThreads, 0, fs>>>(a, nblocks);
+    return finish_end(h, fs);
 }
 
 cudaError_t launch_tile(const sl_lattice* h, const OnArgs& a, cudaStream_t s)
@@ -1680,10 +1693,12 @@ cudaError_t launch_tile(const sl_lattice* h, const OnArgs& a, cudaStream_t s)
     if (grid > kMaxBlocks) grid = kMaxBlocks;
     if (a.measure) heis_tile3<true><<<(int)grid, kTileThreads, dyn, s>>>(a);
     else heis_tile3<false><<<(int)grid, kTileThreads, dyn, s>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !a.measure) return e;
-    on_finish_kernel<<<1, kFinishThreads, 0, s>>>(a, (unsigned)grid);
-    return cudaGetLastError();
+    return a.measure ? launch_finish(h, a, (unsigned)grid, s) : cudaGetLastError();
+}
+
+bool xy_flat_ok(const sl_lattice* h)
+{
+    return h->n == 2 && h->j_layout == SL_J_UNIFORM && h->kernel != 1;
 }
 
 bool on_stream_ok(const sl_lattice* h)
@@ -1696,6 +1711,8 @@ bool on_stream_ok(const sl_lattice* h)
 }  // namespace
 
 bool on_streams(const sl_lattice* h) { return on_stream_ok(h) || (h->kernel == 4 && tile_ok(h)); }
+
+bool on_deferred(const sl_lattice* h) { return on_streams(h) || xy_flat_ok(h); }
 
 bool on_tile_ok(const sl_lattice* h) { return tile_ok(h); }
 
@@ -1750,10 +1767,7 @@ cudaError_t launch_xy_flat(const sl_lattice* h, const OnArgs& a, int var, cudaSt
     if (var == 2) xy_flat<D, EVEN, false, true><<<g, 256, 0, s>>>(a, cs, Wd, Ld);
     else if (var == 1) xy_flat<D, EVEN, true, false><<<g, 256, 0, s>>>(a, cs, Wd, Ld);
     else xy_flat<D, EVEN, false, false><<<g, 256, 0, s>>>(a, cs, Wd, Ld);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !a.measure) return e;
-    on_finish_kernel<<<1, kFinishThreads, 0, s>>>(a, (unsigned)g);
-    return cudaGetLastError();
+    return a.measure ? launch_finish(h, a, (unsigned)g, s) : cudaGetLastError();
 }
 
 template <int NC>
@@ -1802,16 +1816,11 @@ cudaError_t launch_on(const sl_lattice* h, OnArgs a, cudaStream_t s)
             else SPINMC_ON(xy_stream, false, false);
         }
 #undef SPINMC_ON
-        if (a.measure) {
-            const cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            on_finish_kernel<<<1, kFinishThreads, 0, s>>>(a, (unsigned)grid);
-        }
-        return cudaGetLastError();
+        return a.measure ? launch_finish(h, a, (unsigned)grid, s) : cudaGetLastError();
     }
     // XY sweeps with a uniform coupling (SL_OPT_KERNEL 1 asks for on_generic, which
     // also takes float couplings, Heisenberg spins and the standalone measurement)
-    if (NC == 2 && a.update && h->j_layout == SL_J_UNIFORM && h->kernel != 1) {
+    if (a.update && xy_flat_ok(h)) {
         if (h->d == 2)
             return h->W % 2 == 0 ? launch_xy_flat<2, true>(h, a, var, s)
                                  : launch_xy_flat<2, false>(h, a, var, s);
@@ -1878,11 +1887,13 @@ cudaError_t float_bonds_scatter(const sl_lattice* h, const float* nat, cudaStrea
 cudaError_t on_sweeps(const sl_lattice* h, const SweepParams& p, int64_t count, cudaStream_t s)
 {
     for (int64_t k = 0; k < count; ++k) {
+        fork_sweep(h, k);
         for (int c = 0; c < 2; ++c) {
             OnArgs a = make_args(h, c);
             a.rk = p.rk;
             a.beta = p.beta_f;
-            const cudaError_t e = h->n == 2 ? launch_on<2>(h, a, s) : launch_on<3>(h, a, s);
+            cudaError_t e = c == 1 ? fork_join(h, s) : cudaSuccess;
+            if (e == cudaSuccess) e = h->n == 2 ? launch_on<2>(h, a, s) : launch_on<3>(h, a, s);
             if (e != cudaSuccess) return e;
         }
     }
