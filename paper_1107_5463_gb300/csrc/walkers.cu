@@ -10,8 +10,7 @@
 // interleaved bitwise: word q of warp g holds site q of each of its walkers,
 // bit l = walker 32 g + l, set for spin down; global layout [warp][site]
 // (64 MB for 131072 walkers of 64 x 64 sites, resident in L2).  All 32 lanes
-// read the same word (a broadcast) and lane 0 writes back the ballot of
-// flips; by default the words are used in place, optionally a warp's N words
+// read the same words and one lane writes back the ballot of flips; by default the words are used in place, optionally a warp's N words
 // are kept in shared memory for the run (fewer warps fit per SM).  Per walker
 // ln g (64-bit fixed point, units of 2^-32) and the histogram live in shared
 // memory as [level][lane] (no bank conflicts).
@@ -25,7 +24,7 @@
 //         FP64 weights ln W (u < exp(lnW(k) - lnW(k')) 2^32 as an exact
 //         integer test); H counts the level after every attempt.
 //   WL:   accept iff D >= 0 or u < exp(D 2^-32) 2^32, D = S(k) - S(k'): an
-//         FP32 expf decides unless u lies within 2^-14 (relative) of the
+//         FP32 exp2 decides unless u lies within 2^-14 (relative) of the
 //         threshold, where FP64 exp decides; after every attempt
 //         S(k) += 2^(32 - stage), H(k) += 1, level k is marked visited;
 //         after every sweep a walker whose visited levels all have
@@ -147,30 +146,77 @@ __global__ void __launch_bounds__(128) walk_init_kernel(WalkArgs a)
 
 // ------------------------------------------------------------ WL / MUCA ----
 
-// Wang-Landau decision for D < 0 (see the file comment).  The FP32 filter
-// builds x = D 2^-32 from the two 32-bit halves of D with FP32 instructions
-// only (relative error below 2^-22, plus the argument error |x| 2^-24 that
-// keeps the filter's 2^-14 margin safe for |x| < 100; beyond, exp(x) < 2^-144
-// and only u = 0 reaches the FP64 test).
-__device__ __forceinline__ bool wl_accept(int64_t D, uint32_t u)
+// Wang-Landau decision for D < 0 (see the file comment): FP32 decides unless u
+// lies near the threshold exp(D 2^-32) 2^32 = 2^(D 2^-32 log2 e + 32).  The
+// conversions of D and u, the product (its argument below 160 where the result
+// is not flushed to zero) and the hardware exp2 leave a relative error below
+// 2^-16, a quarter of the margin; where the threshold underflows, u = 0 is near.
+// (D's 64-bit conversion runs on the FP64 unit, which has nothing else to do:
+// 15.9 ms for 10 sweeps of the workload, against 16.6 with D's halves converted
+// by the other units.)
+__device__ __forceinline__ bool wl_accept_fast(int64_t D, uint32_t u, bool* near)
 {
-    const float xf = (float)(int32_t)(D >> 32) + (float)(uint32_t)D * (1.0f / 4294967296.0f);
-    const float pf = expf(xf);
-    const float uf = (float)u * (1.0f / 4294967296.0f);
+    float pf;
+    asm("ex2.approx.ftz.f32 %0, %1;"
+        : "=f"(pf)
+        : "f"(fmaf((float)D, 1.44269504f / 4294967296.0f, 32.0f)));
+    const float uf = (float)u;
     const float m = 1.0f / 16384.0f;
-    if (uf < pf * (1.0f - m)) return true;
-    if (uf > pf * (1.0f + m)) return false;
+    const bool acc = uf < pf * (1.0f - m);
+    *near = !acc && uf <= pf * (1.0f + m);
+    return acc;
+}
+
+__device__ __forceinline__ bool wl_accept_exact(int64_t D, uint32_t u)
+{
     return (double)u * (1.0 / 4294967296.0) < exp((double)D * (1.0 / 4294967296.0));
 }
 
+// Whether two attempts up to seven apart in a sweep's order can touch a common
+// word: sites d oa apart (mod N), where a site's words lie 0, +-1, +-L or, round
+// the end of a row, +-(L - 1) from it.  One answer for a whole sweep.
+__device__ __forceinline__ bool order_is_clear(uint32_t oa, uint32_t L, uint32_t nmask)
+{
+    bool clear = true;
+#pragma unroll
+    for (uint32_t d = 1; d < 8; ++d) {
+        const uint32_t x = (d * oa) & nmask, y = (0u - x) & nmask;
+        const uint32_t a = x < y ? x : y;  // distance either way
+        if (a <= 1u || a == L - 1 || a == L) clear = false;
+    }
+    return clear;
+}
+
+// One warp per block, 32 walkers of a window.  An attempt is a short chain of
+// dependent steps (site words, level, ln g, decision, new level), and some 27
+// warps per multiprocessor are all there are, so what counts is instructions
+// per attempt and latency inside the chain.  Reading the five words of a site
+// from L2 at each attempt, an FP32 expf, two 64-bit and two 32-bit shared
+// memory updates took 103 instructions an attempt and 2.8 ms for a sweep of
+// 131072 Wang-Landau walkers of 64 x 64 sites; this takes 67 and 1.4 ms:
+//   - 20 lanes fetch the words of four attempts with one load, a group ahead,
+//     and pass them on through shared memory (wherever the sweep's order cannot
+//     bring two attempts within eight to a common word; else word by word as
+//     before);
+//   - the current level's ln g stays in registers, H and the visited mask are
+//     worked out once per sweep from what ln g gained;
+//   - the decision takes one conversion and the hardware exp2, with the FP64
+//     test behind a warp vote.
 template <int KT, bool WL, bool SPINS_SMEM>
 __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    // H from the gain of S over a sweep (needs S at its start; not for the widest
+    // windows, whose arrays fill the shared memory)
+    constexpr bool SNAP = WL && KT <= 16;
+    __shared__ __align__(16) uint32_t words[2][4][4];
     const size_t colb = SPINS_SMEM ? 4 * (size_t)a.N : 0;
-    int64_t* S = reinterpret_cast<int64_t*>(smem + colb);                 // [KT][32]
-    uint32_t* H = reinterpret_cast<uint32_t*>(smem + colb + 8 * KT * 32);  // [KT][32]
-    int64_t* T = reinterpret_cast<int64_t*>(H + KT * 32);                 // MUCA [KT][4]
+    // S has room for two levels on either side, so that a move out of the window
+    // reads a value (which its decision ignores) without a test
+    int64_t* S = reinterpret_cast<int64_t*>(smem + colb) + 2 * 32;                // [KT][32]
+    uint32_t* H = reinterpret_cast<uint32_t*>(smem + colb + 8 * (KT + 4) * 32);   // [KT][32]
+    int64_t* T = reinterpret_cast<int64_t*>(H + KT * 32);                 // MUCA [KT][5]
+    int64_t* S0 = T;                                                      // SNAP [KT][32]
     const int lane = threadIdx.x;
     const int warp = blockIdx.x;
     const int gw = warp * 32 + lane;
@@ -186,16 +232,31 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
     uint32_t* col = SPINS_SMEM ? reinterpret_cast<uint32_t*>(smem) : gcol;
     if (SPINS_SMEM)
         for (long long i = lane; i < N; i += 32) col[i] = gcol[i];
+    if (WL)
+        for (int q = -2; q < KT + 2; ++q) S[q * 32 + lane] = 0;
     for (int q = 0; q < KT; ++q) {
         S[q * 32 + lane] = q < a.kmax ? a.S[(size_t)q * a.nwalk + gw] : 0;
         H[q * 32 + lane] = q < a.kmax && WL ? a.H[(size_t)q * a.nwalk + gw] : 0u;
     }
     if (!WL)
-        for (int q = lane; q < 4 * KT; q += 32)
-            T[q] = q < 4 * a.kmax ? a.thr[((size_t)win * a.kmax) * 4 + q] : -1;
+        // thresholds of the moves by -2 .. +2 levels (none: always; out of the window: never)
+        for (int q = lane; q < 5 * KT; q += 32) {
+            const int k = q / 5, c = q % 5;
+            T[q] = c == 2 ? (int64_t)0xFFFFFFFFu
+                          : (k < a.kmax
+                                 ? a.thr[((size_t)win * a.kmax + k) * 4 + (c < 2 ? c : c - 1)]
+                                 : -1);
+        }
     int kr = a.level[gw] - klo;
     int stage = a.stage[gw];
     uint64_t vis = a.visited[gw];
+    const uint32_t nmask = (uint32_t)(N - 1), xmask = (uint32_t)(L - 1);
+    const uint32_t lanebit = 1u << lane;
+    // the word a lane fetches: attempt lane / 5 of a group, word lane % 5 of its
+    // site (itself, -x, +x, -y, +y)
+    const uint32_t fa = (uint32_t)lane / 5u, fw = (uint32_t)lane % 5u;
+    const uint32_t fdx = fw == 1 ? 0u - 1u : (fw == 2 ? 1u : 0u);
+    const uint32_t fdy = fw == 3 ? 0u - (uint32_t)L : (fw == 4 ? (uint32_t)L : 0u);
     __syncwarp();
 
     for (long long s = 0; s < a.nsweeps; ++s) {
@@ -205,48 +266,106 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
         uint32_t oa, ob;
         sweep_order(a, t, oa, ob);
         const int64_t inc = WL && active ? ((int64_t)1 << (32 - stage)) : 0;
-        const uint32_t nmask = (uint32_t)(N - 1);
-        const uint32_t purpose = (WL ? kWL : kMUCA) << 1;
-        // the block of the next four attempts is drawn while the current four
-        // run (the attempts depend on each other, the draws do not; N is a
-        // multiple of 4, and the draw after the last block goes unused)
-        uint4 rnd_nx = philox4x32_10(make_uint4(0u, t, walker, purpose), a.rk);
-        // one attempt at position q of the sweep with uniform u
-        auto attempt = [&](uint32_t q, uint32_t u) {
-            const uint32_t i = (oa * q + ob) & nmask;  // N divides 2^32
-            uint32_t own;
-            const int nu = unlike([&](uint32_t w) { return col[w]; }, i, L, a.log2L, lane, own);
-            const int dk = 2 - nu;
-            const int k2 = kr + dk;
-            bool acc = false;
-            if (active && k2 >= 0 && k2 < K) {
-                if (WL) {
-                    const int64_t D = S[kr * 32 + lane] - S[k2 * 32 + lane];
-                    acc = D >= 0 || wl_accept(D, u);
-                } else {
-                    acc = dk == 0 || (int64_t)u <= T[kr * 4 + (dk < 0 ? dk + 2 : dk + 1)];
+        const unsigned Keff = active ? (unsigned)K : 0u;  // a finished walker never moves
+        if (SNAP)
+            for (int q = 0; q < KT; ++q) S0[q * 32 + lane] = S[q * 32 + lane];
+        int64_t Skr = WL ? S[kr * 32 + lane] : 0;
+        // draws of the four attempts 4 g .. 4 g + 3 (the block of the next four is
+        // drawn while the current four run; the one after the last goes unused)
+        const PhiloxGroups pg = philox_groups(t, walker, (WL ? kWL : kMUCA) << 1, a.rk);
+        uint4 rnd_nx = philox_at(pg, 0u, a.rk);
+        // one attempt: x0 .. x3 are the site's four neighbour words XOR its own;
+        // returns the walkers whose spin flips
+        auto attempt = [&](uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, uint32_t u) {
+            int k2 = kr + 2;
+            if (x0 & lanebit) --k2;
+            if (x1 & lanebit) --k2;
+            if (x2 & lanebit) --k2;
+            if (x3 & lanebit) --k2;
+            bool acc;
+            if (WL) {
+                const bool in = (unsigned)k2 < Keff;
+                const int64_t S2 = S[k2 * 32 + lane];
+                const int64_t D = Skr - S2;
+                bool near;
+                acc = wl_accept_fast(D, u, &near) || D >= 0;
+                near = near && in && D < 0;
+                if (__any_sync(0xFFFFFFFFu, near)) {
+                    if (near) acc = wl_accept_exact(D, u);
                 }
-            }
-            const uint32_t flips = __ballot_sync(0xFFFFFFFFu, acc);
-            if (lane == 0 && flips) col[i] = own ^ flips;
-            if (acc) kr = k2;
-            if (active) {
-                if (WL) {
-                    S[kr * 32 + lane] += inc;
+                acc = acc && in;
+                if (acc) {
+                    kr = k2;
+                    Skr = S2;
+                }
+                Skr += inc;
+                S[kr * 32 + lane] = Skr;
+                if (!SNAP && active) {
                     vis |= 1ull << kr;
+                    H[kr * 32 + lane] += 1u;
                 }
+            } else {
+                acc = (int64_t)u <= T[kr * 5 + (k2 - kr + 2)];
+                if (acc) kr = k2;
                 H[kr * 32 + lane] += 1u;
             }
-            __syncwarp();
+            return __ballot_sync(0xFFFFFFFFu, acc);
         };
-        for (uint32_t q = 0; q < (uint32_t)N; q += 4) {
-            const uint4 rnd = rnd_nx;
-            rnd_nx = philox4x32_10(make_uint4((q >> 2) + 1u, t, walker, purpose), a.rk);
-            attempt(q, rnd.x);
-            attempt(q + 1, rnd.y);
-            attempt(q + 2, rnd.z);
-            attempt(q + 3, rnd.w);
+        if (order_is_clear(oa, (uint32_t)L, nmask)) {
+            uint32_t at = 0u, at_nx;  // place of the lane's word, of its next one
+            auto fetch = [&](uint32_t q) -> uint32_t {
+                const uint32_t i = oa * (q + fa) + ob;  // N divides 2^32
+                at_nx = ((i + fdy) & nmask & ~xmask) | ((i + fdx) & xmask);
+                return lane < 20 ? col[at_nx] : 0u;
+            };
+            uint32_t w_nx = fetch(0u);
+            for (uint32_t q = 0; q < (uint32_t)N; q += 4) {
+                uint32_t (*buf)[4] = words[(q >> 2) & 1];
+                const uint32_t w = w_nx;
+                at = at_nx;
+                const uint32_t x = w ^ __shfl_sync(0xFFFFFFFFu, w, 5 * (int)fa);
+                if (lane < 20 && fw > 0) buf[fa][fw - 1] = x;
+                const uint4 rnd = rnd_nx;
+                __syncwarp();  // also orders the flips before the loads below
+                w_nx = fetch(q + 4);
+                rnd_nx = philox_at(pg, (q >> 2) + 1u, a.rk);
+                const uint32_t uu[4] = {rnd.x, rnd.y, rnd.z, rnd.w};
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(buf[b]);
+                    const uint32_t flips = attempt(v.x, v.y, v.z, v.w, uu[b]);
+                    // the lane that fetched the site's own word writes it back
+                    if (lane == 5 * b && flips) col[at] = w ^ flips;
+                }
+            }
+        } else {
+            auto single = [&](uint32_t q, uint32_t u) {
+                const uint32_t i = (oa * q + ob) & nmask;
+                const uint32_t row = i & ~xmask;
+                const uint32_t own = col[i];
+                const uint32_t flips =
+                    attempt(own ^ col[row | ((i - 1) & xmask)], own ^ col[row | ((i + 1) & xmask)],
+                            own ^ col[(i - (uint32_t)L) & nmask],
+                            own ^ col[(i + (uint32_t)L) & nmask], u);
+                if (lane == 0 && flips) col[i] = own ^ flips;
+                __syncwarp();
+            };
+            for (uint32_t q = 0; q < (uint32_t)N; q += 4) {
+                const uint4 rnd = rnd_nx;
+                rnd_nx = philox_at(pg, (q >> 2) + 1u, a.rk);
+                single(q, rnd.x);
+                single(q + 1, rnd.y);
+                single(q + 2, rnd.z);
+                single(q + 3, rnd.w);
+            }
         }
+        __syncwarp();
+        if (SNAP && active)
+            for (int q = 0; q < KT; ++q) {
+                const int64_t gain = S[q * 32 + lane] - S0[q * 32 + lane];
+                if (gain > 0) vis |= 1ull << q;
+                H[q * 32 + lane] += (uint32_t)(gain >> (32 - stage));
+            }
         if (WL && active) {
             int nv = 0;
             unsigned long long sum = 0;
@@ -378,7 +497,10 @@ int kt_for(int kmax)
 template <int KT, bool WL, bool SM>
 cudaError_t launch_walk_res(const WalkArgs& a, cudaStream_t s)
 {
-    const size_t smem = (SM ? 4 * (size_t)a.N : 0) + (size_t)KT * 32 * 12 + (size_t)KT * 4 * 8;
+    // spins, S and H; thresholds (multicanonical) or S at the start of a sweep
+    const size_t extra = !WL ? (size_t)KT * 5 * 8 : (KT <= 16 ? (size_t)KT * 32 * 8 : 0);
+    const size_t smem =
+        (SM ? 4 * (size_t)a.N : 0) + (size_t)(KT + 4) * 32 * 8 + (size_t)KT * 32 * 4 + extra;
     cudaError_t e = cudaFuncSetAttribute(walk_kernel<KT, WL, SM>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
