@@ -63,12 +63,27 @@ __device__ __forceinline__ PhiloxGroups philox_groups(uint32_t t, uint32_t repli
     return c;
 }
 
-__device__ __forceinline__ uint4 philox_at(const PhiloxGroups& pg, uint32_t g, const RoundKeys& rk)
+// What the first two rounds make of g alone, for one z1 (a colour's w).
+struct PhiloxHead {
+    uint32_t x, y, z;
+};
+
+__device__ __forceinline__ PhiloxHead philox_head(uint32_t g, uint32_t z1)
 {
     const uint64_t p0 = (uint64_t)g * 0xD2511F53u;
-    const uint32_t z1 = (uint32_t)(p0 >> 32) ^ pg.z1;
-    const uint64_t p1 = (uint64_t)z1 * 0xCD9E8D57u;
-    uint4 c = make_uint4((uint32_t)(p1 >> 32) ^ pg.x2, (uint32_t)p1, (uint32_t)p0 ^ pg.z2, pg.w2);
+    const uint64_t p1 = (uint64_t)((uint32_t)(p0 >> 32) ^ z1) * 0xCD9E8D57u;
+    PhiloxHead h;
+    h.x = (uint32_t)(p1 >> 32);
+    h.y = (uint32_t)p1;
+    h.z = (uint32_t)p0;
+    return h;
+}
+
+// Both parts and the other eight rounds.
+__device__ __forceinline__ uint4 philox_tail(const PhiloxHead& h, uint32_t x2, uint32_t z2,
+                                             uint32_t w2, const RoundKeys& rk)
+{
+    uint4 c = make_uint4(h.x ^ x2, h.y, h.z ^ z2, w2);
 #pragma unroll
     for (int r = 2; r < 10; ++r) {
         const uint64_t a = (uint64_t)c.x * 0xD2511F53u;
@@ -77,6 +92,11 @@ __device__ __forceinline__ uint4 philox_at(const PhiloxGroups& pg, uint32_t g, c
                        (uint32_t)(a >> 32) ^ c.w ^ rk.k1[r], (uint32_t)a);
     }
     return c;
+}
+
+__device__ __forceinline__ uint4 philox_at(const PhiloxGroups& pg, uint32_t g, const RoundKeys& rk)
+{
+    return philox_tail(philox_head(g, pg.z1), pg.x2, pg.z2, pg.w2, rk);
 }
 
 enum Purpose : uint32_t { kSweep = 0, kInit = 1, kCoupling = 2, kExchange = 3 };
