@@ -5,7 +5,8 @@
 // amalgamation of the tiles through a union-and-find structure).
 //
 // One update is five kernels:
-//   sw_local    one CTA per tile (64 x 32 sites in 2D, 64 x 16 x 8 in 3D):
+//   sw_local2, sw_local3
+//               one CTA per tile (64 x 32 sites in 2D, 64 x 16 x 8 in 3D):
 //               loads the tile's spins and a one-site halo on its +x/+y/+z
 //               faces into shared memory (one warp per row, one lane per site
 //               pair), draws the bond uniforms, joins each row's x-runs of
@@ -48,7 +49,8 @@ constexpr uint32_t kSwBond = 5, kSwFlip = 6;
 constexpr uint32_t kMask = 0x3FFFFFFFu;     // parent index
 constexpr uint32_t kTileRoot = 0x80000000u;  // the site is a tile root
 constexpr uint32_t kFlipBit = 0x40000000u;   // the cluster rooted here flips
-constexpr int kSwThreads = 512;
+constexpr int kSwThreads = 512;    // 3D tiles
+constexpr int kSwThreads2 = 256;   // 2D tiles
 
 template <int D>
 struct SwTile;
@@ -77,6 +79,7 @@ struct SwArgs {
     unsigned* nroots; // their number
     int L;
     int ntx, nty, ntz;
+    FastDiv ntxd, ntyd;
     long long N, ntiles;
     uint32_t thr;     // a satisfied bond is active iff u <= thr
     int never;        // no bond can be active (beta = 0)
@@ -144,14 +147,12 @@ __device__ __forceinline__ void gunion(uint32_t* lab, uint32_t a, uint32_t b)
 }
 
 
+// origin and extents of tile (bx, by, bz)
 template <int D>
-__device__ __forceinline__ void tile_origin(const SwArgs& a, long long b, int& X0, int& Y0, int& Z0,
-                                            int& nx, int& ny, int& nz)
+__device__ __forceinline__ void tile_origin(const SwArgs& a, int bx, int by, int bz, int& X0, int& Y0,
+                                            int& Z0, int& nx, int& ny, int& nz)
 {
     constexpr int TX = SwTile<D>::TX, TY = SwTile<D>::TY, TZ = SwTile<D>::TZ;
-    const int bx = (int)(b % a.ntx);
-    const int by = (int)((b / a.ntx) % a.nty);
-    const int bz = (int)(b / ((long long)a.ntx * a.nty));
     X0 = bx * TX;
     Y0 = by * TY;
     Z0 = bz * TZ;
@@ -199,13 +200,241 @@ __device__ __forceinline__ bool bond_active(const SwArgs& a, uint8_t s0, uint8_t
     return (int)(s0 ^ s1) == a.anti && !a.never && u <= a.thr;
 }
 
-template <int D>
-__global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
+// 2D tiles of 64 x 32 sites.  A row of the tile is two words, the even and the
+// odd sites' spins by ballot, and its four bond uniforms per site pair become
+// four words of "drawn" bits by ballot, so bond activation, run heads, the choice
+// of the bonds to unite and the tile's face are a few word operations per row for
+// the whole warp.  (One lane deciding its own two sites' bonds byte by byte took
+// 340 instructions per warp for its two rows and 46 of 252 us at L = 4096 at the
+// critical point.)  Latency and issue bound: 256 threads and 8 blocks per
+// multiprocessor (32 registers) took 178 us there, 512 threads 221 (3 blocks) and
+// 193 (4 blocks), 128 threads 200, 1024 threads 245.
+__global__ void __launch_bounds__(kSwThreads2, 8) sw_local2(const SwArgs a)
 {
+    constexpr int TX = SwTile<2>::TX, TY = SwTile<2>::TY;
+    constexpr int NW = kSwThreads2 / 32, RPW = TY / NW;  // warps, rows per warp
+    constexpr uint32_t kAll = 0xFFFFFFFFu;
+    static_assert(TX == 64 && TY == 32, "words of a tile");
+    __shared__ __align__(8) uint32_t par[TX * TY];
+    __shared__ uint32_t rowE[TY + 1], rowO[TY + 1];  // spins, with the row after the tile
+    __shared__ uint32_t bx0[TY], bx1[TY];            // active x bonds of even and odd sites
+    __shared__ uint32_t fx;                          // bonds over the +x face
+    __shared__ uint16_t list[NW][RPW * TX];
+    __shared__ unsigned blk_count, blk_base;
+
+    int X0, Y0, Z0, nx, ny, nz;
+    // (one block per tile on a grid of the tiles' shape: recovering the tile from a
+    // linear index took three 64-bit divisions, some 250 instructions a thread)
+    tile_origin<2>(a, blockIdx.x, blockIdx.y, 0, X0, Y0, Z0, nx, ny, nz);
+    const size_t tile = blockIdx.x + (size_t)gridDim.x * blockIdx.y;
+    const uint32_t L = (uint32_t)a.L;
+    const uint32_t t = (uint32_t)a.ctrl->t;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lx0 = 2 * lane, last = (nx >> 1) - 1;  // the lane's pair; lane of the last pair
+    const uint32_t valid = kAll >> (31 - last), below = (1u << lane) - 1u;
+    const bool ex = lane <= last;
+    if (threadIdx.x == 0) {
+        fx = 0u;
+        blk_count = 0;
+    }
+
+    // spins of row ly of the tile (up to ny, the row after it)
+    auto load_row = [&](int ly) {
+        const uint32_t y = (uint32_t)(Y0 + ly) == L ? 0u : (uint32_t)(Y0 + ly);
+        const int ce = (int)(y & 1u);  // colour of the even-x sites
+        const uint32_t j = (L * y + (uint32_t)(X0 + lx0)) >> 1;
+        const int8_t ve = ex ? a.s[ce][j] : (int8_t)0, vo = ex ? a.s[ce ^ 1][j] : (int8_t)0;
+        const uint32_t E = __ballot_sync(kAll, ve != 0), O = __ballot_sync(kAll, vo != 0);
+        if (lane == 0) {
+            rowE[ly] = E;
+            rowO[ly] = O;
+        }
+    };
+    uint32_t hx = 0u;  // bit k: the spin after the last of the warp's row k
+#pragma unroll
+    for (int k = 0; k < RPW; ++k) {
+        const int ly = warp + NW * k;
+        if (ly >= ny) continue;  // uniform across the warp
+        load_row(ly);
+        const uint32_t y = (uint32_t)(Y0 + ly), x = (uint32_t)(X0 + nx) == L ? 0u : (uint32_t)(X0 + nx);
+        hx |= (uint32_t)a.s[(x + y) & 1u][(L * y + x) >> 1] << k;
+    }
+    if (warp == NW - 1) load_row(ny);
+    // drawn bits of the x and y bonds of the even and odd sites (the draws have no
+    // branch between them; rows outside a ragged tile draw bits nobody reads)
+    uint32_t ax0[RPW], ax1[RPW], ay0[RPW], ay1[RPW];
+    {
+        const PhiloxGroups pg = philox_groups(t, a.replica, kSwBond << 1, a.rk);
+        uint4 rnd[RPW];
+#pragma unroll
+        for (int k = 0; k < RPW; ++k)
+            rnd[k] = philox_at(pg, ((uint32_t)(X0 + lx0) + L * (uint32_t)(Y0 + warp + NW * k)) >> 1,
+                               a.rk);
+        const uint32_t may = a.never ? 0u : valid;
+#pragma unroll
+        for (int k = 0; k < RPW; ++k) {
+            ax0[k] = __ballot_sync(kAll, rnd[k].x <= a.thr) & may;
+            ay0[k] = __ballot_sync(kAll, rnd[k].y <= a.thr) & may;
+            ax1[k] = __ballot_sync(kAll, rnd[k].z <= a.thr) & may;
+            ay1[k] = __ballot_sync(kAll, rnd[k].w <= a.thr) & may;
+        }
+    }
+    __syncthreads();
+
+    // Active bonds, and every site's parent: the first site of its x-run.
+    const uint32_t flipw = a.anti ? 0u : kAll;  // like spins satisfy a bond, or unlike ones
+#pragma unroll
+    for (int k = 0; k < RPW; ++k) {
+        const int ly = warp + NW * k;
+        if (ly >= ny) {
+            ay0[k] = ay1[k] = ax0[k] = ax1[k] = 0u;
+            continue;
+        }
+        const uint32_t E = rowE[ly], O = rowO[ly];
+        ax0[k] &= E ^ O ^ flipw;
+        ax1[k] &= O ^ ((E >> 1) | ((hx >> k & 1u) << last)) ^ flipw;
+        ay0[k] &= E ^ rowE[ly + 1] ^ flipw;
+        ay1[k] &= O ^ rowO[ly + 1] ^ flipw;
+        if (lane == 0 && (ax1[k] >> last & 1u)) atomicOr(&fx, 1u << ly);
+        ax1[k] &= ~(1u << last);
+        if (ly + 1 == ny) {  // the +y face
+            uint32_t* f = a.face + tile * SwFace<2>::WORDS;
+            if (lane < 2) f[1 + lane] = lane ? ay1[k] : ay0[k];
+            ay0[k] = ay1[k] = 0u;
+        }
+        if (lane == 0) {
+            bx0[ly] = ax0[k];
+            bx1[ly] = ax1[k];
+        }
+        // run starts: the even site unless the bond from the previous lane's odd
+        // site is active, the odd site unless the pair's bond is
+        const uint32_t R0 = ~(ax1[k] << 1), R1 = ~ax0[k];
+        int rs0 = 2 * (31 - __clz(R0 & ((2u << lane) - 1u)));
+        const uint32_t m1 = R1 & below;
+        if (m1) rs0 = max(rs0, 2 * (31 - __clz(m1)) + 1);
+        const int rs1 = (ax0[k] >> lane & 1u) ? rs0 : lx0 + 1;
+        *reinterpret_cast<uint2*>(&par[TX * ly + lx0]) =
+            make_uint2((uint32_t)(TX * ly + rs0), (uint32_t)(TX * ly + rs1));
+    }
+    __syncthreads();
+
+    // place the sites of two masks (even, odd) of row ly in the warp's list
+    auto put = [&](uint32_t m0, uint32_t m1, int ly, unsigned& n) {
+        const unsigned n0 = __popc(m0);
+        if (m0 >> lane & 1u) list[warp][n + __popc(m0 & below)] = (uint16_t)(TX * ly + lx0);
+        if (m1 >> lane & 1u) list[warp][n + n0 + __popc(m1 & below)] = (uint16_t)(TX * ly + lx0 + 1);
+        n += n0 + __popc(m1);
+    };
+    // The runs are joined along y.  A bond is left out when the two runs are
+    // joined by a bond further left already: c0, c1 mark the even and odd sites
+    // whose left neighbour is joined to its lower one, in both rows to the site.
+    unsigned n = 0;
+#pragma unroll
+    for (int k = 0; k < RPW; ++k) {
+        const int ly = warp + NW * k;
+        if (ly + 1 >= ny) continue;
+        const uint32_t r0 = ax0[k] & bx0[ly + 1], r1 = (ax1[k] & bx1[ly + 1]) << 1;
+        uint32_t c0 = 0u, c1 = 0u;
+#pragma unroll
+        for (int it = 0; it < 3; ++it) {
+            c1 = (ay0[k] | c0) & r0;
+            c0 = (ay1[k] | c1) << 1 & r1;
+        }
+        put(ay0[k] & ~c0, ay1[k] & ~c1, ly, n);
+    }
+    __syncwarp();
+    // One union per remaining bond, lock-free, the bonds dealt out evenly over the
+    // warp: find both roots (path halving) and link the larger below the smaller by
+    // an atomic minimum; if another link got there first, what it linked to is
+    // still to be joined to the smaller root.  Parents only ever point to smaller
+    // indices, so the root of every tile cluster ends as its smallest site whatever
+    // order the unions run in.  (Measured for the whole kernel up to here at L =
+    // 4096, critical point: compare-and-swap with both finds repeated 171 us,
+    // atomic minimum 163, Rem's interleaved splicing 161 but dearer jumps after it;
+    // finds without halving 1.4 times the whole kernel.)
+    volatile uint32_t* vp = par;
+    for (unsigned q = lane; q < n; q += 32) {
+        const uint32_t u = list[warp][q];
+        uint32_t ra = sfind(vp, u), rb = sfind(vp, u + (uint32_t)TX);
+        while (ra != rb) {
+            const uint32_t hi = max(ra, rb), lo = min(ra, rb);
+            const uint32_t old = atomicMin(par + hi, lo);
+            if (old == hi) break;
+            ra = sfind(vp, old);
+            rb = lo;
+        }
+    }
+    // the run heads, listed in the same place, jump to their roots; every other
+    // site's label is read through its head
+    __syncwarp();
+    unsigned nh = 0;
+#pragma unroll
+    for (int k = 0; k < RPW; ++k) {
+        const int ly = warp + NW * k;
+        if (ly < ny) put(~(ax1[k] << 1) & valid, ~ax0[k] & valid, ly, nh);
+    }
+    __syncthreads();
+    for (unsigned q = lane; q < nh; q += 32) {
+        const uint32_t l = list[warp][q];
+        uint32_t p = vp[l];
+        while (true) {
+            const uint32_t g = vp[p];
+            if (g == p) break;
+            p = g;
+        }
+        vp[l] = p;
+    }
+    __syncthreads();
+
+    // labels: the natural index of each site's tile root; tile roots are marked
+    // and appended to the update's list (one global atomic per block)
+    const uint32_t i00 = (uint32_t)X0 + L * (uint32_t)Y0;
+    uint32_t m0[RPW], m1[RPW];  // tile roots among the even and odd sites
+    unsigned cnt = 0;
+#pragma unroll
+    for (int k = 0; k < RPW; ++k) {
+        const int ly = warp + NW * k;
+        m0[k] = m1[k] = 0u;
+        if (ly >= ny) continue;
+        const uint32_t l = (uint32_t)(TX * ly + lx0);
+        const uint2 h = ex ? *reinterpret_cast<const uint2*>(&par[l]) : make_uint2(l, l);
+        const uint32_t ra = par[h.x], rb = par[h.y];
+        const bool root0 = ex && ra == l, root1 = ex && rb == l + 1;
+        m0[k] = __ballot_sync(kAll, root0);
+        m1[k] = __ballot_sync(kAll, root1);
+        cnt += __popc(m0[k]) + __popc(m1[k]);
+        if (ex)
+            *reinterpret_cast<uint2*>(a.lab + i00 + L * (uint32_t)ly + lx0) =
+                make_uint2((i00 + (ra & 63u) + L * (ra >> 6)) | (root0 ? kTileRoot : 0u),
+                           (i00 + (rb & 63u) + L * (rb >> 6)) | (root1 ? kTileRoot : 0u));
+    }
+    unsigned pos = 0;
+    if (lane == 0) pos = atomicAdd(&blk_count, cnt);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        blk_base = atomicAdd(a.nroots, blk_count);
+        a.face[tile * SwFace<2>::WORDS] = fx;
+    }
+    __syncthreads();
+    pos = blk_base + __shfl_sync(kAll, pos, 0);
+#pragma unroll
+    for (int k = 0; k < RPW; ++k) {
+        const uint32_t i = i00 + L * (uint32_t)(warp + NW * k) + lx0;
+        if (m0[k] >> lane & 1u) a.roots[pos + __popc(m0[k] & below)] = i;
+        pos += __popc(m0[k]);
+        if (m1[k] >> lane & 1u) a.roots[pos + __popc(m1[k] & below)] = i + 1;
+        pos += __popc(m1[k]);
+    }
+}
+
+// 3D tiles of 64 x 16 x 8 sites.
+__global__ void __launch_bounds__(kSwThreads, 3) sw_local3(const SwArgs a)
+{
+    constexpr int D = 3;
     constexpr int TX = SwTile<D>::TX, TY = SwTile<D>::TY, TZ = SwTile<D>::TZ;
     static_assert(TX == 64, "one warp lane per site pair of a 64-site row");
     constexpr int NS = TX * TY * TZ;
-    constexpr int HX = TX + 2, HY = TY + 1, HZ = D == 3 ? TZ + 1 : 1;  // halo-padded spin tile
+    constexpr int HX = TX + 2, HY = TY + 1, HZ = TZ + 1;  // halo-padded spin tile
     constexpr int WORDS = SwFace<D>::WORDS;
     constexpr int NW = kSwThreads / 32;
     constexpr int ROWS = TY * TZ;
@@ -215,11 +444,11 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
     __shared__ uint32_t fm[WORDS];
     // per row, per lane bit: active in-tile bonds of the lane's even (0) and
     // odd (1) site along +x, +y and +z
-    __shared__ uint32_t bx[2][ROWS], by[2][ROWS], bz[2][D == 3 ? ROWS : 1];
+    __shared__ uint32_t bx[2][ROWS], by[2][ROWS], bz[2][ROWS];
 
-    const long long b = blockIdx.x;
+    const size_t b = blockIdx.x + gridDim.x * (blockIdx.y + (size_t)gridDim.y * blockIdx.z);
     int X0, Y0, Z0, nx, ny, nz;
-    tile_origin<D>(a, b, X0, Y0, Z0, nx, ny, nz);
+    tile_origin<D>(a, blockIdx.x, blockIdx.y, blockIdx.z, X0, Y0, Z0, nx, ny, nz);
     const uint32_t L = (uint32_t)a.L;
     const uint32_t t = (uint32_t)a.ctrl->t;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -231,11 +460,11 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
     // the +x column
     for (int r = warp; r < HY * HZ; r += NW) {
         const int ly = r % HY, lz = r / HY;
-        if (ly > ny || (D == 3 && lz > nz)) continue;
-        const bool hy = ly == ny, hz = D == 3 && lz == nz;
+        if (ly > ny || lz > nz) continue;
+        const bool hy = ly == ny, hz = lz == nz;
         if (hy && hz) continue;
         const uint32_t y = (uint32_t)(Y0 + ly) == L ? 0u : (uint32_t)(Y0 + ly);
-        const uint32_t z = D == 3 ? ((uint32_t)(Z0 + lz) == L ? 0u : (uint32_t)(Z0 + lz)) : 0u;
+        const uint32_t z = (uint32_t)(Z0 + lz) == L ? 0u : (uint32_t)(Z0 + lz);
         const uint32_t rowbase = L * (y + L * z);
         const int ce = (int)((y + z) & 1u);  // colour of the even-x sites
         uint8_t* dst = sp + (lz * HY + ly) * HX;
@@ -247,18 +476,6 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
         if (lane == 0 && !hy && !hz) {
             const uint32_t x = (uint32_t)(X0 + nx) == L ? 0u : (uint32_t)(X0 + nx);
             dst[nx] = (uint8_t)a.s[(x + y + z) & 1u][(rowbase + x) >> 1];
-        }
-    }
-    // 2D: the bond uniforms of both of the warp's rows are drawn here, with
-    // no branch between them, while the spin loads are in flight (rows
-    // outside a ragged tile draw values nobody reads)
-    uint4 pre[D == 2 ? RPW : 1];
-    if (D == 2) {
-#pragma unroll
-        for (int k = 0; k < RPW; ++k) {
-            const int ly = (warp + NW * k) % TY;
-            const uint32_t i0 = (uint32_t)(X0 + lx0) + L * (uint32_t)(Y0 + ly);
-            pre[k] = philox4x32_10(make_uint4(i0 >> 1, t, a.replica, kSwBond << 1), a.rk);
         }
     }
     __syncthreads();
@@ -277,14 +494,8 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
         if (ex) {
             const uint32_t i0 = (uint32_t)(X0 + lx0) + L * ((uint32_t)(Y0 + ly) + L * (uint32_t)(Z0 + lz));
             // uniforms of the x / y / z bonds of the even (e = 0) and odd site
-            uint4 r0, r1;
-            if (D == 2) {
-                r0 = pre[D == 2 ? k : 0];
-                r1 = make_uint4(r0.z, r0.w, 0u, 0u);
-            } else {
-                r0 = philox4x32_10(make_uint4(i0, t, a.replica, kSwBond << 1), a.rk);
-                r1 = philox4x32_10(make_uint4(i0 + 1, t, a.replica, kSwBond << 1), a.rk);
-            }
+            const uint4 r0 = philox4x32_10(make_uint4(i0, t, a.replica, kSwBond << 1), a.rk);
+            const uint4 r1 = philox4x32_10(make_uint4(i0 + 1, t, a.replica, kSwBond << 1), a.rk);
             const uint8_t s0 = sp[so], s1 = sp[so + 1], s2 = sp[so + 2];
             xb0 = bond_active(a, s0, s1, r0.x);
             xb1 = bond_active(a, s1, s2, r1.x);
@@ -301,7 +512,7 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
                         yb[e] = true;
                     }
                 }
-                if (D == 3 && bond_active(a, own, sp[so + e + HX * HY], re.z)) {
+                if (bond_active(a, own, sp[so + e + HX * HY], re.z)) {
                     if (lz + 1 == nz) {
                         const int bit = TY * TZ + TX * TZ + lx + TX * ly;
                         atomicOr(&fm[bit >> 5], 1u << (bit & 31));
@@ -320,20 +531,15 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
         const uint32_t B1 = __ballot_sync(0xFFFFFFFFu, xb1 && !xcross);
         const uint32_t Y0b = __ballot_sync(0xFFFFFFFFu, yb[0]);
         const uint32_t Y1b = __ballot_sync(0xFFFFFFFFu, yb[1]);
-        uint32_t Z0b = 0u, Z1b = 0u;
-        if (D == 3) {
-            Z0b = __ballot_sync(0xFFFFFFFFu, zb[0]);
-            Z1b = __ballot_sync(0xFFFFFFFFu, zb[1]);
-        }
+        const uint32_t Z0b = __ballot_sync(0xFFFFFFFFu, zb[0]);
+        const uint32_t Z1b = __ballot_sync(0xFFFFFFFFu, zb[1]);
         if (lane == 0) {
             bx[0][row] = B0;
             bx[1][row] = B1;
             by[0][row] = Y0b;
             by[1][row] = Y1b;
-            if (D == 3) {
-                bz[0][D == 3 ? row : 0] = Z0b;
-                bz[1][D == 3 ? row : 0] = Z1b;
-            }
+            bz[0][row] = Z0b;
+            bz[1][row] = Z1b;
         }
         if (ex) {
             // run starts: the even site starts a run unless the bond from the
@@ -364,8 +570,8 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
 #pragma unroll
             for (int mu = 1; mu < D; ++mu) {
                 const int nrow = mu == 1 ? row + 1 : row + TY;
-                const uint32_t c0 = mu == 1 ? by[0][row] : bz[0][D == 3 ? row : 0];
-                const uint32_t c1 = mu == 1 ? by[1][row] : bz[1][D == 3 ? row : 0];
+                const uint32_t c0 = mu == 1 ? by[0][row] : bz[0][row];
+                const uint32_t c1 = mu == 1 ? by[1][row] : bz[1][row];
                 // even site 2k: its left neighbour is lane k-1's odd site
                 bool p0 = (c0 >> lane) & 1u;
                 if (p0 && lane > 0 && ((c1 >> (lane - 1)) & 1u) &&
@@ -384,51 +590,34 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
     }
     // Every parent is a run head (the first site of an x-run), so after the
     // heads have jumped to their roots a label is read through the head (two
-    // steps).  The warp lists the heads of its rows in shared memory (each
-    // lane places its own by a population count of the ballot below it) and
-    // deals the list out over its lanes for the jump; the heads are decided
-    // by the x-bond ballots.
-    // (3D, whose tile already fills most of the shared memory, keeps the
-    // heads in registers instead: lane l takes the l-th and (l + 32)-th
-    // head of each of its rows)
-    __shared__ uint16_t hlist[NW][D == 2 ? RPW * TX : 1];
-    unsigned nh = 0;                   // 2D: heads listed by the warp (warp-uniform)
-    uint32_t heads[D == 2 ? 1 : RPW];  // 3D: per row two 16-bit sites, 0xFFFF = none
+    // steps); the heads are decided by the x-bond ballots.  Lane l takes the l-th
+    // and (l + 32)-th head of each of its rows.
+    uint32_t heads[RPW];  // per row two 16-bit sites, 0xFFFF = none
     {
         const uint32_t valid = nx >= 64 ? 0xFFFFFFFFu : ((1u << (nx >> 1)) - 1u);
-        const uint32_t below = (1u << lane) - 1u;
 #pragma unroll
         for (int k = 0; k < RPW; ++k) {
-            if (D == 3) heads[D == 2 ? 0 : k] = 0xFFFFFFFFu;
+            heads[k] = 0xFFFFFFFFu;
             const int row = warp + NW * k;
             const int ly = row % TY, lz = row / TY;
             if (ly >= ny || lz >= nz) continue;
             const uint32_t h0 = ~(bx[1][row] << 1) & valid;  // even sites starting a run
             const uint32_t h1 = ~bx[0][row] & valid;         // odd sites starting a run
             const unsigned n0 = __popc(h0);
-            if (D == 2) {
-                if ((h0 >> lane) & 1u)
-                    hlist[warp][nh + __popc(h0 & below)] = (uint16_t)(TX * row + lx0);
-                if ((h1 >> lane) & 1u)
-                    hlist[warp][nh + n0 + __popc(h1 & below)] = (uint16_t)(TX * row + lx0 + 1);
-                nh += n0 + __popc(h1);
-            } else {
-                const int n = (int)n0 + __popc(h1);
-                uint32_t w = 0;
+            const int n = (int)n0 + __popc(h1);
+            uint32_t w = 0;
 #pragma unroll
-                for (int slot = 0; slot < 2; ++slot) {
-                    const int q = lane + 32 * slot;
-                    uint32_t site = 0xFFFFu;
-                    if (q < n)
-                        site = (uint32_t)(TX * row) +
-                               (q < (int)n0 ? 2u * (uint32_t)nth_set_bit(h0, q)
-                                            : 2u * (uint32_t)nth_set_bit(h1, q - (int)n0) + 1u);
-                    w |= site << (16 * slot);
-                }
-                heads[D == 2 ? 0 : k] = w;
+            for (int slot = 0; slot < 2; ++slot) {
+                const int q = lane + 32 * slot;
+                uint32_t site = 0xFFFFu;
+                if (q < n)
+                    site = (uint32_t)(TX * row) +
+                           (q < (int)n0 ? 2u * (uint32_t)nth_set_bit(h0, q)
+                                        : 2u * (uint32_t)nth_set_bit(h1, q - (int)n0) + 1u);
+                w |= site << (16 * slot);
             }
+            heads[k] = w;
         }
-        __syncwarp();
     }
     // One union per remaining y/z bond, lock-free: find both roots (path
     // halving), link the larger root below the smaller by compare-and-swap,
@@ -447,38 +636,13 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
             rb = sfind(vp, lo);
         }
     };
-    if (D == 2) {
-        // the warp's bonds are packed into a shared list (a scan of the lanes'
-        // counts places them) and dealt out evenly, so the warp runs as many
-        // union rounds as its mean load needs rather than its busiest lane's
-        __shared__ uint16_t plist[NW][D == 2 ? 2 * RPW * 32 : 1];
-        const unsigned cnt = __popc(pend);
-        unsigned incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned x = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += x;
-        }
-        const unsigned total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-        unsigned pos = incl - cnt;
-        for (uint32_t bits = pend; bits; bits &= bits - 1) {
-            const int bit = __ffs(bits) - 1;  // bit 2k + e: row k, site e
-            plist[warp][pos++] = (uint16_t)(lx0 + (bit & 1) + TX * (warp + NW * (bit >> 1)));
-        }
-        __syncwarp();
-        for (unsigned q = lane; q < total; q += 32) {
-            const uint32_t u = plist[warp][q];
-            unite(u, u + (uint32_t)TX);
-        }
-    } else {
-        for (uint32_t bits = pend; bits; bits &= bits - 1) {
-            const int bit = __ffs(bits) - 1;
-            const int k = bit / (2 * (D - 1));
-            const int e = (bit / (D - 1)) & 1;
-            const int mu = 1 + bit % (D - 1);
-            const uint32_t u = (uint32_t)(lx0 + e + TX * (warp + NW * k));
-            unite(u, u + (mu == 1 ? (uint32_t)TX : (uint32_t)(TX * TY)));
-        }
+    for (uint32_t bits = pend; bits; bits &= bits - 1) {
+        const int bit = __ffs(bits) - 1;
+        const int k = bit / (2 * (D - 1));
+        const int e = (bit / (D - 1)) & 1;
+        const int mu = 1 + bit % (D - 1);
+        const uint32_t u = (uint32_t)(lx0 + e + TX * (warp + NW * k));
+        unite(u, u + (mu == 1 ? (uint32_t)TX : (uint32_t)(TX * TY)));
     }
     __syncthreads();
     auto jump = [&](uint32_t l) {
@@ -490,17 +654,13 @@ __global__ void __launch_bounds__(kSwThreads, 3) sw_local(const SwArgs a)
         }
         vp[l] = p;
     };
-    if (D == 2) {
-        for (unsigned q = lane; q < nh; q += 32) jump(hlist[warp][q]);
-    } else {
 #pragma unroll
-        for (int k = 0; k < RPW; ++k)
+    for (int k = 0; k < RPW; ++k)
 #pragma unroll
-            for (int slot = 0; slot < 2; ++slot) {
-                const uint32_t l = (heads[D == 2 ? 0 : k] >> (16 * slot)) & 0xFFFFu;
-                if (l != 0xFFFFu) jump(l);
-            }
-    }
+        for (int slot = 0; slot < 2; ++slot) {
+            const uint32_t l = (heads[k] >> (16 * slot)) & 0xFFFFu;
+            if (l != 0xFFFFu) jump(l);
+        }
     __syncthreads();
 
     // labels: the natural index of each site's tile root; tile roots marked
@@ -564,16 +724,20 @@ __global__ void __launch_bounds__(256) sw_merge(const SwArgs a)
 {
     constexpr int TX = SwTile<D>::TX, TY = SwTile<D>::TY, TZ = SwTile<D>::TZ;
     constexpr int WORDS = SwFace<D>::WORDS;
-    const long long total = a.ntiles * WORDS * 32;
+    // (N <= 2^30 keeps the number of face bits below 2^31)
+    const uint32_t total = (uint32_t)(a.ntiles * WORDS * 32);
     const int L = a.L;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long b = q / (WORDS * 32);
+    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < total;
+         q += gridDim.x * blockDim.x) {
+        const uint32_t b = q / (WORDS * 32);
         const int bit = (int)(q % (WORDS * 32));
-        const uint32_t word = __ldg(a.face + b * WORDS + (bit >> 5));
+        const uint32_t word = __ldg(a.face + (size_t)b * WORDS + (bit >> 5));
         if (!((word >> (bit & 31)) & 1u)) continue;
+        const uint32_t brow = a.ntxd.div(b);
+        const uint32_t bz = D == 3 ? a.ntyd.div(brow) : 0u;
         int X0, Y0, Z0, nx, ny, nz;
-        tile_origin<D>(a, b, X0, Y0, Z0, nx, ny, nz);
+        tile_origin<D>(a, (int)(b - brow * a.ntxd.d),
+                       (int)(D == 3 ? brow - bz * a.ntyd.d : brow), (int)bz, X0, Y0, Z0, nx, ny, nz);
         int lx, ly, lz, mu;
         if (bit < TY * TZ) {
             mu = 0;
@@ -582,10 +746,11 @@ __global__ void __launch_bounds__(256) sw_merge(const SwArgs a)
             lz = bit / TY;
         } else if (bit < TY * TZ + TX * TZ) {
             mu = 1;
+            // (2D: the even sites' word, then the odd sites')
             const int k = bit - TY * TZ;
-            lx = k % TX;
+            lx = D == 2 ? 2 * (k & 31) + (k >> 5) : k % TX;
             ly = ny - 1;
-            lz = k / TX;
+            lz = D == 2 ? 0 : k / TX;
         } else {
             mu = 2;
             const int k = bit - TY * TZ - TX * TZ;
@@ -839,7 +1004,9 @@ cudaError_t sw_update(const SwArgs& a0, cudaStream_t s)
     const long long mergers = a.ntiles * SwFace<D>::WORDS * 32;
     cudaError_t e = cudaMemsetAsync(a.nroots, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
-    sw_local<D><<<(unsigned)a.ntiles, kSwThreads, 0, s>>>(a);
+    const dim3 tiles((unsigned)a.ntx, (unsigned)a.nty, (unsigned)a.ntz);
+    if (D == 2) sw_local2<<<tiles, kSwThreads2, 0, s>>>(a);
+    else sw_local3<<<tiles, kSwThreads, 0, s>>>(a);
     sw_merge<D><<<grid_for(mergers, 256), 256, 0, s>>>(a);
     sw_resolve<<<grid_for(a.N, 256), 256, 0, s>>>(a);
     sw_flip<<<grid_for((a.N / 2 + 3) / 4, 256), 256, 0, s>>>(a);  // at most one block per row used
@@ -879,6 +1046,8 @@ cudaError_t ising_sw_sweeps(const sl_lattice* h, const SweepParams& p, int64_t c
     a.N = h->N;
     a.ntiles = h->d == 2 ? tiles_of<2>(h->L, a.ntx, a.nty, a.ntz)
                          : tiles_of<3>(h->L, a.ntx, a.nty, a.ntz);
+    a.ntxd = make_fast_div((uint32_t)a.ntx);
+    a.ntyd = make_fast_div((uint32_t)a.nty);
     a.thr = p.tab.sw_thr;
     a.never = p.tab.sw_never;
     a.anti = h->J < 0.0;
