@@ -274,16 +274,19 @@ void check_graph_key(sl_lattice* h, const SweepParams& p)
     std::memcpy(h->graph_key, key, sizeof key);
 }
 
-int sync_and_check(sl_lattice* h)
+// Wait for the stream and check the error word; the control block comes back in
+// the same trip (one copy of 88 bytes in place of a synchronisation and a copy
+// each for the error word and the observables, some 10 us apiece).
+int sync_and_check(sl_lattice* h, Ctrl* out = nullptr)
 {
-    cudaError_t e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-    unsigned err = 0;
-    e = cudaMemcpy(&err, &h->ctrl->error, sizeof err, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "read error word");
-    if (err & 1u)
-        return fail(SL_ETIMEOUT, "a kernel's bounded wait for its staged copies ran out; the "
+    Ctrl c;
+    cudaError_t e = cudaMemcpyAsync(&c, h->ctrl, sizeof c, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "wait for the stream");
+    if (c.error & 1u)
+        return fail(SL_ETIMEOUT, "a kernel's bounded wait ran out; the "
                                  "configuration is not valid");
+    if (out) *out = c;
     return SL_OK;
 }
 
@@ -622,11 +625,10 @@ int sl_measure(sl_lattice* h, double* energy, double* magnetisation)
     else if (h->storage == SL_STORE_BITS) e = ising_bits_measure(h, h->stream);
     else if (h->n > 1) e = on_measure(h, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "measure launch");
-    int st = sync_and_check(h);
+    Ctrl c;
+    const int st = sync_and_check(h, &c);
     if (st != SL_OK) return st;
-    double obs[4];
-    e = cudaMemcpy(obs, h->ctrl->obs, sizeof obs, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "read observables");
+    const double* obs = c.obs;
     if (energy) *energy = obs[0];
     if (magnetisation) {
         double m2 = 0.0;
