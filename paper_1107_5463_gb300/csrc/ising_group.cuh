@@ -34,7 +34,8 @@ struct GroupGeo {
 //   an aligned word): the entry beside the group that the row's parity calls
 //   for in each colour's pass, the byte selector that shifts it in, and the
 //   offsets of the rows y -/+ 1;
-//   otherwise the column k, row y and parity p of its first site.
+//   otherwise the column k, row y and parity p of its first site (2D: y is not
+//   used).
 struct GroupPos {
     int l;
     int edge[2];
@@ -69,46 +70,113 @@ __device__ __forceinline__ GroupPos group_at(int l, const GroupGeo& e, const Fas
     return g;
 }
 
+// The four bytes at o + a (a of any alignment and sign): two words and a shift.
+// Reads up to 3 bytes before them and 7 after.
+__device__ __forceinline__ uint32_t read4(const uint8_t* o, int a)
+{
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(o + (a & ~3));
+    return __funnelshift_r(w[0], w[1], 8 * (a & 3));
+}
+
+// the low n bytes (0 <= n <= 4)
+__device__ __forceinline__ uint32_t low_bytes(int n)
+{
+    return n <= 0 ? 0u : 0xFFFFFFFFu >> (32 - 8 * n);
+}
+
+// w with byte b replaced by v
+__device__ __forceinline__ uint32_t put_byte(uint32_t w, int b, uint32_t v)
+{
+    return (w & ~(0xFFu << (8 * b))) | v << (8 * b);
+}
+
 // The other colour's bytes beside the group's four sites in the pass of colour
 // c, one word per direction: [0] the x neighbour with the site's own column
 // (the word at l), [1] the other x neighbour, then -y, +y (3D only), then the
-// slowest axis -, +).  slow(l, up) reads a word (ALIGNED) or a byte of the plane
-// before (up = false) or after the one that holds entry l.
-template <int D, bool ALIGNED, typename Slow>
+// slowest axis -, +.  slow(l, up) gives the word of the plane before (up =
+// false) or after the one that holds entry l.  SLACK: 16 bytes before and after
+// the array may be read (shared memory), so short rows are put together without
+// branches.
+template <int D, bool ALIGNED, bool SLACK, typename Slow>
 __device__ __forceinline__ void group_neighbours(const uint8_t* o, const GroupPos& g,
                                                  const GroupGeo& e, int c, uint32_t (&nw)[2 * D],
                                                  Slow slow)
 {
     const int l = g.l;
-    const uint32_t cur = *reinterpret_cast<const uint32_t*>(o + l);
+    const uint32_t* ow = reinterpret_cast<const uint32_t*>(o + l);
+    const uint32_t cur = ow[0];
     nw[0] = cur;
+    nw[2 * D - 2] = slow(l, false);
+    nw[2 * D - 1] = slow(l, true);
     if (ALIGNED) {
         nw[1] = __byte_perm(cur, (uint32_t)o[c ? g.edge[1] : g.edge[0]], c ? g.sel[1] : g.sel[0]);
         if (D == 3) {
             nw[2] = *reinterpret_cast<const uint32_t*>(o + g.ym);
             nw[3] = *reinterpret_cast<const uint32_t*>(o + g.yp);
         }
-        nw[2 * D - 2] = slow(l, false);
-        nw[2 * D - 1] = slow(l, true);
+    } else if (e.W >= (SLACK ? 8 : 4)) {
+        // the group holds n1 sites of one row and 4 - n1 of the next
+        const int p = g.p ^ c, n1 = min(4, e.W - g.k);
+        const bool two = n1 < 4, plane = D == 3 && g.y == e.L - 1;  // next row in the next plane
+        const int p2 = plane ? p : p ^ 1;
+        const uint32_t m1 = low_bytes(n1);
+        const uint32_t before = __funnelshift_l(l > 0 ? ow[-1] : 0u, cur, 8);
+        const uint32_t after = __funnelshift_r(cur, ow[1], 8);
+        uint32_t x = ((p ? after : before) & m1) | ((p2 ? after : before) & ~m1);
+        // the bytes that come from the other end of a row: rare on long rows, where
+        // most warps skip them, a chain of divergent branches on short ones
+        auto edge = [&](bool cond, int b, int i) {
+            if (SLACK && e.W < 64) {
+                const uint32_t y = put_byte(x, b, o[cond ? i : l]);
+                x = cond ? y : x;
+            } else if (cond) {
+                x = put_byte(x, b, o[i]);
+            }
+        };
+        edge(!p && g.k == 0, 0, l + e.W - 1);
+        edge(p && g.k + n1 == e.W, n1 - 1, l + n1 - e.W);
+        edge(two && !p2, n1 & 3, l + n1 + e.W - 1);
+        nw[1] = x;
+        if (D == 3) {
+            const int wrap = (e.L - 1) * e.W;
+            uint32_t ym = read4(o, g.y == 0 ? l + wrap : l - e.W);
+            uint32_t yp = read4(o, plane ? l - wrap : l + e.W);
+            // the second row's neighbours where they wrap differently from the first's
+            auto second = [&](uint32_t w, int off) {
+                if (SLACK) return (w & m1) | (read4(o, l + off) & ~m1);
+                for (int b = n1; b < 4; ++b) w = put_byte(w, b, o[l + b + off]);
+                return w;
+            };
+            if (two && plane) {  // row L - 1, then row 0
+                ym = second(ym, wrap);
+                yp = second(yp, e.W);
+            } else if (two && g.y == 0) {
+                ym = second(ym, -e.W);
+            } else if (two && g.y == e.L - 2) {
+                yp = second(yp, -wrap);
+            }
+            nw[2] = ym;
+            nw[3] = yp;
+        }
     } else {
-        // the group may run over a row end: every site finds its own neighbours
+        // rows shorter than a group (in shared memory also rows hardly longer): every
+        // site finds its own neighbours
         int k = g.k, y = g.y, p = g.p ^ c;
 #pragma unroll
-        for (int q = 1; q < 2 * D; ++q) nw[q] = 0u;
+        for (int q = 1; q < 2 * D - 2; ++q) nw[q] = 0u;
+        uint32_t x = 0u;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
             const int lb = l + b;
             const int xo = p ? (k + 1 == e.W ? lb + 1 - e.W : lb + 1)
                              : (k == 0 ? lb + e.W - 1 : lb - 1);
-            nw[1] |= (uint32_t)o[xo] << (8 * b);
+            x |= (uint32_t)o[xo] << (8 * b);
             if (D == 3) {
                 const int ym = y == 0 ? lb + (e.L - 1) * e.W : lb - e.W;
                 const int yp = y == e.L - 1 ? lb - (e.L - 1) * e.W : lb + e.W;
                 nw[2] |= (uint32_t)o[ym] << (8 * b);
                 nw[3] |= (uint32_t)o[yp] << (8 * b);
             }
-            nw[2 * D - 2] |= slow(lb, false) << (8 * b);
-            nw[2 * D - 1] |= slow(lb, true) << (8 * b);
             if (++k == e.W) {  // next row; a new plane keeps the alternation (L is even)
                 k = 0;
                 if (D == 2) {
@@ -120,6 +188,7 @@ __device__ __forceinline__ void group_neighbours(const uint8_t* o, const GroupPo
                 }
             }
         }
+        nw[1] = x;
     }
 }
 
@@ -177,10 +246,12 @@ __device__ __forceinline__ uint32_t group_update(uint32_t av, const uint32_t (&n
                                                  const uint32_t* s_hb, uint32_t valid,
                                                  GroupCounts& m)
 {
-    const uint32_t nd = neighbour_sum<D>(nw);
+    uint32_t nd = neighbour_sum<D>(nw);
     uint32_t na, flip, an;
     if (HB) {
-        // h = 2d - 2 nd; the new spin is down iff u > hb[h + 2d]
+        // h = 2d - 2 nd; the new spin is down iff u > hb[h + 2d].  (Bytes past the
+        // lattice's end hold anything, and they index the table: cleared.)
+        nd &= valid * 0xFFu;
         const uint32_t u[4] = {rnd.x, rnd.y, rnd.z, rnd.w};
         flip = 0u;
 #pragma unroll

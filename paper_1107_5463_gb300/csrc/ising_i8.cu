@@ -203,13 +203,24 @@ __global__ void __launch_bounds__(256) i8_flat(const I8Args a, const FastDiv Wd,
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < ngroups; q += gridDim.x * blockDim.x) {
         const GroupPos g = group_at<D, ALIGNED>(4 * q, e, Wd, Ld, a.c);
         uint32_t nw[2 * D];
-        group_neighbours<D, ALIGNED>(o, g, e, 0, nw, [&](int l, bool up) {
+        group_neighbours<D, ALIGNED, false>(o, g, e, 0, nw, [&](int l, bool up) {
             int z = up ? l + e.P : l - e.P;
-            if (z < 0) z += e.H;
-            if (z >= e.H) z -= e.H;
-            // (entries past the lattice's last, whose results are masked, stay inside)
-            if (!ALIGNED && z >= e.H) z -= e.H;
-            return ALIGNED ? *reinterpret_cast<const uint32_t*>(o + z) : (uint32_t)o[z];
+            if (ALIGNED) {
+                if (z < 0) z += e.H;
+                if (z >= e.H) z -= e.H;
+                return *reinterpret_cast<const uint32_t*>(o + z);
+            }
+            if (z >= 0 && z + 4 <= e.H) return read4(o, z);
+            // the group meets the periodic boundary (entries past the lattice's last,
+            // whose results are masked, stay inside too)
+            uint32_t v = 0u;
+            for (int b = 0; b < 4; ++b) {
+                int zb = z + b;
+                if (zb < 0) zb += e.H;
+                while (zb >= e.H) zb -= e.H;
+                v |= (uint32_t)o[zb] << (8 * b);
+            }
+            return v;
         });
         const uint32_t cur = nw[0];
         const uint32_t av = *reinterpret_cast<const uint32_t*>(a.own + g.l);

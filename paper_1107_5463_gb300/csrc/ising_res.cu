@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kResThreads, 1) i8_resident(const ResArgs a)
     const int jlo = base == 0 ? H - P : base - P, jhi = base + nown == H ? 0 : base + nown;
     bool ok = true;  // no wait has run out
     PhiloxGroups pg = philox_groups((uint32_t)t0, a.replica, kSweep << 1, a.rk);
-    uint4 rnd0 = philox_at(pg, (uint32_t)(base >> 2) + tid, a.rk);
+    uint4 rnd0 = philox_at(pg, (uint32_t)(base + l0) >> 2, a.rk);
     GroupCounts m = {0u, 0u, 0u, 0u};
 
     // one group of a pass of colour C; edge: it holds sites of the first or last plane
@@ -199,16 +199,35 @@ __global__ void __launch_bounds__(kResThreads, 1) i8_resident(const ResArgs a)
         uint8_t* own = rsm + c * a.cstride + a.oown;
         const int l = g.l;
         uint32_t nw[2 * D];
-        group_neighbours<D, ALIGNED>(o, g, a.geo, c, nw, [&](int e, bool up) {
-            if (!ALIGNED && e >= nown) return 0u;  // past the end of the lattice: masked
-            if (MULTI && edge && (up ? e >= nown - P : e < P)) {
-                const int j = up ? jhi + e - (nown - P) : jlo + e;
-                uint32_t v;
-                if (!wait_word(a.s[1 - c] + (ALIGNED ? j : j & ~3), waited, v)) ok = false;
-                return ALIGNED ? v : v >> (8 * (j & 3)) & 1u;
-            }
+        group_neighbours<D, ALIGNED, true>(o, g, a.geo, c, nw, [&](int e, bool up) {
             const int z = up ? e + P : e - P;
-            return ALIGNED ? *reinterpret_cast<const uint32_t*>(o + z) : (uint32_t)o[z];
+            if (!MULTI || !edge || !(up ? e + 4 > nown - P : e < P))
+                return ALIGNED ? *reinterpret_cast<const uint32_t*>(o + z) : read4(o, z);
+            if (ALIGNED) {
+                uint32_t v;
+                if (!wait_word(a.s[1 - c] + (up ? jhi + e - (nown - P) : jlo + e), waited, v))
+                    ok = false;
+                return v;
+            }
+            // bytes b0 .. b1 - 1 of the group have their neighbours in the other
+            // block's plane, at entries j on: in one of its words or in two
+            const int b0 = up ? max(0, nown - P - e) : 0;
+            const int b1 = up ? min(4, nown - e) : min(4, P - e);
+            const int j = up ? jhi + e + b0 - (nown - P) : jlo + e;
+            const int8_t* w = a.s[1 - c] + (j & ~3);
+            const bool two = (j & 3) + b1 - b0 > 4;
+            uint32_t v0, v1 = waited;
+            unsigned it = 0;
+            do {
+                v0 = ld_word(w);
+                if (two) v1 = ld_word(w + 4);
+            } while (waited != 0u && ((v0 & 0xFEFEFEFEu) != waited || (v1 & 0xFEFEFEFEu) != waited) &&
+                     ++it < kResWaitLimit);
+            if (it == kResWaitLimit) ok = false;
+            const uint32_t far = __funnelshift_r(v0, v1, 8 * (j & 3)) & 0x01010101u;
+            if (b0 == 0 && b1 == 4) return far;
+            const uint32_t mask = low_bytes(b1) & ~low_bytes(b0);
+            return ((far << (8 * b0)) & mask) | (read4(o, z) & ~mask);
         });
         const uint32_t cur = nw[0];
         const uint32_t av = *reinterpret_cast<const uint32_t*>(own + l);
@@ -250,7 +269,7 @@ __global__ void __launch_bounds__(kResThreads, 1) i8_resident(const ResArgs a)
             update(C, s, group_at<D, ALIGNED>(l, a.geo, a.Wd, a.Ld, z0),
                    l < P || l + 4 > nown - P, philox_at(pg, (uint32_t)(base + l) >> 2, a.rk));
         pg = philox_groups((uint32_t)t0 + (uint32_t)s + c, a.replica, (kSweep << 1) | (1 - c), a.rk);
-        rnd0 = philox_at(pg, (uint32_t)(base >> 2) + tid, a.rk);
+        rnd0 = philox_at(pg, (uint32_t)(base + l0) >> 2, a.rk);
         if (c == 1) {
             const uint32_t v = __reduce_add_sync(0xFFFFFFFFu, unsatisfied_after<D>(m));
             const uint32_t down = __reduce_add_sync(0xFFFFFFFFu, m.down);
@@ -380,16 +399,16 @@ bool res_shape(const sl_lattice* h, ResShape* y)
     y->unit = P % 4 == 0 ? 1 : (P % 2 == 0 ? 2 : 4);
     y->nunits = (h->L + y->unit - 1) / y->unit;
     const int most = h->sms < kResMaxBlocks ? h->sms : kResMaxBlocks;
-    // one block, and one barrier between passes, up to 2^14 sites (RESULT);
-    // beyond, at least 256 groups of each colour per block
-    long long G = h->N <= 16384 ? 1 : (h->N + 2047) / 2048;
+    // One block, whose passes are a barrier apart, for small lattices; beyond,
+    // about 256 groups of each colour per block.
+    long long G = h->N <= (P % 4 == 0 ? 5000 : 10000) ? 1 : (h->N + 2047) / 2048;
     if (G > most) G = most;
     if (G > y->nunits) G = y->nunits;
     y->G = (int)G;
     const long long np = (long long)((y->nunits + G - 1) / G) * y->unit;
     const long long nown = np * P;
-    y->oown = G == 1 ? up16(P) : 0;
-    y->cstride = y->oown + up16(nown + P + 4);
+    y->oown = G == 1 ? up16(P) : 16;  // (a few bytes before the first entry may be read)
+    y->cstride = y->oown + up16(nown + P + 12);
     y->jstride = h->j_layout == SL_J_BONDS ? up16(nown) : 0;
     y->smem = 2 * (size_t)y->cstride + 4 * (size_t)h->d * y->jstride;
     const long long groups = (nown + 3) / 4;
