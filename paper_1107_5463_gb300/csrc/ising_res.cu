@@ -414,7 +414,22 @@ bool res_shape(const sl_lattice* h, ResShape* y)
     const long long groups = (nown + 3) / 4;
     y->threads = groups >= kResThreads ? kResThreads : (int)((groups + 31) / 32 * 32);
     // the static arrays take 8.3 KB of a block's 227 KB
-    return y->smem <= 216 * 1024;
+    if (y->smem > 216 * 1024) return false;
+    if (G == 1) return true;
+    // Several blocks finish with the one that owns most sites; the kernels in
+    // global memory spread evenly but pay launches.  Microseconds a sweep, fitted to
+    // both sides measured at L = 50 to 5120 (2D L = 2048: 6.3 against 10.4 streaming,
+    // 4096: 22.0 and 22.5, 5120: 34.2 and 33.3; 3D L = 128: 6.2 and 7.8, 160: 15.0
+    // and 11.9; ragged 2D L = 1002: 3.1 and 6.5 flat; 3D L = 102: 10.9 and 8.4).
+    const bool al = h->W % 4 == 0, d3 = h->d == 3;
+    const double own = 2.0 * (double)nown;
+    const double site = d3 ? (al ? (np == 1 ? 0.37e-3 : 0.29e-3) : (np == 1 ? 0.95e-3 : 0.43e-3))
+                           : (al ? 0.20e-3 : 0.27e-3);
+    const bool bonds = h->j_layout == SL_J_BONDS;
+    const double other = h->W % 16 == 0 ? (d3 ? 1.4e-6 : 1.05e-6)           // i8_stream
+                         : bonds        ? 9.0e-6                             // i8_generic
+                                        : (d3 ? (al ? 1.9e-6 : 2.5e-6) : (al ? 1.4e-6 : 1.85e-6));
+    return 1.2 + own * site < 4.6 + (double)h->N * other;
 }
 
 }  // namespace

@@ -278,7 +278,7 @@ __device__ __forceinline__ V3 heis_heatbath(float hx, float hy, float hz, float 
 // tau = 1 + sqrt(1 + 4 kappa^2), the half-angle factor g = (1 - rho) / (1 + rho)
 // and the numerator of the test quantity, (tau + sqrt(2 tau)) (1 - rho^2)^2 / 4.
 struct VonMises {
-    float rho, g, cnum, base;  // base: angle of h in turns
+    float rho, g, cnum, arg;  // arg: angle of h in radians
 };
 
 __device__ __forceinline__ VonMises von_mises_setup(float hx, float hy, float beta)
@@ -291,7 +291,7 @@ __device__ __forceinline__ VonMises von_mises_setup(float hx, float hy, float be
     m.g = (1.f - m.rho) / (1.f + m.rho);
     const float q = 1.f - m.rho * m.rho;
     m.cnum = 0.25f * (tau + s2) * q * q;
-    m.base = atan2f(hy, hx) * (1.0f / kTwoPiF);
+    m.arg = atan2f(hy, hx);
     return m;
 }
 
@@ -302,21 +302,26 @@ __device__ __forceinline__ bool von_mises_accept(const VonMises& m, uint32_t o1,
     float sw, cw;
     sincos_turns(0.25f * u24(o1), &sw, &cw);
     const float omr = 1.f - m.rho;
-    const float cc = m.cnum / (omr * omr + 4.f * m.rho * cw * cw);
+    // (the roundings spelled out: a compiler that fuses the other product flips a
+    // decision in some 10^7)
+    const float cc = m.cnum / __fmaf_rn(__fmul_rn(__fmul_rn(4.f, m.rho), cw), cw,
+                                        __fmul_rn(omr, omr));
     const float U2 = u24(o2);
     return cc * (2.f - cc) > U2 || logf(cc / U2) + 1.f - cc >= 0.f;
 }
 
 // The new angle, in turns in [0, 1), of the accepted attempt with output o1:
 // the angle of h plus or minus (bit 0 of o1) delta, tan(delta/2) = g tan w.
-// Kept out of the attempt loop so that a warp pays for it once.
+// Kept out of the attempt loop so that a warp pays for it once.  (The angle of h is
+// turned into turns inside the addition, one rounding; spelled out, as a chain
+// depends on it in its last bits.)
 __device__ __forceinline__ float von_mises_angle(const VonMises& m, uint32_t o1)
 {
     float sw, cw;
     sincos_turns(0.25f * u24(o1), &sw, &cw);
-    float dt = atan2f(m.g * sw, cw) * (1.0f / kPiF);
+    float dt = __fmul_rn(atan2f(m.g * sw, cw), 1.0f / kPiF);
     if (o1 & 1u) dt = -dt;
-    float tn = m.base + dt;
+    float tn = __fmaf_rn(m.arg, 1.0f / kTwoPiF, dt);
     tn -= floorf(tn);
     return tn < 1.f ? tn : 0.f;
 }
@@ -1152,12 +1157,12 @@ __global__ void __launch_bounds__(kTileThreads, 3) heis_tile3(const OnArgs a)
 
 // XY, 2D: each thread owns the column pair (2q, 2q+1), whose sites share one
 // Philox block (group j >> 1).
-template <bool FAST, bool HB, bool MEAS>
+template <bool FAST, bool MEAS>
 __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
 {
     __shared__ double red[32];  // 4 per warp
     // Metropolis with accurate functions: sin and cos from the shared table
-    constexpr bool TAB = !FAST && !HB;
+    constexpr bool TAB = !FAST;
     __shared__ float2 tab[TAB ? kTurnTab : 1];
     if (TAB) fill_turn_table(tab);
     auto sc = [&](float tt, float* sn, float* cs) {
@@ -1198,9 +1203,8 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
             if (p0 ? lane == 31 : lane == 0)
                 edge_pf = __ldg(a.oth + (long long)m0 * W + (p0 ? kr : kl));
         }
-        // two rows at a time for Metropolis (their draws and sin/cos interleave);
-        // the heat-bath's attempt loops do better one row at a time
-#pragma unroll (HB ? 1 : 2)
+        // two rows at a time (their draws and sin/cos interleave)
+#pragma unroll 2
         for (int r = 0; r < R; ++r) {
             const int m = m0 + r;
             const int p = (m + a.c) & 1;
@@ -1249,32 +1253,7 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
             float sx0, sy0, sx1, sy1;
             sc(th.x, &sy0, &sx0);
             sc(th.y, &sy1, &sx1);
-            if (a.update && HB) {
-                // both sites of the pair draw from the same Philox block per attempt
-                const VonMises m0 = von_mises_setup(hx0, hy0, a.beta);
-                const VonMises m1 = von_mises_setup(hx1, hy1, a.beta);
-                bool p0 = true, p1 = true;
-                uint32_t acc0 = 0u, acc1 = 0u;  // U1 outputs of the accepted attempts
-                for (int at = 0; at < kVonMisesAttempts && (p0 || p1); ++at) {
-                    const uint4 rnd = philox4x32_10(
-                        make_uint4((uint32_t)(j >> 1), t, a.replica,
-                                   ((uint32_t)at << 16) | (kSweep << 1) | (uint32_t)a.c),
-                        a.rk);
-                    if (p0 && von_mises_accept(m0, rnd.x, rnd.y)) {
-                        acc0 = rnd.x;
-                        p0 = false;
-                    }
-                    if (p1 && von_mises_accept(m1, rnd.z, rnd.w)) {
-                        acc1 = rnd.z;
-                        p1 = false;
-                    }
-                }
-                if (!p0) th.x = von_mises_angle(m0, acc0);
-                if (!p1) th.y = von_mises_angle(m1, acc1);
-                sincos_angle<FAST>(th.x, &sy0, &sx0);
-                sincos_angle<FAST>(th.y, &sy1, &sx1);
-                *reinterpret_cast<float2*>(a.own + j) = th;
-            } else if (a.update) {
+            if (a.update) {
                 const uint4 rnd = philox4x32_10(
                     make_uint4((uint32_t)(j >> 1), t, a.replica, (kSweep << 1) | (uint32_t)a.c),
                     a.rk);
@@ -1310,6 +1289,172 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
             cur = nxt;
         }
     }
+    if (!MEAS) return;
+    const Partial mine = fp_partial(pe, pmx, pmy, 0.f, red);
+    store_partial(a.partials, mine);
+}
+
+// XY heat-bath, 2D, on the same column pairs.  Best and Fisher's method takes
+// some 1.4 attempts per site, but a warp that repeats attempts until its slowest
+// of 64 sites accepts runs 4 or 5 (18 of 32 lanes active; 227 us a pass at L =
+// 4096).  Here every site makes its first attempt in place; the sites it rejects
+// go to a list in shared memory, one list per warp, and whenever 32 are waiting
+// each lane takes one for its next attempt and those rejected again go back.  The
+// list also carries across rows, so every attempt but the last few of a warp runs
+// with all lanes.  Attempts, their random numbers and the arithmetic of a site
+// are those of the loop; an own-colour angle written late is read by nobody in
+// the pass.
+constexpr int kHbList = 96;  // fewer than 32 waiting, then up to 64 from a row
+
+template <bool MEAS>
+__global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
+{
+    __shared__ double red[32];  // 4 per warp
+    struct List {
+        uint32_t j[kHbList], at[kHbList];
+        float rho[kHbList], g[kHbList], cnum[kHbList], arg[kHbList];
+        float hx[MEAS ? kHbList : 1], hy[MEAS ? kHbList : 1];
+    };
+    __shared__ List lists[8];
+    List& q = lists[threadIdx.x >> 5];
+    const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
+    const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
+    const int L = a.L, W = a.W, R = a.R;  // (L^2 <= 2^31: offsets fit in 32 bits)
+    const int WP = W / 2;
+    const int lane = threadIdx.x & 31;
+    const uint32_t below = (1u << lane) - 1u;
+    const long long nitems = (long long)WP * (L / R);
+    const float J = a.J;
+    float pe = 0.f, pmx = 0.f, pmy = 0.f;
+    int nq = 0;  // sites waiting (the same in every lane)
+    auto push = [&](bool wait, uint32_t j, uint32_t at, const VonMises& m, float hx, float hy) {
+        const uint32_t b = __ballot_sync(0xFFFFFFFFu, wait);
+        if (wait) {
+            const int k = nq + __popc(b & below);
+            q.j[k] = j;
+            q.at[k] = at;
+            q.rho[k] = m.rho;
+            q.g[k] = m.g;
+            q.cnum[k] = m.cnum;
+            q.arg[k] = m.arg;
+            if (MEAS) {
+                q.hx[k] = hx;
+                q.hy[k] = hy;
+            }
+        }
+        nq += __popc(b);
+        __syncwarp();
+    };
+    // the accepted attempt's angle (U1 output o1) becomes site j's
+    auto settle = [&](uint32_t j, float th, float hx, float hy) {
+        a.own[j] = th;
+        if (MEAS) {
+            float sx, sy;
+            sincos_turns(th, &sy, &sx);
+            pe -= sx * hx + sy * hy;
+            pmx += sx;
+            pmy += sy;
+        }
+    };
+    // the next attempt of the last n waiting sites, one per lane
+    auto serve = [&](int n) {
+        const int k = nq - n + lane;
+        const bool mine = lane < n;
+        uint32_t j = 0u, at = 0u;
+        VonMises m = {0.f, 1.f, 1.f, 0.f};
+        float hx = 0.f, hy = 0.f;
+        if (mine) {
+            j = q.j[k];
+            at = q.at[k];
+            m.rho = q.rho[k];
+            m.g = q.g[k];
+            m.cnum = q.cnum[k];
+            m.arg = q.arg[k];
+            if (MEAS) {
+                hx = q.hx[k];
+                hy = q.hy[k];
+            }
+        }
+        nq -= n;
+        __syncwarp();
+        const uint32_t w = (at << 16) | (kSweep << 1) | (uint32_t)a.c;
+        const uint4 rnd =
+            philox_tail(philox_head(j >> 1, w ^ a.rk.k1[0]), pg.x2, pg.z2, pg.w2, a.rk);
+        const uint32_t o1 = (j & 1u) ? rnd.z : rnd.x, o2 = (j & 1u) ? rnd.w : rnd.y;
+        const bool acc = mine && von_mises_accept(m, o1, o2);
+        if (acc) settle(j, von_mises_angle(m, o1), hx, hy);
+        // (after the last attempt the old angle stays)
+        const bool keep = mine && !acc && at + 1 == kVonMisesAttempts;
+        if (MEAS && keep) settle(j, a.own[j], hx, hy);
+        push(mine && !acc && !keep, j, at + 1, m, hx, hy);
+    };
+    for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nitems;
+         it += (long long)gridDim.x * blockDim.x) {
+        const int k0 = 2 * (int)(it % WP);
+        const int m0 = (int)(it / WP) * R;
+        const int kl = k0 == 0 ? W - 1 : k0 - 1, kr = k0 + 2 == W ? 0 : k0 + 2;
+        auto pair = [&](int m) { return cs_pair<false>(a.oth, (long long)m * W + k0); };
+        CS2 prev = pair(m0 == 0 ? L - 1 : m0 - 1), cur = pair(m0);
+        float2 nxt_pf = __ldg(reinterpret_cast<const float2*>(
+            a.oth + (long long)(m0 == L - 1 ? 0 : m0 + 1) * W + k0));
+#pragma unroll 1
+        for (int r = 0; r < R; ++r) {
+            const int m = m0 + r;
+            const int p = (m + a.c) & 1;
+            const uint32_t j = (uint32_t)m * (uint32_t)W + (uint32_t)k0;
+            CS2 nxt;
+            sincos_turns(nxt_pf.x, &nxt.s0, &nxt.c0);
+            sincos_turns(nxt_pf.y, &nxt.s1, &nxt.c1);
+            if (r + 1 < R) {
+                const int m2 = m + 2 >= L ? m + 2 - L : m + 2;
+                nxt_pf = __ldg(reinterpret_cast<const float2*>(a.oth + (long long)m2 * W + k0));
+            }
+            // the column beside the pair: 2q-1 (p = 0) or 2q+2 (p = 1)
+            float ec, es;
+            if (p == 0) {
+                ec = __shfl_up_sync(0xffffffffu, cur.c1, 1);
+                es = __shfl_up_sync(0xffffffffu, cur.s1, 1);
+                if (lane == 0) sincos_turns(__ldg(a.oth + (long long)m * W + kl), &es, &ec);
+            } else {
+                ec = __shfl_down_sync(0xffffffffu, cur.c0, 1);
+                es = __shfl_down_sync(0xffffffffu, cur.s0, 1);
+                if (lane == 31) sincos_turns(__ldg(a.oth + (long long)m * W + kr), &es, &ec);
+            }
+            float hx0, hy0, hx1, hy1;
+            if (p == 0) {
+                hx0 = ec + cur.c0;
+                hy0 = es + cur.s0;
+                hx1 = cur.c0 + cur.c1;
+                hy1 = cur.s0 + cur.s1;
+            } else {
+                hx0 = cur.c0 + cur.c1;
+                hy0 = cur.s0 + cur.s1;
+                hx1 = cur.c1 + ec;
+                hy1 = cur.s1 + es;
+            }
+            hx0 = J * (hx0 + prev.c0 + nxt.c0);
+            hy0 = J * (hy0 + prev.s0 + nxt.s0);
+            hx1 = J * (hx1 + prev.c1 + nxt.c1);
+            hy1 = J * (hy1 + prev.s1 + nxt.s1);
+            const VonMises v0 = von_mises_setup(hx0, hy0, a.beta);
+            const VonMises v1 = von_mises_setup(hx1, hy1, a.beta);
+            const uint4 rnd = philox_at(pg, j >> 1, a.rk);
+            const bool a0 = von_mises_accept(v0, rnd.x, rnd.y);
+            const bool a1 = von_mises_accept(v1, rnd.z, rnd.w);
+            if (a0) settle(j, von_mises_angle(v0, rnd.x), hx0, hy0);
+            if (a1) settle(j + 1, von_mises_angle(v1, rnd.z), hx1, hy1);
+            if (MEAS) {
+                pmx += cur.c0 + cur.c1;
+                pmy += cur.s0 + cur.s1;
+            }
+            push(!a0, j, 1u, v0, hx0, hy0);
+            push(!a1, j + 1, 1u, v1, hx1, hy1);
+            while (nq >= 32) serve(32);
+            prev = cur;
+            cur = nxt;
+        }
+    }
+    while (nq > 0) serve(nq < 32 ? nq : 32);
     if (!MEAS) return;
     const Partial mine = fp_partial(pe, pmx, pmy, 0.f, red);
     store_partial(a.partials, mine);
@@ -1811,9 +1956,14 @@ cudaError_t launch_on(const sl_lattice* h, OnArgs a, cudaStream_t s)
                 else SPINMC_ON(heis_stream, 3, false, false);
             }
         } else {
-            if (var == 2) SPINMC_ON(xy_stream, false, true);
-            else if (var == 1) SPINMC_ON(xy_stream, true, false);
-            else SPINMC_ON(xy_stream, false, false);
+            if (var == 2) {
+                if (a.measure) xy_heatbath<true><<<grid, 256, 0, s>>>(a);
+                else xy_heatbath<false><<<grid, 256, 0, s>>>(a);
+            } else if (var == 1) {
+                SPINMC_ON(xy_stream, true);
+            } else {
+                SPINMC_ON(xy_stream, false);
+            }
         }
 #undef SPINMC_ON
         return a.measure ? launch_finish(h, a, (unsigned)grid, s) : cudaGetLastError();
