@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
     auto zprev = [&](int m) { return m == 0 ? (SLAB ? -1 : Lz - 1) : m - 1; };
     auto znext = [&](int m) { return m == Lz - 1 ? (SLAB ? Lz : 0) : m + 1; };
     const long long nitems = (long long)W16 * (D == 3 ? L : 1) * nseg;
-    const uint32_t ctr_w = (kSweep << 1) | (uint32_t)a.c;
+    const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
     const uint32_t two_d = 0x01010101u * (uint32_t)(2 * D);
     const uint32_t ones = 0x01010101u;
     // Counts of the measuring pass.  2D: 32-bit per-thread counters across
@@ -323,8 +323,9 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
         const int seg = D == 3 ? (int)(rest / L) : (int)rest;
         const int k0 = cx << 4;
         const int m0 = seg * R;
-        auto off = [&](int yy, int zz) -> long long { return ((long long)zz * L + yy) * W; };
-        auto moff = [&](int m) -> long long { return D == 3 ? off(y3, m) : off(m, 0); };
+        // (a colour array holds fewer than 2^31 entries)
+        auto off = [&](int yy, int zz) -> int { return (zz * L + yy) * W; };
+        auto moff = [&](int m) -> int { return D == 3 ? off(y3, m) : off(m, 0); };
         const int mprev = zprev(m0);
         uint4 prev = ld_rows(a.oth + moff(mprev) + k0);
         uint4 cur = ld_rows(a.oth + moff(m0) + k0);
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
             int yy, zz;
             row_of(m, yy, zz);
             const int p = (yy + zz + a.c + par) & 1;
-            const long long ro = off(yy, zz);
+            const int ro = off(yy, zz);
             const int eidx = edge_idx(p);
             const uint4 A = A_nx;
             const uint32_t edge = edge_nx;
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
                     // heat-bath: na = neighbours with Jb_k s_k = -1, so h = 2d - 2 na;
                     // the new spin is down iff u > hb[h + 2d]
                     if (!BONDS) {
-                        na = nxm + nxp + w_of(prev, k) + w_of(nxt, k);
+                        na = w_of(cur, k) + w_of(S, k) + w_of(prev, k) + w_of(nxt, k);
                         if (D == 3) na += w_of(ym, k) + w_of(yp, k);
                     } else {
                         na = (nxm ^ w_of(jx_oth, k)) + (nxp ^ w_of(jx_own, k));
@@ -433,7 +434,7 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
                                   (w_of(prev, k) ^ w_of(jz_oth, k)) + (w_of(nxt, k) ^ w_of(jz_own, k));
                         }
                     }
-                    const uint4 rnd = philox4x32_10(make_uint4(g0 + k, t, a.replica, ctr_w), a.rk);
+                    const uint4 rnd = philox_at(pg, g0 + k, a.rk);
                     const uint32_t u[4] = {rnd.x, rnd.y, rnd.z, rnd.w};
                     uint32_t down_new = 0;
 #pragma unroll
@@ -455,7 +456,7 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
                     continue;
                 }
                 if (!BONDS) {
-                    uint32_t nd = nxm + nxp + w_of(prev, k) + w_of(nxt, k);
+                    uint32_t nd = w_of(cur, k) + w_of(S, k) + w_of(prev, k) + w_of(nxt, k);
                     if (D == 3) nd += w_of(ym, k) + w_of(yp, k);
                     // own spin down: na = 2d - nd = (nd ^ 7) - (7 - 2d)
                     na = (nd ^ (av * 7u)) - av * (uint32_t)(7 - 2 * D);
@@ -472,7 +473,7 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
                     }
                 }
                 if (JNEG) na = two_d - na;
-                const uint4 rnd = philox4x32_10(make_uint4(g0 + k, t, a.replica, ctr_w), a.rk);
+                const uint4 rnd = philox_at(pg, g0 + k, a.rk);
                 // byte bit 7 set iff na >= q(u): accept
                 const uint32_t flip = ((na + q_bias<D>(rnd, a.tab)) & 0x80808080u) >> 7;
                 const uint32_t an = av ^ flip;
