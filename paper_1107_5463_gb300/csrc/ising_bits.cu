@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(128) bits_stream(const BitArgs a)
     auto zprev = [&](int m) { return m == 0 ? (SLAB ? -1 : Lz - 1) : m - 1; };
     auto znext = [&](int m) { return m == Lz - 1 ? (SLAB ? Lz : 0) : m + 1; };
     const long long nitems = (long long)WW * (D == 3 ? L : 1) * nseg;
-    const uint32_t ctr_w = (kSweep << 1) | (uint32_t)a.c;
+    const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
     const uint32_t inv = JNEG ? 0xFFFFFFFFu : 0u;
     unsigned long long s_na = 0, s_flip = 0, s_flipna = 0, down = 0, nsite = 0;
 
@@ -162,14 +162,15 @@ __global__ void __launch_bounds__(128) bits_stream(const BitArgs a)
                 const uint32_t grp = (uint32_t)((rr * a.W + gofs + 32 * w) >> 2);
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
-                    const uint4 rnd = philox4x32_10(make_uint4(grp + q, t, a.replica, ctr_w), a.rk);
+                    const uint4 rnd = philox_at(pg, grp + q, a.rk);
                     const uint32_t u[4] = {rnd.x, rnd.y, rnd.z, rnd.w};
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {
                         const uint32_t bit = 1u << (4 * q + b);
-                        if (u[b] > a.tab.thr[0]) g0 |= bit;
-                        if (u[b] > a.tab.thr[1]) g1 |= bit;
-                        if (D == 3 && u[b] > a.tab.thr[2]) g2 |= bit;
+                        // (added, not or-ed: an add can go to the FMA pipe)
+                        if (u[b] > a.tab.thr[0]) g0 += bit;
+                        if (u[b] > a.tab.thr[1]) g1 += bit;
+                        if (D == 3 && u[b] > a.tab.thr[2]) g2 += bit;
                     }
                 }
                 flip = (~g0 | ge1) & (~g1 | ge2);
