@@ -696,6 +696,7 @@ __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
     const uint32_t t = (uint32_t)t64;
     const bool renorm = a.update && a.renorm_every > 0 &&
                         (t64 + 1) % (unsigned long long)a.renorm_every == 0;
+    const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
     const int L = a.L, W = a.W, R = a.R;
     const int WP = W / 2;
     const long long H = a.H;  // < 2^31: every offset below fits in 32 bits
@@ -811,9 +812,7 @@ __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
                 uint4 rnd2[2];
 #pragma unroll
                 for (int b = 0; b < 2; ++b)
-                    rnd2[b] = philox4x32_10(
-                        make_uint4((uint32_t)(j + b), t, a.replica, (kSweep << 1) | (uint32_t)a.c),
-                        a.rk);
+                    rnd2[b] = philox_at(pg, (uint32_t)(j + b), a.rk);
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
                     const uint4 rnd = rnd2[b];
@@ -1169,7 +1168,7 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
         if (TAB) sincos_turns_tab(tab, tt, sn, cs);
         else sincos_angle<FAST>(tt, sn, cs);
     };
-    auto sc_pair = [&](const float* p, long long i) {
+    auto sc_pair = [&](const float* p, int i) {
         const float2 th = __ldg(reinterpret_cast<const float2*>(p + i));
         CS2 r;
         sc(th.x, &r.s0, &r.c0);
@@ -1179,6 +1178,7 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
     const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
     const int L = a.L, W = a.W, R = a.R;
     const int WP = W / 2;
+    const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
     const int lane = threadIdx.x & 31;
     const long long nitems = (long long)WP * (L / R);
     const float J = a.J;
@@ -1189,11 +1189,11 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
         const int m0 = (int)(it / WP) * R;
         const int k0 = 2 * q;
         const int mprev = m0 == 0 ? L - 1 : m0 - 1;
-        CS2 prev = sc_pair(a.oth, (long long)mprev * W + k0);
-        CS2 cur = sc_pair(a.oth, (long long)m0 * W + k0);
+        CS2 prev = sc_pair(a.oth, mprev * W + k0);
+        CS2 cur = sc_pair(a.oth, m0 * W + k0);
         float2 nxt_pf = __ldg(reinterpret_cast<const float2*>(
-            a.oth + (long long)(m0 == L - 1 ? 0 : m0 + 1) * W + k0));
-        float2 own_pf = *reinterpret_cast<const float2*>(a.own + (long long)m0 * W + k0);
+            a.oth + (m0 == L - 1 ? 0 : m0 + 1) * W + k0));
+        float2 own_pf = *reinterpret_cast<const float2*>(a.own + m0 * W + k0);
         // angle of the x neighbour a warp-edge lane cannot get by shuffle:
         // column 2q-1 for lane 0 when p = 0, column 2q+2 for lane 31 when p = 1
         const int kl = k0 == 0 ? W - 1 : k0 - 1, kr = k0 + 2 == W ? 0 : k0 + 2;
@@ -1201,14 +1201,14 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
         {
             const int p0 = (m0 + a.c) & 1;
             if (p0 ? lane == 31 : lane == 0)
-                edge_pf = __ldg(a.oth + (long long)m0 * W + (p0 ? kr : kl));
+                edge_pf = __ldg(a.oth + m0 * W + (p0 ? kr : kl));
         }
         // two rows at a time (their draws and sin/cos interleave)
 #pragma unroll 2
         for (int r = 0; r < R; ++r) {
             const int m = m0 + r;
             const int p = (m + a.c) & 1;
-            const long long j = (long long)m * W + k0;
+            const int j = m * W + k0;  // (fewer than 2^31 entries)
             CS2 nxt;
             sc(nxt_pf.x, &nxt.s0, &nxt.c0);
             sc(nxt_pf.y, &nxt.s1, &nxt.c1);
@@ -1216,11 +1216,11 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
             const float edge = edge_pf;
             if (r + 1 < R) {
                 const int m2 = m + 2 >= L ? m + 2 - L : m + 2;
-                nxt_pf = __ldg(reinterpret_cast<const float2*>(a.oth + (long long)m2 * W + k0));
-                own_pf = *reinterpret_cast<const float2*>(a.own + (long long)(m + 1) * W + k0);
+                nxt_pf = __ldg(reinterpret_cast<const float2*>(a.oth + m2 * W + k0));
+                own_pf = *reinterpret_cast<const float2*>(a.own + (m + 1) * W + k0);
                 const int p1 = p ^ 1;
                 if (p1 ? lane == 31 : lane == 0)
-                    edge_pf = __ldg(a.oth + (long long)(m + 1) * W + (p1 ? kr : kl));
+                    edge_pf = __ldg(a.oth + (m + 1) * W + (p1 ? kr : kl));
             }
             // x neighbours of column 2q and 2q+1:
             //   p = 0: (2q-1, 2q) and (2q, 2q+1);  p = 1: (2q, 2q+1) and (2q+1, 2q+2)
@@ -1254,9 +1254,7 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
             sc(th.x, &sy0, &sx0);
             sc(th.y, &sy1, &sx1);
             if (a.update) {
-                const uint4 rnd = philox4x32_10(
-                    make_uint4((uint32_t)(j >> 1), t, a.replica, (kSweep << 1) | (uint32_t)a.c),
-                    a.rk);
+                const uint4 rnd = philox_at(pg, (uint32_t)j >> 1, a.rk);
                 const float n0 = u24(rnd.y), n1 = u24(rnd.w);
                 float nx0, ny0, nx1, ny1;
                 sc(n0, &ny0, &nx0);
