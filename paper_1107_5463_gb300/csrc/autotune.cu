@@ -8,8 +8,8 @@
 // capped at 0, 2, 4, 8 or 16 blocks per SM, and for Heisenberg spins the
 // column-pair, single-column or staged-tile kernel where each applies) on the
 // lattice itself, restores its spins and sweep counter, and keeps the
-// fastest.  Choices can be cached
-// in a file of JSON lines, one per (device, d, L, n, storage, couplings,
+// fastest, or the automatic shape where that is faster still.  Choices can be
+// cached in a file of JSON lines, one per (device, d, L, n, storage, couplings,
 // update rule, fast math), read before timing and appended after.
 #include <cstdio>
 #include <cstring>
@@ -76,7 +76,8 @@ bool int_field(const char* line, const char* name, int* v)
     return true;
 }
 
-bool cache_lookup(const char* path, const TuneKey& k, int* rows, int* caps, int* kernel)
+bool cache_lookup(const char* path, const TuneKey& k, int* rows, int* caps, int* kernel,
+                  int* automatic)
 {
     FILE* f = std::fopen(path, "r");
     if (!f) return false;
@@ -96,6 +97,7 @@ bool cache_lookup(const char* path, const TuneKey& k, int* rows, int* caps, int*
             *rows = v[8];
             *caps = cap;
             *kernel = kern;
+            if (!int_field(line, "auto", automatic)) *automatic = 0;
             found = true;  // the last matching line wins
         }
     }
@@ -103,7 +105,8 @@ bool cache_lookup(const char* path, const TuneKey& k, int* rows, int* caps, int*
     return found;
 }
 
-void cache_append(const char* path, const TuneKey& k, int rows, int caps, int kernel, double ms)
+void cache_append(const char* path, const TuneKey& k, int rows, int caps, int kernel,
+                  int automatic, double ms)
 {
     FILE* f = std::fopen(path, "a");
     if (!f) return;
@@ -111,9 +114,9 @@ void cache_append(const char* path, const TuneKey& k, int rows, int caps, int ke
                  "{\"device\": \"%s\", \"sms\": %d, \"d\": %d, \"L\": %d, \"n\": %d, "
                  "\"storage\": %d, \"j_layout\": %d, \"update\": %d, \"fast\": %d, "
                  "\"rows\": %d, \"blocks_per_sm\": %d, \"kernel\": %d, "
-                 "\"ms_per_sweep\": %.6f}\n",
+                 "\"auto\": %d, \"ms_per_sweep\": %.6f}\n",
                  k.device.c_str(), k.sms, k.d, k.L, k.n, k.storage, k.j_layout, k.update, k.fast,
-                 rows, caps, kernel, ms);
+                 rows, caps, kernel, automatic, ms);
     std::fclose(f);
 }
 
@@ -143,12 +146,13 @@ extern "C" int sl_autotune(sl_lattice* h, double beta, int trial_sweeps, const c
     };
     if (!tunable(h)) return report();
     const TuneKey key = key_of(h);
-    int r = 0, c = 0, kc = 0;
-    if (cache_path && cache_lookup(cache_path, key, &r, &c, &kc) && r > 0 && h->Lz % r == 0 &&
+    int r = 0, c = 0, kc = 0, au = 0;
+    if (cache_path && cache_lookup(cache_path, key, &r, &c, &kc, &au) && r > 0 && h->Lz % r == 0 &&
         (kc == 0 || kc == 2 || (kc == 3 && h->n == 3) || (kc == 4 && h->n == 3 && h->d == 3))) {
         h->rows = r;
         h->blocks_per_sm = c;
         h->shape_tuned = 1;
+        h->shape_auto = au == 1;
         if (kc) h->kernel = kc;
         forget_graphs(h);
         return report();
@@ -177,6 +181,18 @@ extern "C" int sl_autotune(sl_lattice* h, double beta, int trial_sweeps, const c
     const int saved_rows = h->rows, saved_caps = h->blocks_per_sm, saved_kernel = h->kernel;
     int best_r = saved_rows, best_c = saved_caps, best_k = saved_kernel;
     float best = -1.f;
+    // milliseconds of the trial with the shape that h holds
+    auto trial = [&]() {
+        float ms = 0.f;
+        st = sweep_plain(h, p, 1, s);  // warm-up
+        if (st == SL_OK) e = cudaEventRecord(e0, s);
+        if (e == cudaSuccess && st == SL_OK) st = sweep_plain(h, p, trial_sweeps, s);
+        if (e == cudaSuccess && st == SL_OK) e = cudaEventRecord(e1, s);
+        if (e == cudaSuccess && st == SL_OK) e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess && st == SL_OK) e = cudaEventElapsedTime(&ms, e0, e1);
+        return ms;
+    };
+    h->shape_auto = 0;
     // Heisenberg: the kernel as set, single columns (3) where pairs are the
     // default, and the staged 3D tiles (4) where they apply
     int kernels[3] = {saved_kernel, -1, -1};
@@ -194,13 +210,7 @@ extern "C" int sl_autotune(sl_lattice* h, double beta, int trial_sweeps, const c
             h->kernel = kern;
             h->rows = R;
             h->blocks_per_sm = cap;
-            st = sweep_plain(h, p, 1, s);  // warm-up
-            if (st == SL_OK) e = cudaEventRecord(e0, s);
-            if (e == cudaSuccess && st == SL_OK) st = sweep_plain(h, p, trial_sweeps, s);
-            if (e == cudaSuccess && st == SL_OK) e = cudaEventRecord(e1, s);
-            if (e == cudaSuccess && st == SL_OK) e = cudaEventSynchronize(e1);
-            float ms = 0.f;
-            if (e == cudaSuccess && st == SL_OK) e = cudaEventElapsedTime(&ms, e0, e1);
+            const float ms = trial();
             if (e == cudaSuccess && st == SL_OK && (best < 0.f || ms < best)) {
                 best = ms;
                 best_r = R;
@@ -209,10 +219,27 @@ extern "C" int sl_autotune(sl_lattice* h, double beta, int trial_sweeps, const c
             }
         }
     }
+    // Segments in whole waves, which the automatic shape deals out for continuous
+    // spins, are mostly the faster choice: then they run, and the caller still learns
+    // the best of the shapes that the options can name (3D Heisenberg L = 256: 166 us
+    // and 143).
+    int automatic = 0;
+    for (int kern : kernels) {
+        if (h->n == 1 || kern < 0 || kern == 4 || e != cudaSuccess || st != SL_OK) continue;
+        h->kernel = kern;
+        h->rows = h->blocks_per_sm = 0;
+        const float ms = trial();
+        if (e == cudaSuccess && st == SL_OK && ms < best) {
+            best = ms;
+            best_k = kern;
+            automatic = 1;
+        }
+    }
     // put the state back whatever happened
     h->rows = best_r;
     h->blocks_per_sm = best_c;
     h->shape_tuned = 1;
+    h->shape_auto = automatic;
     h->kernel = best_k;
     cudaError_t e2 = cudaMemcpyAsync(h->spins[0], keep, colour_bytes, cudaMemcpyDeviceToDevice, s);
     if (e2 == cudaSuccess)
@@ -227,6 +254,7 @@ extern "C" int sl_autotune(sl_lattice* h, double beta, int trial_sweeps, const c
     if (e != cudaSuccess) return cuda_fail(e, "sl_autotune");
     if (e2 != cudaSuccess) return cuda_fail(e2, "sl_autotune: restore");
     if (cache_path && best >= 0.f)
-        cache_append(cache_path, key, best_r, best_c, best_k, best / trial_sweeps);
+        cache_append(cache_path, key, best_r, best_c, best_k, automatic,
+                     best / trial_sweeps);
     return report();
 }

@@ -43,6 +43,12 @@ struct SweepParams {
 
 constexpr int kGraphSizes = 6;       // captured runs of 1, 2, 4 .. 32 sweeps
 
+// The rows of a streaming kernel's marching axis dealt out to its items: nseg
+// segments, the first `rem` of q + 1 rows, the others of q.
+struct Segments {
+    int nseg, q, rem;
+};
+
 // A run of sweeps captured into a graph with the finishing kernel of every
 // measuring pass on a side branch: it takes 2 us (Ising) to 8 us (FP64 totals)
 // that the next sweep's colour-0 pass need not wait for.  The passes of sweep k
@@ -91,7 +97,8 @@ struct sl_lattice {
     // options
     int renorm_every, fast_math, kernel, rows, use_graph;
     int blocks_per_sm;       // cap of the streaming kernels' grids per SM (0 = none)
-    int shape_tuned;         // rows and blocks_per_sm come from sl_autotune, not from the user
+    int shape_tuned;         // rows and blocks_per_sm come from sl_autotune, not from the user,
+    int shape_auto;          // which measured them slower than the automatic shape: ignored
     int update;              // SL_UPDATE_METROPOLIS, _HEATBATH or _SW
     int multihit, tile;      // k-fold multi-hit sweeps in tiles of side `tile` (0 = off)
     // cached graphs of 2^i sweeps, captured when a call first needs one
@@ -122,6 +129,12 @@ int sweep_params(const sl_lattice* h, double beta, uint64_t seed, SweepParams* p
 cudaError_t set_sweep_index(const sl_lattice* h, int64_t t, cudaStream_t s);
 cudaError_t clear_series(const sl_lattice* h, cudaStream_t s);
 void forget_graphs(sl_lattice* h);
+// segments for `cols` columns of items on blocks of `threads` threads running
+// `kernel`, whose start costs a block as much as `start` rows
+Segments pick_segments(const sl_lattice* h, long long cols, int threads, const void* kernel,
+                       double start);
+// a streaming kernel's grid under the cap of SL_OPT_BLOCKS_PER_SM
+int grid_cap(const sl_lattice* h, int grid);
 // forked runs: which sweep's index and how far the finishing kernel advances it;
 // the stream of a finishing kernel; the joins around it (lattice.cu)
 inline unsigned fork_offset(const sl_lattice* h) { return h->fork ? h->fork->k : 0u; }

@@ -268,7 +268,7 @@ void check_graph_key(sl_lattice* h, const SweepParams& p)
              ((uint64_t)h->fast_math << 24) ^ ((uint64_t)h->update << 40) ^
              (uint64_t)h->renorm_every;
     key[3] = ((uint64_t)h->multihit << 16) ^ (uint64_t)h->tile ^
-             ((uint64_t)h->blocks_per_sm << 40);
+             ((uint64_t)h->blocks_per_sm << 40) ^ ((uint64_t)h->shape_auto << 56);
     if (std::memcmp(key, h->graph_key, sizeof key) == 0) return;
     drop_graphs(h);
     std::memcpy(h->graph_key, key, sizeof key);
@@ -434,7 +434,7 @@ int create_lattice(int d, int L, int n, int j_layout, int storage, double J, con
     h->kernel = 0;
     h->rows = 0;
     h->blocks_per_sm = 0;
-    h->shape_tuned = 0;
+    h->shape_tuned = h->shape_auto = 0;
     h->use_graph = 1;
     h->update = 0;
     h->multihit = 0;
@@ -520,6 +520,49 @@ cudaError_t clear_series(const sl_lattice* h, cudaStream_t s)
 }
 
 void forget_graphs(sl_lattice* h) { drop_graphs(h); }
+
+Segments pick_segments(const sl_lattice* h, long long cols, int threads, const void* kernel,
+                       double start)
+{
+    const int rows = h->Lz;
+    if (h->rows > 0 && !h->shape_auto) return Segments{rows / h->rows, h->rows, 0};
+    // Whole waves of resident blocks: k waves of n segments each, n as large as
+    // k waves hold.  In rows a pass takes k (rows / n) for the updates, k times
+    // what a block pays to start (half a row to fill its window, 3.5 where it
+    // also fills the sine table) and, as blocks do not end together, some 15% of
+    // a segment.  Power-of-two segments left the last wave up to three quarters
+    // empty: per sweep 3D Heisenberg L = 256 166 us, now 143 (k = 2; 155, 144,
+    // 147 for k = 1, 3, 4), L = 128 55 and 23; 2D XY L = 4096 105 and 92 (k = 1),
+    // L = 2048 46 and 30.  Ising kernels keep equal segments of 2^i rows: the row
+    // loop's end must be the same for a whole warp, or its addresses and keys
+    // leave the uniform registers (64 registers a thread became 78, and L = 16384
+    // 247 us a sweep became 255).
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, 0) != cudaSuccess ||
+        occ < 1)
+        occ = 1;
+    const double slots = (double)occ * h->sms;
+    Segments g{0, 0, 0};
+    double best = 0.0;
+    for (int k = 1; k <= 4; ++k) {
+        const double fit = std::floor(k * slots * threads / (double)cols);
+        const int n = fit < 1.0 ? 1 : (fit > rows ? rows : (int)fit);
+        const double waves = std::ceil(std::ceil((double)cols * n / threads) / slots);
+        const int seg = (rows + n - 1) / n;
+        const double cost = waves * (seg + start) + 0.15 * seg;
+        if (g.nseg == 0 || cost < best) {
+            g = Segments{n, rows / n, rows % n};
+            best = cost;
+        }
+    }
+    return g;
+}
+
+int grid_cap(const sl_lattice* h, int grid)
+{
+    const int cap = h->shape_auto ? 0 : h->sms * h->blocks_per_sm;
+    return cap > 0 && grid > cap ? cap : grid;
+}
 
 void fork_sweep(const sl_lattice* h, int64_t k)
 {
@@ -737,12 +780,12 @@ int sl_set_option(sl_lattice* h, int option, int64_t value)
         if (value < 0 || (value > 0 && (h->Lz % value != 0)))
             return fail(SL_EINVAL, "rows must be 0 (automatic) or divide the planes held");
         h->rows = (int)value;
-        h->shape_tuned = 0;
+        h->shape_tuned = h->shape_auto = 0;
         return SL_OK;
     case SL_OPT_BLOCKS_PER_SM:
         if (value < 0 || value > 64) return fail(SL_EINVAL, "blocks_per_sm must be in [0, 64]");
         h->blocks_per_sm = (int)value;
-        h->shape_tuned = 0;
+        h->shape_tuned = h->shape_auto = 0;
         return SL_OK;
     case SL_OPT_GRAPH:
         if (value != 0 && value != 1) return fail(SL_EINVAL, "graph must be 0 or 1");

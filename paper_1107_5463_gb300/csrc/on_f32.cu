@@ -41,7 +41,8 @@ struct OnArgs {
     const float* oth;
     const float* Jown[3];
     const float* Joth[3];
-    int d, L, W, c, R;
+    int d, L, W, c;
+    Segments seg;
     long long H, N;
     uint32_t replica;
     RoundKeys rk;
@@ -545,10 +546,10 @@ __global__ void __launch_bounds__(256, D == 2 && !HB ? 4 : 3) heis_stream(const 
     const uint32_t t = (uint32_t)t64;
     const bool renorm = a.update && a.renorm_every > 0 &&
                         (t64 + 1) % (unsigned long long)a.renorm_every == 0;
-    const int L = a.L, W = a.W, R = a.R;
+    const int L = a.L, W = a.W, nseg = a.seg.nseg;
     const long long H = a.H;  // < 2^31: every offset below fits in 32 bits
     const int lane = threadIdx.x & 31;
-    const long long nitems = (long long)W * (D == 3 ? L : 1) * (L / R);
+    const long long nitems = (long long)W * (D == 3 ? L : 1) * nseg;
     const float J = a.J;
     const float* ox = a.oth;
     const float* oy = a.oth + H;
@@ -569,7 +570,8 @@ __global__ void __launch_bounds__(256, D == 2 && !HB ? 4 : 3) heis_stream(const 
         const int k = (int)(it % W);
         const long long rest = it / W;
         const int y3 = D == 3 ? (int)(rest % L) : 0;
-        const int m0 = (int)(D == 3 ? rest / L : rest) * R;
+        const int sg = (int)(D == 3 ? rest / L : rest);
+        const int m0 = sg * a.seg.q + min(sg, a.seg.rem), R = a.seg.q + (sg < a.seg.rem);
         // offset of the colour entry at column k of the row at march index m
         // (2D: row y = m; 3D: row (y3, z = m)); rows y3 -/+ 1 in the same plane
         auto off = [&](int m) -> int { return (D == 3 ? m * L + y3 : m) * W + k; };
@@ -697,11 +699,11 @@ __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
     const bool renorm = a.update && a.renorm_every > 0 &&
                         (t64 + 1) % (unsigned long long)a.renorm_every == 0;
     const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
-    const int L = a.L, W = a.W, R = a.R;
+    const int L = a.L, W = a.W, nseg = a.seg.nseg;
     const int WP = W / 2;
     const long long H = a.H;  // < 2^31: every offset below fits in 32 bits
     const int lane = threadIdx.x & 31;
-    const long long nitems = (long long)WP * (D == 3 ? L : 1) * (L / R);
+    const long long nitems = (long long)WP * (D == 3 ? L : 1) * nseg;
     const float J = a.J;
     const float* ox = a.oth;
     const float* oy = a.oth + H;
@@ -736,7 +738,8 @@ __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
         const int k0 = 2 * (int)(it % WP);
         const long long rest = it / WP;
         const int y3 = D == 3 ? (int)(rest % L) : 0;
-        const int m0 = (int)(D == 3 ? rest / L : rest) * R;
+        const int sg = (int)(D == 3 ? rest / L : rest);
+        const int m0 = sg * a.seg.q + min(sg, a.seg.rem), R = a.seg.q + (sg < a.seg.rem);
         auto off = [&](int m) -> int { return (D == 3 ? m * L + y3 : m) * W + k0; };
         const int dym = (y3 == 0 ? L - 1 : -1) * W, dyp = (y3 == L - 1 ? 1 - L : 1) * W;
         const int mprev = m0 == 0 ? L - 1 : m0 - 1;
@@ -1176,17 +1179,18 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
         return r;
     };
     const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
-    const int L = a.L, W = a.W, R = a.R;
+    const int L = a.L, W = a.W, nseg = a.seg.nseg;
     const int WP = W / 2;
     const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
     const int lane = threadIdx.x & 31;
-    const long long nitems = (long long)WP * (L / R);
+    const long long nitems = (long long)WP * nseg;
     const float J = a.J;
     float pe = 0.f, pmx = 0.f, pmy = 0.f;
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nitems;
          it += (long long)gridDim.x * blockDim.x) {
         const int q = (int)(it % WP);
-        const int m0 = (int)(it / WP) * R;
+        const int sg = (int)(it / WP);
+        const int m0 = sg * a.seg.q + min(sg, a.seg.rem), R = a.seg.q + (sg < a.seg.rem);
         const int k0 = 2 * q;
         const int mprev = m0 == 0 ? L - 1 : m0 - 1;
         CS2 prev = sc_pair(a.oth, mprev * W + k0);
@@ -1317,11 +1321,11 @@ __global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
     List& q = lists[threadIdx.x >> 5];
     const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
     const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
-    const int L = a.L, W = a.W, R = a.R;  // (L^2 <= 2^31: offsets fit in 32 bits)
+    const int L = a.L, W = a.W, nseg = a.seg.nseg;  // (L^2 <= 2^31: offsets fit in 32 bits)
     const int WP = W / 2;
     const int lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;
-    const long long nitems = (long long)WP * (L / R);
+    const long long nitems = (long long)WP * nseg;
     const float J = a.J;
     float pe = 0.f, pmx = 0.f, pmy = 0.f;
     int nq = 0;  // sites waiting (the same in every lane)
@@ -1389,7 +1393,8 @@ __global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nitems;
          it += (long long)gridDim.x * blockDim.x) {
         const int k0 = 2 * (int)(it % WP);
-        const int m0 = (int)(it / WP) * R;
+        const int sg = (int)(it / WP);
+        const int m0 = sg * a.seg.q + min(sg, a.seg.rem), R = a.seg.q + (sg < a.seg.rem);
         const int kl = k0 == 0 ? W - 1 : k0 - 1, kr = k0 + 2 == W ? 0 : k0 + 2;
         auto pair = [&](int m) { return cs_pair<false>(a.oth, (long long)m * W + k0); };
         CS2 prev = pair(m0 == 0 ? L - 1 : m0 - 1), cur = pair(m0);
@@ -1789,7 +1794,7 @@ OnArgs make_args(const sl_lattice* h, int c)
     a.partials = h->partials;
     a.measure = c == 1;
     a.update = 1;
-    a.R = 1;
+    a.seg = Segments{1, 1, 0};
     a.renorm_every = h->renorm_every;
     return a;
 }
@@ -1881,15 +1886,6 @@ namespace spinmc {
 
 namespace {
 
-int on_rows(const sl_lattice* h, long long cols)
-{
-    if (h->rows > 0) return h->rows;
-    const long long cross = h->d == 3 ? h->L : 1;
-    int R = 32;
-    while (R > 1 && (h->L % R != 0 || cols * cross * (h->L / R) < (long long)h->sms * 1024)) R >>= 1;
-    return R;
-}
-
 // kernel variant: 0 Metropolis, 1 Metropolis with intrinsics, 2 heat-bath
 // (whose draws and fields use the accurate functions only)
 template <int D, bool EVEN>
@@ -1923,15 +1919,17 @@ cudaError_t launch_on(const sl_lattice* h, OnArgs a, cudaStream_t s)
         // single columns); XY always takes pairs
         const bool pairs = NC == 2 || (h->W % 64 == 0 && h->kernel != 3);
         const long long cols = pairs ? h->W / 2 : h->W;
-        a.R = on_rows(h, cols);
-        const long long items = cols * (h->d == 3 ? h->L : 1) * (h->L / a.R);
-        int grid = grid_for(items, 256);
-        if (h->blocks_per_sm > 0 && grid > h->sms * h->blocks_per_sm)
-            grid = h->sms * h->blocks_per_sm;
-#define SPINMC_ON(K, ...)                                                      \
-    do {                                                                       \
-        if (a.measure) K<__VA_ARGS__, true><<<grid, 256, 0, s>>>(a);          \
-        else K<__VA_ARGS__, false><<<grid, 256, 0, s>>>(a);                   \
+        const long long lanes = cols * (h->d == 3 ? h->L : 1);
+        int grid = 0;
+        auto run = [&](void (*k)(const OnArgs)) {
+            a.seg = pick_segments(h, lanes, 256, (const void*)k, var == 0 ? 3.5 : 0.5);
+            grid = grid_cap(h, grid_for(lanes * a.seg.nseg, 256));
+            k<<<grid, 256, 0, s>>>(a);
+        };
+#define SPINMC_ON(K, ...)                         \
+    do {                                          \
+        if (a.measure) run(K<__VA_ARGS__, true>); \
+        else run(K<__VA_ARGS__, false>);          \
     } while (0)
         if (NC == 3 && pairs) {
             if (h->d == 2) {
@@ -1955,8 +1953,8 @@ cudaError_t launch_on(const sl_lattice* h, OnArgs a, cudaStream_t s)
             }
         } else {
             if (var == 2) {
-                if (a.measure) xy_heatbath<true><<<grid, 256, 0, s>>>(a);
-                else xy_heatbath<false><<<grid, 256, 0, s>>>(a);
+                if (a.measure) run(xy_heatbath<true>);
+                else run(xy_heatbath<false>);
             } else if (var == 1) {
                 SPINMC_ON(xy_stream, true);
             } else {
