@@ -37,6 +37,7 @@
 // (u N) >> 32, u = output 0 of Philox(a, 0, walker, 8 << 1), iff that moves
 // the energy towards the window without passing its far edge; 1000 N
 // attempts at most.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -49,6 +50,10 @@ namespace {
 
 constexpr uint32_t kWalkInit = 8, kWL = 9, kMUCA = 10, kOrder = 11;
 constexpr int kKMax = 64;
+constexpr uint32_t kWalkRun = 1024u;             // attempts between a block's barriers
+constexpr uint32_t kWalkWords = 2 * 4 * 4 * 4;  // bytes of a warp's site words
+// most warps of a block, by the room for levels (72 registers a thread; 128)
+constexpr int walk_block(int KT) { return KT == 8 ? 28 : 16; }
 
 struct WalkArgs {
     uint32_t* spins;      // [warp][site] words
@@ -146,24 +151,24 @@ __global__ void __launch_bounds__(128) walk_init_kernel(WalkArgs a)
 
 // ------------------------------------------------------------ WL / MUCA ----
 
-// Wang-Landau decision for D < 0 (see the file comment): FP32 decides unless u
-// lies near the threshold exp(D 2^-32) 2^32 = 2^(D 2^-32 log2 e + 32).  The
-// conversions of D and u, the product (its argument below 160 where the result
-// is not flushed to zero) and the hardware exp2 leave a relative error below
-// 2^-16, a quarter of the margin; where the threshold underflows, u = 0 is near.
-// (D's 64-bit conversion runs on the FP64 unit, which has nothing else to do:
-// 15.9 ms for 10 sweeps of the workload, against 16.6 with D's halves converted
-// by the other units.)
-__device__ __forceinline__ bool wl_accept_fast(int64_t D, uint32_t u, bool* near)
+// Wang-Landau decision (see the file comment) in FP32: accept iff D >= 0 or
+// u 2^-32 < exp(D 2^-32), unless the two lie within 2^-16 of each other.  v is
+// 1 + u 2^-32, rounded down to 23 bits.  For D < 0 the threshold is a power of two of
+// D in units of 2^-20 (truncated; its high word clamped at -2048, where the threshold
+// has long underflowed): truncation, conversion, product (its argument below 35 where
+// the threshold is above 2^-50) and the hardware exp2 leave an error below 2^-18, v
+// and the difference 2^-22 more.  The one conversion runs on 32 bits: from 64 bits it
+// takes the FP64 unit 16 cycles a warp, 430 of the 700 that an attempt of a
+// multiprocessor's 27 warps took.
+__device__ __forceinline__ bool wl_accept_fast(int64_t D, float v, bool* near)
 {
+    const int hi = max((int)(D >> 32), -2048);
+    const int x = (int)__funnelshift_r((uint32_t)D, (uint32_t)hi, 12);
     float pf;
-    asm("ex2.approx.ftz.f32 %0, %1;"
-        : "=f"(pf)
-        : "f"(fmaf((float)D, 1.44269504f / 4294967296.0f, 32.0f)));
-    const float uf = (float)u;
-    const float m = 1.0f / 16384.0f;
-    const bool acc = uf < pf * (1.0f - m);
-    *near = !acc && uf <= pf * (1.0f + m);
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(pf) : "f"((float)x * (1.44269504f / 1048576.0f)));
+    const float e = pf - v, m = 1.0f / 65536.0f;
+    const bool acc = D >= 0 || e > m - 1.0f;
+    *near = !acc && e >= -1.0f - m;
     return acc;
 }
 
@@ -187,13 +192,13 @@ __device__ __forceinline__ bool order_is_clear(uint32_t oa, uint32_t L, uint32_t
     return clear;
 }
 
-// One warp per block, 32 walkers of a window.  An attempt is a short chain of
-// dependent steps (site words, level, ln g, decision, new level), and some 27
-// warps per multiprocessor are all there are, so what counts is instructions
-// per attempt and latency inside the chain.  Reading the five words of a site
-// from L2 at each attempt, an FP32 expf, two 64-bit and two 32-bit shared
-// memory updates took 103 instructions an attempt and 2.8 ms for a sweep of
-// 131072 Wang-Landau walkers of 64 x 64 sites; this takes 67 and 1.4 ms:
+// A warp is 32 walkers of a window.  An attempt is a short chain of dependent
+// steps (site words, level, ln g, decision, new level), and some 27 warps per
+// multiprocessor are all there are, so what counts is instructions per attempt,
+// latency inside the chain and having all warps at work.  Reading the five words
+// of a site from L2 at each attempt, an FP32 expf, two 64-bit and two 32-bit
+// shared memory updates took 103 instructions an attempt and 2.8 ms for a sweep
+// of 131072 Wang-Landau walkers of 64 x 64 sites; this takes 62 and 1.15 ms:
 //   - 20 lanes fetch the words of four attempts with one load, a group ahead,
 //     and pass them on through shared memory (wherever the sweep's order cannot
 //     bring two attempts within eight to a common word; else word by word as
@@ -201,24 +206,34 @@ __device__ __forceinline__ bool order_is_clear(uint32_t oa, uint32_t L, uint32_t
 //   - the current level's ln g stays in registers, H and the visited mask are
 //     worked out once per sweep from what ln g gained;
 //   - the decision takes one conversion and the hardware exp2, with the FP64
-//     test behind a warp vote.
+//     test behind a warp vote;
+//   - the warps of a multiprocessor are one block and meet every 1024 attempts.
+//     As single-warp blocks the older ones ran ahead, and the last ones then ran
+//     with too few others to fill the gaps: 20 warps in flight on average of 27,
+//     1.28 ms against 1.15 (multicanonical 1.01 and 0.88; every 64 attempts 1.16,
+//     every 4096 1.14).
 template <int KT, bool WL, bool SPINS_SMEM>
-__global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
+__global__ void __launch_bounds__(32 * walk_block(KT), 1) walk_kernel(const WalkArgs a,
+                                                                      const uint32_t warp_bytes)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
+    extern __shared__ __align__(16) unsigned char block_smem[];
     // H from the gain of S over a sweep (needs S at its start; not for the widest
     // windows, whose arrays fill the shared memory)
     constexpr bool SNAP = WL && KT <= 16;
-    __shared__ __align__(16) uint32_t words[2][4][4];
+    const int lane = threadIdx.x & 31;
+    const int warp_of = blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5);
+    const bool present = warp_of < a.nwalk / 32;  // (the last block may have idle warps)
+    const int warp = present ? warp_of : a.nwalk / 32 - 1;
+    unsigned char* smem = block_smem + (threadIdx.x >> 5) * warp_bytes;
+    uint32_t (*words)[4][4] = reinterpret_cast<uint32_t (*)[4][4]>(smem);  // [2][4][4]
+    smem += kWalkWords;
     const size_t colb = SPINS_SMEM ? 4 * (size_t)a.N : 0;
     // S has room for two levels on either side, so that a move out of the window
     // reads a value (which its decision ignores) without a test
-    int64_t* S = reinterpret_cast<int64_t*>(smem + colb) + 2 * 32;                // [KT][32]
-    uint32_t* H = reinterpret_cast<uint32_t*>(smem + colb + 8 * (KT + 4) * 32);   // [KT][32]
-    int64_t* T = reinterpret_cast<int64_t*>(H + KT * 32);                 // MUCA [KT][5]
-    int64_t* S0 = T;                                                      // SNAP [KT][32]
-    const int lane = threadIdx.x;
-    const int warp = blockIdx.x;
+    int64_t* S = reinterpret_cast<int64_t*>(smem + colb) + 2 * 32 + lane;  // [KT][32]
+    uint32_t* H = reinterpret_cast<uint32_t*>(smem + colb + 8 * (KT + 4) * 32) + lane;
+    int64_t* T = reinterpret_cast<int64_t*>(H - lane + KT * 32);  // MUCA [KT][5]
+    int64_t* S0 = T + lane;                                       // SNAP [KT][32]
     const int gw = warp * 32 + lane;
     const uint32_t walker = (uint32_t)gw;
     const int win = gw / a.wpw;  // the whole warp shares it (wpw % 32 == 0)
@@ -233,10 +248,10 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
     if (SPINS_SMEM)
         for (long long i = lane; i < N; i += 32) col[i] = gcol[i];
     if (WL)
-        for (int q = -2; q < KT + 2; ++q) S[q * 32 + lane] = 0;
+        for (int q = -2; q < KT + 2; ++q) S[q * 32] = 0;
     for (int q = 0; q < KT; ++q) {
-        S[q * 32 + lane] = q < a.kmax ? a.S[(size_t)q * a.nwalk + gw] : 0;
-        H[q * 32 + lane] = q < a.kmax && WL ? a.H[(size_t)q * a.nwalk + gw] : 0u;
+        S[q * 32] = q < a.kmax ? a.S[(size_t)q * a.nwalk + gw] : 0;
+        H[q * 32] = q < a.kmax && WL ? a.H[(size_t)q * a.nwalk + gw] : 0u;
     }
     if (!WL)
         // thresholds of the moves by -2 .. +2 levels (none: always; out of the window: never)
@@ -261,15 +276,19 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
 
     for (long long s = 0; s < a.nsweeps; ++s) {
         const uint32_t t = a.t0 + (uint32_t)s;
-        const bool active = !WL || stage <= a.final_stage;
-        if (!__any_sync(0xFFFFFFFFu, active)) break;
+        const bool active = present && (!WL || stage <= a.final_stage);
+        if (!__syncthreads_or(active)) break;
+        if (!__any_sync(0xFFFFFFFFu, active)) {
+            for (uint32_t q0 = 0; q0 < (uint32_t)N; q0 += kWalkRun) __syncthreads();
+            continue;
+        }
         uint32_t oa, ob;
         sweep_order(a, t, oa, ob);
         const int64_t inc = WL && active ? ((int64_t)1 << (32 - stage)) : 0;
         const unsigned Keff = active ? (unsigned)K : 0u;  // a finished walker never moves
         if (SNAP)
-            for (int q = 0; q < KT; ++q) S0[q * 32 + lane] = S[q * 32 + lane];
-        int64_t Skr = WL ? S[kr * 32 + lane] : 0;
+            for (int q = 0; q < KT; ++q) S0[q * 32] = S[q * 32];
+        int64_t Skr = WL ? S[kr * 32] : 0;
         // draws of the four attempts 4 g .. 4 g + 3 (the block of the next four is
         // drawn while the current four run; the one after the last goes unused)
         const PhiloxGroups pg = philox_groups(t, walker, (WL ? kWL : kMUCA) << 1, a.rk);
@@ -277,19 +296,20 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
         // one attempt: x0 .. x3 are the site's four neighbour words XOR its own;
         // returns the walkers whose spin flips
         auto attempt = [&](uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3, uint32_t u) {
-            int k2 = kr + 2;
-            if (x0 & lanebit) --k2;
-            if (x1 & lanebit) --k2;
-            if (x2 & lanebit) --k2;
-            if (x3 & lanebit) --k2;
+            // (summed apart from kr, the end of the chain of earlier attempts)
+            int dk = 2;
+            if (x0 & lanebit) --dk;
+            if (x1 & lanebit) --dk;
+            if (x2 & lanebit) --dk;
+            if (x3 & lanebit) --dk;
+            const int k2 = kr + dk;
             bool acc;
             if (WL) {
                 const bool in = (unsigned)k2 < Keff;
-                const int64_t S2 = S[k2 * 32 + lane];
+                const int64_t S2 = S[k2 * 32];
                 const int64_t D = Skr - S2;
                 bool near;
-                acc = wl_accept_fast(D, u, &near) || D >= 0;
-                near = near && in && D < 0;
+                acc = wl_accept_fast(D, __uint_as_float(0x3F800000u | (u >> 9)), &near);
                 if (__any_sync(0xFFFFFFFFu, near)) {
                     if (near) acc = wl_accept_exact(D, u);
                 }
@@ -299,15 +319,15 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
                     Skr = S2;
                 }
                 Skr += inc;
-                S[kr * 32 + lane] = Skr;
+                S[kr * 32] = Skr;
                 if (!SNAP && active) {
                     vis |= 1ull << kr;
-                    H[kr * 32 + lane] += 1u;
+                    H[kr * 32] += 1u;
                 }
             } else {
-                acc = (int64_t)u <= T[kr * 5 + (k2 - kr + 2)];
+                acc = (int64_t)u <= T[kr * 5 + dk + 2];
                 if (acc) kr = k2;
-                H[kr * 32 + lane] += 1u;
+                H[kr * 32] += 1u;
             }
             return __ballot_sync(0xFFFFFFFFu, acc);
         };
@@ -319,23 +339,28 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
                 return lane < 20 ? col[at_nx] : 0u;
             };
             uint32_t w_nx = fetch(0u);
-            for (uint32_t q = 0; q < (uint32_t)N; q += 4) {
-                uint32_t (*buf)[4] = words[(q >> 2) & 1];
-                const uint32_t w = w_nx;
-                at = at_nx;
-                const uint32_t x = w ^ __shfl_sync(0xFFFFFFFFu, w, 5 * (int)fa);
-                if (lane < 20 && fw > 0) buf[fa][fw - 1] = x;
-                const uint4 rnd = rnd_nx;
-                __syncwarp();  // also orders the flips before the loads below
-                w_nx = fetch(q + 4);
-                rnd_nx = philox_at(pg, (q >> 2) + 1u, a.rk);
-                const uint32_t uu[4] = {rnd.x, rnd.y, rnd.z, rnd.w};
+            for (uint32_t q0 = 0; q0 < (uint32_t)N; q0 += kWalkRun) {
+                __syncthreads();
+                const uint32_t q1 = min(q0 + kWalkRun, (uint32_t)N);
+                for (uint32_t q = q0; q < q1; q += 4) {
+                    uint32_t (*buf)[4] = words[(q >> 2) & 1];
+                    const uint32_t w = w_nx;
+                    at = at_nx;
+                    const uint32_t x = w ^ __shfl_sync(0xFFFFFFFFu, w, 5 * (int)fa);
+                    if (lane < 20 && fw > 0) buf[fa][fw - 1] = x;
+                    const uint4 rnd = rnd_nx;
+                    __syncwarp();  // also orders the flips before the loads below
+                    w_nx = fetch(q + 4);
+                    rnd_nx = philox_at(pg, (q >> 2) + 1u, a.rk);
+                    const uint32_t uu[4] = {rnd.x, rnd.y, rnd.z, rnd.w};
+                    uint32_t mine = 0u;  // flips of the site whose own word the lane fetched
 #pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const uint4 v = *reinterpret_cast<const uint4*>(buf[b]);
-                    const uint32_t flips = attempt(v.x, v.y, v.z, v.w, uu[b]);
-                    // the lane that fetched the site's own word writes it back
-                    if (lane == 5 * b && flips) col[at] = w ^ flips;
+                    for (int b = 0; b < 4; ++b) {
+                        const uint4 v = *reinterpret_cast<const uint4*>(buf[b]);
+                        const uint32_t flips = attempt(v.x, v.y, v.z, v.w, uu[b]);
+                        if (fa == (uint32_t)b) mine = flips;
+                    }
+                    if (fw == 0 && mine) col[at] = w ^ mine;  // (lanes 20 .. 31 hold none)
                 }
             }
         } else {
@@ -351,6 +376,7 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
                 __syncwarp();
             };
             for (uint32_t q = 0; q < (uint32_t)N; q += 4) {
+                if (q % kWalkRun == 0) __syncthreads();
                 const uint4 rnd = rnd_nx;
                 rnd_nx = philox_at(pg, (q >> 2) + 1u, a.rk);
                 single(q, rnd.x);
@@ -362,9 +388,9 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
         __syncwarp();
         if (SNAP && active)
             for (int q = 0; q < KT; ++q) {
-                const int64_t gain = S[q * 32 + lane] - S0[q * 32 + lane];
+                const int64_t gain = S[q * 32] - S0[q * 32];
                 if (gain > 0) vis |= 1ull << q;
-                H[q * 32 + lane] += (uint32_t)(gain >> (32 - stage));
+                H[q * 32] += (uint32_t)(gain >> (32 - stage));
             }
         if (WL && active) {
             int nv = 0;
@@ -372,32 +398,33 @@ __global__ void __launch_bounds__(32) walk_kernel(const WalkArgs a)
             for (int q = 0; q < KT; ++q)
                 if ((vis >> q) & 1ull) {
                     ++nv;
-                    sum += H[q * 32 + lane];
+                    sum += H[q * 32];
                 }
             bool flat = nv > 0;
             for (int q = 0; q < KT; ++q)
                 if (((vis >> q) & 1ull) &&
-                    (unsigned long long)H[q * 32 + lane] * (unsigned long long)nv * 100ull <
+                    (unsigned long long)H[q * 32] * (unsigned long long)nv * 100ull <
                         (unsigned long long)a.flat_percent * sum)
                     flat = false;
             if (flat) {
                 int64_t mn = INT64_MAX;
                 for (int q = 0; q < KT; ++q)
-                    if (((vis >> q) & 1ull) && S[q * 32 + lane] < mn) mn = S[q * 32 + lane];
+                    if (((vis >> q) & 1ull) && S[q * 32] < mn) mn = S[q * 32];
                 for (int q = 0; q < KT; ++q) {
-                    if ((vis >> q) & 1ull) S[q * 32 + lane] -= mn;
-                    H[q * 32 + lane] = 0u;
+                    if ((vis >> q) & 1ull) S[q * 32] -= mn;
+                    H[q * 32] = 0u;
                 }
                 ++stage;
             }
         }
     }
+    if (!present) return;
     __syncwarp();
     if (SPINS_SMEM)
         for (long long i = lane; i < N; i += 32) gcol[i] = col[i];
     for (int q = 0; q < a.kmax && q < KT; ++q) {
-        if (WL) a.S[(size_t)q * a.nwalk + gw] = S[q * 32 + lane];
-        a.H[(size_t)q * a.nwalk + gw] = H[q * 32 + lane];
+        if (WL) a.S[(size_t)q * a.nwalk + gw] = S[q * 32];
+        a.H[(size_t)q * a.nwalk + gw] = H[q * 32];
     }
     a.level[gw] = kr + klo;
     a.stage[gw] = stage;
@@ -497,14 +524,30 @@ int kt_for(int kmax)
 template <int KT, bool WL, bool SM>
 cudaError_t launch_walk_res(const WalkArgs& a, cudaStream_t s)
 {
-    // spins, S and H; thresholds (multicanonical) or S at the start of a sweep
+    // words, spins, S and H; thresholds (multicanonical) or S at the start of a sweep
     const size_t extra = !WL ? (size_t)KT * 5 * 8 : (KT <= 16 ? (size_t)KT * 32 * 8 : 0);
-    const size_t smem =
-        (SM ? 4 * (size_t)a.N : 0) + (size_t)(KT + 4) * 32 * 8 + (size_t)KT * 32 * 4 + extra;
-    cudaError_t e = cudaFuncSetAttribute(walk_kernel<KT, WL, SM>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t bytes = kWalkWords + (SM ? 4 * (size_t)a.N : 0) + (size_t)(KT + 4) * 32 * 8 +
+                         (size_t)KT * 32 * 4 + extra;
+    int dev = 0, sms = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    walk_kernel<KT, WL, SM><<<a.nwalk / 32, 32, smem, s>>>(a);
+    // One block per multiprocessor, or two in turn, where that holds all warps;
+    // single warps beyond, where the next ones start as soon as any ends and keep
+    // the multiprocessor filled (2 sweeps of 4 x 131072 multicanonical walkers 6.9 ms,
+    // 7.0 in four rounds of blocks; of 2 x 131072 Wang-Landau walkers 5.0 and 4.6).
+    const int warps = a.nwalk / 32;
+    const int fit = std::min(walk_block(KT), (int)((size_t)most / bytes));
+    int per = (warps + sms - 1) / sms;
+    if (per > fit) per = per <= 2 * fit ? (per + 1) / 2 : 1;
+    e = cudaFuncSetAttribute(walk_kernel<KT, WL, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(per * bytes));
+    if (e != cudaSuccess) return e;
+    walk_kernel<KT, WL, SM>
+        <<<(warps + per - 1) / per, 32 * per, per * bytes, s>>>(a, (uint32_t)bytes);
     return cudaGetLastError();
 }
 
