@@ -36,10 +36,18 @@ struct PairMeta {
 
 // A queue entry: `count` samples of side L (class_samples[first ...]) run
 // side by side, one per sub-group of blockDim / k threads, `stride` bytes of
-// shared memory each.
+// shared memory each, through the sweeps from c0 / kCuts to c1 / kCuts of the
+// run; `next` is the entry with the pack's following sweeps (-1: none), `pred`
+// whether there is one with its earlier sweeps.
+constexpr int kCuts = 6;
+
 struct WorkItem {
-    int first, count, L, k, stride;
+    int first, stride, next;
+    uint8_t count, L, k, c0, c1, pred;
+    uint16_t unused;
 };
+constexpr int kSplitSweeps = 4;  // runs of fewer sweeps are not worth cutting
+static_assert(sizeof(WorkItem) == 20, "the queue's room is counted in 20-byte entries");
 
 struct BatchArgs {
     uint32_t* spins;
@@ -49,6 +57,7 @@ struct BatchArgs {
     const WorkItem* items;      // the work queue
     int nitems;
     unsigned* counter;          // next queue entry
+    unsigned* arrive;           // per entry with a predecessor: see ea_pt_persistent
     const long long* word_off;  // per sample: first spin word (colour 0), colour 1 at + H
     int d, ntemps;
     uint32_t sample0;  // global index of sample 0 (Philox counters use global indices)
@@ -134,12 +143,12 @@ __device__ __forceinline__ void group_sync(int bar, int nthr)
     else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthr) : "memory");
 }
 
-// All sweeps of one sample by a sub-group of nthr threads (local index tid)
+// Sweeps step0 .. step1 - 1 of one sample by a sub-group of nthr threads (local index tid)
 // whose shared memory starts at base; the sample's couplings and the spins of
-// all its replicas stay in shared memory for the whole run.
+// all its replicas stay in shared memory meanwhile.
 template <int D>
 __device__ void run_sample(const BatchArgs& a, int s, int L, unsigned char* base, int tid,
-                           int nthr, int bar)
+                           int nthr, int bar, int step0, int step1)
 {
     uint4* smem_u4 = reinterpret_cast<uint4*>(base);
     const int nt = a.ntemps;
@@ -167,12 +176,12 @@ __device__ void run_sample(const BatchArgs& a, int s, int L, unsigned char* base
     // load the sample
     const long long w0 = a.word_off[s];
     for (int q = tid; q < 2 * H; q += nthr) {
-        S0[q] = a.spins[w0 + q];
+        S0[q] = __ldcg(a.spins + w0 + q);  // (may come from another multiprocessor)
         B0[q] = a.bonds[w0 + q];
     }
     if (tid < kMaxTemps) {
         unsat[tid] = 0;
-        sot[tid] = tid < nt ? a.perm[s * kMaxTemps + tid] : tid;
+        sot[tid] = tid < nt ? __ldcg(a.perm + s * kMaxTemps + tid) : tid;
     }
     group_sync(bar, nthr);
     // thresholds of temperature k and Philox parts of sweep tt for the slot r that
@@ -184,10 +193,10 @@ __device__ void run_sample(const BatchArgs& a, int s, int L, unsigned char* base
         thr_slot[r] = make_uint4(~th.x, ~th.y, ~th.z, pg.w2);
         ph_slot[r] = make_uint2(pg.x2, pg.z2);
     };
-    if (tid < nt) set_slot(tid, sot[tid], a.t0);
+    if (tid < nt) set_slot(tid, sot[tid], a.t0 + step0);
     group_sync(bar, nthr);
 
-    for (int step = 0; step < a.nsweeps; ++step) {
+    for (int step = step0; step < step1; ++step) {
         const long long t = a.t0 + step;
         uint32_t cnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         for (int c = 0; c < 2; ++c) {
@@ -347,27 +356,56 @@ __device__ void run_sample(const BatchArgs& a, int s, int L, unsigned char* base
     if (tid < nt) a.perm[s * kMaxTemps + tid] = sot[tid];
 }
 
-// One persistent launch for the whole batch: every CTA takes work items
-// (packs of k samples of one size, k sub-groups of blockDim / k threads, each
-// with its own named barrier and shared-memory slice) from a queue ordered
-// largest first, until the queue is empty.
+// One persistent launch for the whole batch: every CTA takes entries (packs of k
+// samples of one size, k sub-groups of blockDim / k threads, each with its own
+// named barrier and shared-memory slice) from a queue until it is empty.
+//
+// Samples of very different cost do not divide evenly over the CTAs: 103 of side
+// 32, 102 of side 24 and 307 smaller ones kept 152 CTAs busy for 3.26 ms per 20
+// sweeps where the work, spread evenly, takes 2.8.  So packs are cut by sweeps
+// (plan_pieces orders the pieces).  No CTA ever waits: a piece with a predecessor
+// belongs to whoever comes second, the CTA that takes it from the queue or the one
+// that finishes the predecessor; the first to come leaves it to the other.  That
+// takes 2.91 ms (4 sweeps 0.64, whole packs 0.68), with 4 cuts 3.01, with 8 2.92 and
+// with 20 2.87, where runs of fewer sweeps lose as much as they gain.
+__device__ __forceinline__ bool comes_second(const BatchArgs& a, int it)
+{
+    __threadfence();  // the predecessor's results before the arrival
+    if (atomicAdd(a.arrive + it, 1u) == 0u) return false;
+    a.arrive[it] = 0u;  // for the next run
+    __threadfence();
+    return true;
+}
+
 template <int D>
 __global__ void __launch_bounds__(1024) ea_pt_persistent(const BatchArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int item;
+    int go_on = -1;  // (thread 0) the entry that follows the one just finished
     while (true) {
-        if (threadIdx.x == 0) item = (int)atomicAdd(a.counter, 1u);
+        if (threadIdx.x == 0) {
+            int it = go_on;
+            while (it < 0) {
+                it = (int)atomicAdd(a.counter, 1u);
+                if (it >= a.nitems) break;
+                if (a.items[it].pred && !comes_second(a, it)) it = -1;
+            }
+            item = it;
+        }
         __syncthreads();
         const int it = item;
         if (it >= a.nitems) break;
         const WorkItem w = a.items[it];
         const int nthr = blockDim.x / w.k;
         const int g = threadIdx.x / nthr;
-        if (g < w.count)
+        const int step0 = (int)((long long)a.nsweeps * w.c0 / kCuts);
+        const int step1 = (int)((long long)a.nsweeps * w.c1 / kCuts);
+        if (g < w.count && step0 < step1)
             run_sample<D>(a, a.class_samples[w.first + g], w.L, smem_raw + (size_t)g * w.stride,
-                          threadIdx.x - g * nthr, nthr, w.k == 1 ? 0 : g + 1);
+                          threadIdx.x - g * nthr, nthr, w.k == 1 ? 0 : g + 1, step0, step1);
         __syncthreads();
+        if (threadIdx.x == 0) go_on = w.next >= 0 && comes_second(a, w.next) ? w.next : -1;
     }
 }
 
@@ -491,6 +529,12 @@ struct sl_batch {
     std::vector<double> class_cost;  // measured SM-milliseconds per sample-sweep (0: untimed)
     int nitems, grid;
     size_t smem_dyn;
+    // the queue of pieces for runs of kSplitSweeps and more (nsplit 0: none)
+    WorkItem* split_dev;
+    unsigned* arrive;
+    int nsplit, split_grid;
+    size_t split_smem;
+    std::vector<std::vector<double>> pack_ms;  // per class, per log2 k: a pack's sweep (-1)
     int autotune, force_k, tuned;
     cudaStream_t cap_stream;
     cudaGraph_t graph_def;       // kept alive: kernel_node belongs to it
@@ -628,10 +672,15 @@ void class_items(const sl_batch* b, int ci, int k, std::vector<WorkItem>& items)
     for (int q = 0; q < n; q += k) {
         WorkItem w;
         w.first = b->class_dev_off[ci] + q;
-        w.count = std::min(k, n - q);
-        w.L = b->class_L[ci];
-        w.k = k;
-        w.stride = (int)pack_stride(b->d, w.L);
+        w.count = (uint8_t)std::min(k, n - q);
+        w.L = (uint8_t)b->class_L[ci];
+        w.k = (uint8_t)k;
+        w.stride = (int)pack_stride(b->d, b->class_L[ci]);
+        w.c0 = 0;
+        w.c1 = kCuts;
+        w.pred = 0;
+        w.unused = 0;
+        w.next = -1;
         items.push_back(w);
     }
 }
@@ -639,8 +688,11 @@ void class_items(const sl_batch* b, int ci, int k, std::vector<WorkItem>& items)
 template <int D>
 cudaError_t launch_persistent(const BatchArgs& a, int grid, size_t smem, cudaStream_t st)
 {
+    // (one limit for every queue of every batch, whichever was set up last)
+    const int most = dev_attr(cudaDevAttrMaxSharedMemoryPerBlockOptin, 227 * 1024) - 1024;
     cudaError_t e = cudaFuncSetAttribute(ea_pt_persistent<D>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         std::max(most, (int)smem));
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
@@ -664,6 +716,7 @@ BatchArgs base_args(const sl_batch* b)
     a.class_samples = b->class_dev;
     a.items = b->items_dev;
     a.counter = b->counter;
+    a.arrive = b->arrive;
     a.d = b->d;
     a.ntemps = b->ntemps;
     a.sample0 = b->sample0;
@@ -783,6 +836,7 @@ int autotune(sl_batch* b)
             b->class_cost[ci] = item_ms[ci][lk] / best_ks[ci];  // ms per sample-sweep on one CTA
         }
     }
+    if (e == cudaSuccess) b->pack_ms = item_ms;
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (e == cudaSuccess)
@@ -793,6 +847,125 @@ int autotune(sl_batch* b)
                             cudaMemcpyDeviceToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     return e == cudaSuccess ? SL_OK : cuda_fail(e, "batch autotune");
+}
+
+// The pieces of packs that cost `cost` each, in the order in which m CTAs start them
+// when each, a sixth of a pack done, goes on with the pack that has the most work
+// left; returns the time at which the last one ends.
+struct Piece {
+    int pack, c0, c1;
+};
+
+double plan_pieces(const std::vector<double>& cost, int m, std::vector<Piece>& pieces)
+{
+    typedef std::pair<double, int> Entry;  // (work left, -pack), (-time, piece)
+    std::vector<Entry> waiting, running;
+    auto push = [](std::vector<Entry>& h, Entry x) {
+        h.push_back(x);
+        std::push_heap(h.begin(), h.end());
+    };
+    auto pop = [](std::vector<Entry>& h) {
+        std::pop_heap(h.begin(), h.end());
+        const Entry x = h.back();
+        h.pop_back();
+        return x;
+    };
+    std::vector<int> done(cost.size(), 0);
+    for (size_t q = 0; q < cost.size(); ++q) push(waiting, Entry(cost[q], -(int)q));
+    pieces.clear();
+    auto start = [&](double t) {
+        if (waiting.empty()) return;
+        const int p = -pop(waiting).second;
+        pieces.push_back(Piece{p, done[p], done[p] + 1});
+        push(running, Entry(-(t + cost[p] / kCuts), (int)pieces.size() - 1));
+    };
+    for (int c = 0; c < m; ++c) start(0.0);
+    double end = 0.0;
+    while (!running.empty()) {
+        const Entry e = pop(running);
+        Piece& x = pieces[e.second];
+        const int p = x.pack;
+        end = -e.first;
+        done[p] = x.c1;
+        const double left = cost[p] * (kCuts - done[p]) / kCuts;
+        if (done[p] == kCuts) {
+            start(end);
+        } else if (!waiting.empty() && waiting.front().first > left) {
+            start(end);
+            push(waiting, Entry(left, -p));
+        } else {
+            x.c1 = done[p] + 1;
+            push(running, Entry(-(end + cost[p] / kCuts), e.second));
+        }
+    }
+    return end;
+}
+
+// The queue of pieces, where it ends earlier than the queue of whole packs.  It is
+// kept where the tuner's copy of the spins was, which is needed no more.
+cudaError_t build_split(sl_batch* b, int nsm, double whole)
+{
+    b->nsplit = 0;
+    const int nc = (int)b->class_L.size();
+    if ((int)b->pack_ms.size() != nc || b->force_k > 0) return cudaSuccess;
+    // packs as cheap per sample as can be, unless one alone takes longer than the rest
+    std::vector<int> lks(nc, 0), best(nc, 0);
+    double best_end = 1e300, best_sum = 1e300;
+    std::function<void(int, double, double)> rec = [&](int ci, double sum, double most) {
+        if (ci == nc) {
+            const double e = std::max(sum / nsm, most);
+            if (e < best_end || (e == best_end && sum < best_sum)) {
+                best_end = e;
+                best_sum = sum;
+                best = lks;
+            }
+            return;
+        }
+        for (int lk = 0; lk < 4; ++lk) {
+            const double ms = b->pack_ms[ci][lk];
+            if (ms < 0.0) continue;
+            lks[ci] = lk;
+            const int n = ((int)b->class_ids[ci].size() + (1 << lk) - 1) >> lk;
+            rec(ci + 1, sum + n * ms, std::max(most, ms));
+        }
+    };
+    rec(0, 0.0, 0.0);
+    if (!(best_end < 0.97 * whole)) return cudaSuccess;
+    std::vector<WorkItem> packs;
+    std::vector<double> cost;
+    size_t smem = 0;
+    for (int ci = 0; ci < nc; ++ci) {
+        class_items(b, ci, 1 << best[ci], packs);
+        cost.resize(packs.size(), b->pack_ms[ci][best[ci]]);
+        smem = std::max(smem, ((size_t)1 << best[ci]) * pack_stride(b->d, b->class_L[ci]));
+    }
+    std::vector<Piece> pieces;
+    if (!(plan_pieces(cost, nsm, pieces) < 0.97 * whole)) return cudaSuccess;
+    const size_t n = pieces.size();
+    if (align_up(n * sizeof(WorkItem)) + n * sizeof(unsigned) > (size_t)b->total_words * 4)
+        return cudaSuccess;
+    std::vector<WorkItem> queue(n);
+    std::vector<int> last(packs.size(), -1);
+    for (size_t q = 0; q < n; ++q) {
+        const Piece& x = pieces[q];
+        queue[q] = packs[x.pack];
+        queue[q].c0 = (uint8_t)x.c0;
+        queue[q].c1 = (uint8_t)x.c1;
+        queue[q].pred = x.c0 > 0;
+        if (last[x.pack] >= 0) queue[last[x.pack]].next = (int)q;
+        last[x.pack] = (int)q;
+    }
+    b->split_dev = (WorkItem*)b->backup_spins;
+    b->arrive = (unsigned*)((char*)b->backup_spins + align_up(n * sizeof(WorkItem)));
+    cudaError_t e = cudaMemcpyAsync(b->split_dev, queue.data(), n * sizeof(WorkItem),
+                                    cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->arrive, 0, n * sizeof(unsigned), b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return e;
+    b->split_grid = std::min((int)n, nsm);
+    b->split_smem = smem;
+    b->nsplit = (int)n;
+    return cudaSuccess;
 }
 
 // Work queue from the chosen pack sizes, most expensive packs first, and the
@@ -832,6 +1005,11 @@ int build_queue(sl_batch* b)
     cudaError_t e = cudaMemcpyAsync(b->items_dev, sorted.data(), sorted.size() * sizeof(WorkItem),
                                     cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e == cudaSuccess) {
+        std::vector<int> ks(nc);
+        for (int ci = 0; ci < nc; ++ci) ks[ci] = b->class_k[ci];
+        e = build_split(b, nsm, b->pack_ms.empty() ? 0.0 : simulate(b, ks, b->pack_ms, nsm));
+    }
     if (e != cudaSuccess) return cuda_fail(e, "batch work queue");
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
@@ -949,6 +1127,9 @@ int sl_batch_create(int d, const int* L_per_sample, int nsamples, int ntemps, co
     b->counter = (unsigned*)(base + y.off_counter);
     b->backup_spins = (uint32_t*)(base + y.off_backup);
     b->backup_perm = (int32_t*)(base + y.off_backup_perm);
+    b->split_dev = nullptr;
+    b->arrive = nullptr;
+    b->nsplit = 0;
     b->nitems = 0;
     b->grid = 0;
     b->smem_dyn = 0;
@@ -1044,7 +1225,9 @@ int sl_batch_run(sl_batch* b, int64_t nsweeps, uint64_t seed, double* dev_E)
         b->tuned = 1;
     }
     BatchArgs a = base_args(b);
-    a.nitems = b->nitems;
+    const bool split = b->nsplit > 0 && nsweeps >= kSplitSweeps;
+    if (split) a.items = b->split_dev;
+    a.nitems = split ? b->nsplit : b->nitems;
     a.t0 = b->sweeps_done;
     a.nsweeps = (int)nsweeps;
     a.rk = make_round_keys(seed);
@@ -1053,9 +1236,9 @@ int sl_batch_run(sl_batch* b, int64_t nsweeps, uint64_t seed, double* dev_E)
     cudaKernelNodeParams kp = {};
     void* args[1] = {&a};
     kp.func = b->d == 3 ? (void*)ea_pt_persistent<3> : (void*)ea_pt_persistent<2>;
-    kp.gridDim = dim3((unsigned)b->grid);
+    kp.gridDim = dim3((unsigned)(split ? b->split_grid : b->grid));
     kp.blockDim = dim3(1024);
-    kp.sharedMemBytes = (unsigned)b->smem_dyn;
+    kp.sharedMemBytes = (unsigned)(split ? b->split_smem : b->smem_dyn);
     kp.kernelParams = args;
     kp.extra = nullptr;
     cudaError_t e = cudaGraphExecKernelNodeSetParams(b->graph, b->kernel_node, &kp);
