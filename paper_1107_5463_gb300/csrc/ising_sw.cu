@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kSwThreads2, 8) sw_local2(const SwArgs a)
     uint32_t hx = 0u;  // bit k: the spin after the last of the warp's row k
 #pragma unroll
     for (int k = 0; k < RPW; ++k) {
-        const int ly = warp + NW * k;
+        const int ly = RPW * warp + k;
         if (ly >= ny) continue;  // uniform across the warp
         load_row(ly);
         const uint32_t y = (uint32_t)(Y0 + ly), x = (uint32_t)(X0 + nx) == L ? 0u : (uint32_t)(X0 + nx);
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kSwThreads2, 8) sw_local2(const SwArgs a)
         uint4 rnd[RPW];
 #pragma unroll
         for (int k = 0; k < RPW; ++k)
-            rnd[k] = philox_at(pg, ((uint32_t)(X0 + lx0) + L * (uint32_t)(Y0 + warp + NW * k)) >> 1,
+            rnd[k] = philox_at(pg, ((uint32_t)(X0 + lx0) + L * (uint32_t)(Y0 + RPW * warp + k)) >> 1,
                                a.rk);
         const uint32_t may = a.never ? 0u : valid;
 #pragma unroll
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kSwThreads2, 8) sw_local2(const SwArgs a)
     const uint32_t flipw = a.anti ? 0u : kAll;  // like spins satisfy a bond, or unlike ones
 #pragma unroll
     for (int k = 0; k < RPW; ++k) {
-        const int ly = warp + NW * k;
+        const int ly = RPW * warp + k;
         if (ly >= ny) {
             ay0[k] = ay1[k] = ax0[k] = ax1[k] = 0u;
             continue;
@@ -328,10 +328,14 @@ __global__ void __launch_bounds__(kSwThreads2, 8) sw_local2(const SwArgs a)
     // The runs are joined along y.  A bond is left out when the two runs are
     // joined by a bond further left already: c0, c1 mark the even and odd sites
     // whose left neighbour is joined to its lower one, in both rows to the site.
-    unsigned n = 0;
+    // First come the bonds within the warp's rows (within pairs of rows, then
+    // between the pairs), then those to the next warp's.
+    unsigned n = 0, inner = 0;
 #pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-        const int ly = warp + NW * k;
+    for (int kk = 0; kk < RPW; ++kk) {
+        const int k = kk == 1 ? 2 : kk == 2 ? 1 : kk;
+        const int ly = RPW * warp + k;
+        if (k == RPW - 1) inner = n;
         if (ly + 1 >= ny) continue;
         const uint32_t r0 = ax0[k] & bx0[ly + 1], r1 = (ax1[k] & bx1[ly + 1]) << 1;
         uint32_t c0 = 0u, c1 = 0u;
@@ -348,29 +352,38 @@ __global__ void __launch_bounds__(kSwThreads2, 8) sw_local2(const SwArgs a)
     // an atomic minimum; if another link got there first, what it linked to is
     // still to be joined to the smaller root.  Parents only ever point to smaller
     // indices, so the root of every tile cluster ends as its smallest site whatever
-    // order the unions run in.  (Measured for the whole kernel up to here at L =
-    // 4096, critical point: compare-and-swap with both finds repeated 171 us,
-    // atomic minimum 163, Rem's interleaved splicing 161 but dearer jumps after it;
-    // finds without halving 1.4 times the whole kernel.)
+    // order the unions run in; but the order decides how long the paths grow.  A warp
+    // has four rows that follow each other and joins them before any warp joins its
+    // rows to the next one's: the whole update took 995 us at L = 8192 with every
+    // eighth row to a warp, 886 with four rows on end, 870 with the barrier.
+    // (Measured for the whole kernel up to here at L = 4096, critical point, every
+    // eighth row: compare-and-swap with both finds repeated 171 us, atomic minimum
+    // 163, Rem's interleaved splicing 161 but dearer jumps after it; finds without
+    // halving 1.4 times the whole kernel.)
     volatile uint32_t* vp = par;
-    for (unsigned q = lane; q < n; q += 32) {
-        const uint32_t u = list[warp][q];
-        uint32_t ra = sfind(vp, u), rb = sfind(vp, u + (uint32_t)TX);
-        while (ra != rb) {
-            const uint32_t hi = max(ra, rb), lo = min(ra, rb);
-            const uint32_t old = atomicMin(par + hi, lo);
-            if (old == hi) break;
-            ra = sfind(vp, old);
-            rb = lo;
+    auto unite = [&](unsigned q, unsigned end) {
+        for (; q < end; q += 32) {
+            const uint32_t u = list[warp][q];
+            uint32_t ra = sfind(vp, u), rb = sfind(vp, u + (uint32_t)TX);
+            while (ra != rb) {
+                const uint32_t hi = max(ra, rb), lo = min(ra, rb);
+                const uint32_t old = atomicMin(par + hi, lo);
+                if (old == hi) break;
+                ra = sfind(vp, old);
+                rb = lo;
+            }
         }
-    }
+    };
+    unite(lane, inner);
+    __syncthreads();
+    unite(inner + lane, n);
     // the run heads, listed in the same place, jump to their roots; every other
     // site's label is read through its head
     __syncwarp();
     unsigned nh = 0;
 #pragma unroll
     for (int k = 0; k < RPW; ++k) {
-        const int ly = warp + NW * k;
+        const int ly = RPW * warp + k;
         if (ly < ny) put(~(ax1[k] << 1) & valid, ~ax0[k] & valid, ly, nh);
     }
     __syncthreads();
@@ -393,7 +406,7 @@ __global__ void __launch_bounds__(kSwThreads2, 8) sw_local2(const SwArgs a)
     unsigned cnt = 0;
 #pragma unroll
     for (int k = 0; k < RPW; ++k) {
-        const int ly = warp + NW * k;
+        const int ly = RPW * warp + k;
         m0[k] = m1[k] = 0u;
         if (ly >= ny) continue;
         const uint32_t l = (uint32_t)(TX * ly + lx0);
@@ -419,7 +432,7 @@ __global__ void __launch_bounds__(kSwThreads2, 8) sw_local2(const SwArgs a)
     pos = blk_base + __shfl_sync(kAll, pos, 0);
 #pragma unroll
     for (int k = 0; k < RPW; ++k) {
-        const uint32_t i = i00 + L * (uint32_t)(warp + NW * k) + lx0;
+        const uint32_t i = i00 + L * (uint32_t)(RPW * warp + k) + lx0;
         if (m0[k] >> lane & 1u) a.roots[pos + __popc(m0[k] & below)] = i;
         pos += __popc(m0[k]);
         if (m1[k] >> lane & 1u) a.roots[pos + __popc(m1[k] & below)] = i + 1;
