@@ -161,25 +161,6 @@ __device__ __forceinline__ void tile_origin(const SwArgs& a, int bx, int by, int
     nz = D == 3 ? min(TZ, a.L - Z0) : 1;
 }
 
-// position of the q-th (from 0) set bit of m; q < popc(m)
-__device__ __forceinline__ int nth_set_bit(uint32_t m, int q)
-{
-    int pos = 0;
-#pragma unroll
-    for (int w = 16; w > 0; w >>= 1) {
-        const uint32_t low = m & ((1u << w) - 1u);
-        const int c = __popc(low);
-        if (q >= c) {
-            q -= c;
-            m >>= w;
-            pos += w;
-        } else {
-            m = low;
-        }
-    }
-    return pos;
-}
-
 // root of x in the shared parent array, halving the path on the way (a
 // halving store only ever replaces a non-root's parent by an ancestor)
 __device__ __forceinline__ uint32_t sfind(volatile uint32_t* par, uint32_t x)
@@ -193,11 +174,6 @@ __device__ __forceinline__ uint32_t sfind(volatile uint32_t* par, uint32_t x)
         p = par[x];
     }
     return x;
-}
-
-__device__ __forceinline__ bool bond_active(const SwArgs& a, uint8_t s0, uint8_t s1, uint32_t u)
-{
-    return (int)(s0 ^ s1) == a.anti && !a.never && u <= a.thr;
 }
 
 // 2D tiles of 64 x 32 sites.  A row of the tile is two words, the even and the
@@ -440,295 +416,234 @@ __global__ void __launch_bounds__(kSwThreads2, 8) sw_local2(const SwArgs a)
     }
 }
 
-// 3D tiles of 64 x 16 x 8 sites.
+// 3D tiles of 64 x 16 x 8 sites, by words as in 2D: a warp has eight rows on end,
+// half of a plane.  It joins them along y first; then the rows are joined to the next
+// warp's and along z.  (A lane deciding its own sites' bonds from bytes and uniting
+// them one after another, every sixteenth row to a warp: an update at L = 256 took 450
+// us at the critical point, 497 at beta = 0.4 and 405 at 0.15, now 428, 466 and 406;
+// L = 100 98 and 89.  Issue bound; 2 and 4 blocks a multiprocessor: 462 and 423 at L =
+// 256, 87 and 90 at L = 100.)
 __global__ void __launch_bounds__(kSwThreads, 3) sw_local3(const SwArgs a)
 {
-    constexpr int D = 3;
-    constexpr int TX = SwTile<D>::TX, TY = SwTile<D>::TY, TZ = SwTile<D>::TZ;
-    static_assert(TX == 64, "one warp lane per site pair of a 64-site row");
-    constexpr int NS = TX * TY * TZ;
-    constexpr int HX = TX + 2, HY = TY + 1, HZ = TZ + 1;  // halo-padded spin tile
-    constexpr int WORDS = SwFace<D>::WORDS;
-    constexpr int NW = kSwThreads / 32;
-    constexpr int ROWS = TY * TZ;
-    constexpr int RPW = ROWS / NW;  // rows per warp
-    __shared__ uint32_t par[NS];
-    __shared__ uint8_t sp[HZ * HY * HX];
+    constexpr int TX = SwTile<3>::TX, TY = SwTile<3>::TY, TZ = SwTile<3>::TZ;
+    constexpr int HY = TY + 1, HZ = TZ + 1;  // rows with those after the tile
+    constexpr int WORDS = SwFace<3>::WORDS;
+    constexpr int NW = kSwThreads / 32, ROWS = TY * TZ, RPW = ROWS / NW;
+    constexpr uint32_t kAll = 0xFFFFFFFFu;
+    static_assert(TX == 64 && RPW == 8 && TY % RPW == 0, "rows of a warp");
+    __shared__ __align__(8) uint32_t par[TX * ROWS];
+    __shared__ uint32_t rowE[HZ * HY], rowO[HZ * HY];  // spins of even and odd sites
+    __shared__ uint32_t bx[2][ROWS], by[2][ROWS], bz[2][ROWS];  // active bonds in the tile
     __shared__ uint32_t fm[WORDS];
-    // per row, per lane bit: active in-tile bonds of the lane's even (0) and
-    // odd (1) site along +x, +y and +z
-    __shared__ uint32_t bx[2][ROWS], by[2][ROWS], bz[2][ROWS];
+    __shared__ uint16_t list[NW][5 * TX];
+    __shared__ unsigned blk_count, blk_base;
 
-    const size_t b = blockIdx.x + gridDim.x * (blockIdx.y + (size_t)gridDim.y * blockIdx.z);
+    const size_t tile = blockIdx.x + gridDim.x * (blockIdx.y + (size_t)gridDim.y * blockIdx.z);
     int X0, Y0, Z0, nx, ny, nz;
-    tile_origin<D>(a, blockIdx.x, blockIdx.y, blockIdx.z, X0, Y0, Z0, nx, ny, nz);
+    tile_origin<3>(a, blockIdx.x, blockIdx.y, blockIdx.z, X0, Y0, Z0, nx, ny, nz);
     const uint32_t L = (uint32_t)a.L;
     const uint32_t t = (uint32_t)a.ctrl->t;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int lx0 = 2 * lane;
-    const bool ex = lx0 < nx;  // the lane's site pair lies in the tile
+    const int lx0 = 2 * lane, last = (nx >> 1) - 1;  // the lane's pair; lane of the last pair
+    const uint32_t valid = kAll >> (31 - last), below = (1u << lane) - 1u;
+    const bool ex = lane <= last;
+    const int row0 = RPW * warp, ly0 = row0 % TY, lz = row0 / TY;  // the warp's first row
+    // the rows of the warp that lie in the tile
+    const int rows = lz >= nz || ly0 >= ny ? 0 : min(RPW, ny - ly0);
+    const uint32_t zb = L * (L * (uint32_t)(Z0 + lz) + (uint32_t)(Y0 + ly0));  // its row's first site
 
-    for (int w = threadIdx.x; w < WORDS; w += blockDim.x) fm[w] = 0u;
-    // the tile's rows plus the +y row and +z plane (one warp per row), and
-    // the +x column
-    for (int r = warp; r < HY * HZ; r += NW) {
-        const int ly = r % HY, lz = r / HY;
-        if (ly > ny || lz > nz) continue;
-        const bool hy = ly == ny, hz = lz == nz;
-        if (hy && hz) continue;
-        const uint32_t y = (uint32_t)(Y0 + ly) == L ? 0u : (uint32_t)(Y0 + ly);
-        const uint32_t z = (uint32_t)(Z0 + lz) == L ? 0u : (uint32_t)(Z0 + lz);
-        const uint32_t rowbase = L * (y + L * z);
-        const int ce = (int)((y + z) & 1u);  // colour of the even-x sites
-        uint8_t* dst = sp + (lz * HY + ly) * HX;
-        if (ex) {
-            const uint32_t j = (rowbase + (uint32_t)(X0 + lx0)) >> 1;
-            dst[lx0] = (uint8_t)a.s[ce][j];
-            dst[lx0 + 1] = (uint8_t)a.s[ce ^ 1][j];
-        }
-        if (lane == 0 && !hy && !hz) {
-            const uint32_t x = (uint32_t)(X0 + nx) == L ? 0u : (uint32_t)(X0 + nx);
-            dst[nx] = (uint8_t)a.s[(x + y + z) & 1u][(rowbase + x) >> 1];
-        }
-    }
-    __syncthreads();
-
-    // Bond activation, one warp per row.  A row splits into x-runs of sites
-    // joined by active bonds; every site's parent becomes the first site of
-    // its run, found from the warp's ballots.  Bonds leaving the tile set
-    // their face bit.
-#pragma unroll
-    for (int k = 0; k < RPW; ++k) {
-        const int row = warp + NW * k;
-        const int ly = row % TY, lz = row / TY;
-        if (ly >= ny || lz >= nz) continue;  // uniform across the warp
-        const int so = (lz * HY + ly) * HX + lx0;
-        bool xb0 = false, xb1 = false, yb[2] = {false, false}, zb[2] = {false, false};
-        if (ex) {
-            const uint32_t i0 = (uint32_t)(X0 + lx0) + L * ((uint32_t)(Y0 + ly) + L * (uint32_t)(Z0 + lz));
-            // uniforms of the x / y / z bonds of the even (e = 0) and odd site
-            const uint4 r0 = philox4x32_10(make_uint4(i0, t, a.replica, kSwBond << 1), a.rk);
-            const uint4 r1 = philox4x32_10(make_uint4(i0 + 1, t, a.replica, kSwBond << 1), a.rk);
-            const uint8_t s0 = sp[so], s1 = sp[so + 1], s2 = sp[so + 2];
-            xb0 = bond_active(a, s0, s1, r0.x);
-            xb1 = bond_active(a, s1, s2, r1.x);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const uint8_t own = e ? s1 : s0;
-                const int lx = lx0 + e;
-                const uint4 re = e ? r1 : r0;
-                if (bond_active(a, own, sp[so + e + HX], re.y)) {
-                    if (ly + 1 == ny) {
-                        const int bit = TY * TZ + lx + TX * lz;
-                        atomicOr(&fm[bit >> 5], 1u << (bit & 31));
-                    } else {
-                        yb[e] = true;
-                    }
-                }
-                if (bond_active(a, own, sp[so + e + HX * HY], re.z)) {
-                    if (lz + 1 == nz) {
-                        const int bit = TY * TZ + TX * TZ + lx + TX * ly;
-                        atomicOr(&fm[bit >> 5], 1u << (bit & 31));
-                    } else {
-                        zb[e] = true;
-                    }
-                }
-            }
-        }
-        const bool xcross = xb1 && lx0 + 2 == nx;
-        if (xcross) {
-            const int bit = ly + TY * lz;
-            atomicOr(&fm[bit >> 5], 1u << (bit & 31));
-        }
-        const uint32_t B0 = __ballot_sync(0xFFFFFFFFu, xb0);
-        const uint32_t B1 = __ballot_sync(0xFFFFFFFFu, xb1 && !xcross);
-        const uint32_t Y0b = __ballot_sync(0xFFFFFFFFu, yb[0]);
-        const uint32_t Y1b = __ballot_sync(0xFFFFFFFFu, yb[1]);
-        const uint32_t Z0b = __ballot_sync(0xFFFFFFFFu, zb[0]);
-        const uint32_t Z1b = __ballot_sync(0xFFFFFFFFu, zb[1]);
-        if (lane == 0) {
-            bx[0][row] = B0;
-            bx[1][row] = B1;
-            by[0][row] = Y0b;
-            by[1][row] = Y1b;
-            bz[0][row] = Z0b;
-            bz[1][row] = Z1b;
-        }
-        if (ex) {
-            // run starts: the even site starts a run unless the bond from the
-            // previous lane's odd site is active, the odd site unless xb0 is
-            const uint32_t R0 = ~(B1 << 1);
-            const uint32_t R1 = ~B0;
-            int rs0 = 2 * (31 - __clz(R0 & ((2u << lane) - 1u)));
-            const uint32_t m1 = R1 & ((1u << lane) - 1u);
-            if (m1) rs0 = max(rs0, 2 * (31 - __clz(m1)) + 1);
-            const int rs1 = xb0 ? rs0 : lx0 + 1;
-            const int base = TX * (ly + TY * lz);
-            par[base + lx0] = (uint32_t)(base + rs0);
-            par[base + lx0 + 1] = (uint32_t)(base + rs1);
-        }
-    }
-    __syncthreads();
-
-    // The runs are joined along y and z by the active bonds between rows.  A
-    // bond is left out when the bond at x - 1 is active and x - 1, x are
-    // joined in both rows (the same two runs).
-    uint32_t pend = 0;  // bit (k, e, mu): y/z bond of row k, site e, direction mu
-    if (ex) {
-#pragma unroll
-        for (int k = 0; k < RPW; ++k) {
-            const int row = warp + NW * k;
-            const int ly = row % TY, lz = row / TY;
-            if (ly >= ny || lz >= nz) continue;
-#pragma unroll
-            for (int mu = 1; mu < D; ++mu) {
-                const int nrow = mu == 1 ? row + 1 : row + TY;
-                const uint32_t c0 = mu == 1 ? by[0][row] : bz[0][row];
-                const uint32_t c1 = mu == 1 ? by[1][row] : bz[1][row];
-                // even site 2k: its left neighbour is lane k-1's odd site
-                bool p0 = (c0 >> lane) & 1u;
-                if (p0 && lane > 0 && ((c1 >> (lane - 1)) & 1u) &&
-                    ((bx[1][row] >> (lane - 1)) & 1u) && ((bx[1][nrow] >> (lane - 1)) & 1u))
-                    p0 = false;
-                // odd site 2k+1: its left neighbour is lane k's even site
-                bool p1 = (c1 >> lane) & 1u;
-                if (p1 && ((c0 >> lane) & 1u) && ((bx[0][row] >> lane) & 1u) &&
-                    ((bx[0][nrow] >> lane) & 1u))
-                    p1 = false;
-                const int base = k * 2 * (D - 1) + (mu - 1);
-                if (p0) pend |= 1u << base;
-                if (p1) pend |= 1u << (base + (D - 1));
-            }
-        }
-    }
-    // Every parent is a run head (the first site of an x-run), so after the
-    // heads have jumped to their roots a label is read through the head (two
-    // steps); the heads are decided by the x-bond ballots.  Lane l takes the l-th
-    // and (l + 32)-th head of each of its rows.
-    uint32_t heads[RPW];  // per row two 16-bit sites, 0xFFFF = none
-    {
-        const uint32_t valid = nx >= 64 ? 0xFFFFFFFFu : ((1u << (nx >> 1)) - 1u);
-#pragma unroll
-        for (int k = 0; k < RPW; ++k) {
-            heads[k] = 0xFFFFFFFFu;
-            const int row = warp + NW * k;
-            const int ly = row % TY, lz = row / TY;
-            if (ly >= ny || lz >= nz) continue;
-            const uint32_t h0 = ~(bx[1][row] << 1) & valid;  // even sites starting a run
-            const uint32_t h1 = ~bx[0][row] & valid;         // odd sites starting a run
-            const unsigned n0 = __popc(h0);
-            const int n = (int)n0 + __popc(h1);
-            uint32_t w = 0;
-#pragma unroll
-            for (int slot = 0; slot < 2; ++slot) {
-                const int q = lane + 32 * slot;
-                uint32_t site = 0xFFFFu;
-                if (q < n)
-                    site = (uint32_t)(TX * row) +
-                           (q < (int)n0 ? 2u * (uint32_t)nth_set_bit(h0, q)
-                                        : 2u * (uint32_t)nth_set_bit(h1, q - (int)n0) + 1u);
-                w |= site << (16 * slot);
-            }
-            heads[k] = w;
-        }
-    }
-    // One union per remaining y/z bond, lock-free: find both roots (path
-    // halving), link the larger root below the smaller by compare-and-swap,
-    // retry from the new roots if another link got there first.  Parents only
-    // ever point to smaller indices and a root links only below a smaller
-    // root, so the root of every tile cluster ends as its smallest site
-    // whatever order the unions run in.  Then every head jumps to its root.
-    volatile uint32_t* vp = par;
-    auto unite = [&](uint32_t u, uint32_t v) {
-        uint32_t ra = sfind(vp, u), rb = sfind(vp, v);
-        while (ra != rb) {
-            const uint32_t hi = max(ra, rb), lo = min(ra, rb);
-            const uint32_t old = atomicCAS(par + hi, hi, lo);
-            if (old == hi) break;
-            ra = sfind(vp, old);
-            rb = sfind(vp, lo);
-        }
-    };
-    for (uint32_t bits = pend; bits; bits &= bits - 1) {
-        const int bit = __ffs(bits) - 1;
-        const int k = bit / (2 * (D - 1));
-        const int e = (bit / (D - 1)) & 1;
-        const int mu = 1 + bit % (D - 1);
-        const uint32_t u = (uint32_t)(lx0 + e + TX * (warp + NW * k));
-        unite(u, u + (mu == 1 ? (uint32_t)TX : (uint32_t)(TX * TY)));
-    }
-    __syncthreads();
-    auto jump = [&](uint32_t l) {
-        uint32_t p = vp[l];
-        while (true) {
-            const uint32_t g = vp[p];
-            if (g == p) break;
-            p = g;
-        }
-        vp[l] = p;
-    };
-#pragma unroll
-    for (int k = 0; k < RPW; ++k)
-#pragma unroll
-        for (int slot = 0; slot < 2; ++slot) {
-            const uint32_t l = (heads[k] >> (16 * slot)) & 0xFFFFu;
-            if (l != 0xFFFFu) jump(l);
-        }
-    __syncthreads();
-
-    // labels: the natural index of each site's tile root; tile roots marked
-    // and counted (bit 2k + e of `mine`)
-    uint32_t mine = 0;
-    if (ex) {
-#pragma unroll
-        for (int k = 0; k < RPW; ++k) {
-            const int row = warp + NW * k;
-            const int ly = row % TY, lz = row / TY;
-            if (ly >= ny || lz >= nz) continue;
-            const uint32_t l0 = (uint32_t)(lx0 + TX * row);
-            uint32_t w[2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const uint32_t m = vp[vp[l0 + e]];  // smallest site of the tile cluster
-                const uint32_t rx = m % TX, rrow = m / TX;
-                const uint32_t ry = rrow % TY, rz = rrow / TY;
-                w[e] = ((uint32_t)X0 + rx) + L * (((uint32_t)Y0 + ry) + L * ((uint32_t)Z0 + rz));
-                if (m == l0 + e) {
-                    w[e] |= kTileRoot;
-                    mine |= 1u << (2 * k + e);
-                }
-            }
-            const uint32_t i0 = (uint32_t)(X0 + lx0) + L * ((uint32_t)(Y0 + ly) + L * (uint32_t)(Z0 + lz));
-            *reinterpret_cast<uint2*>(a.lab + i0) = make_uint2(w[0], w[1]);
-        }
-    }
-    for (int w = threadIdx.x; w < WORDS; w += blockDim.x) a.face[b * WORDS + w] = fm[w];
-    // append the tile roots to the update's list: a warp scan of the counts,
-    // one shared atomic per warp, one global atomic per block
-    __shared__ unsigned blk_count, blk_base;
+    for (int w = threadIdx.x; w < WORDS; w += kSwThreads) fm[w] = 0u;
     if (threadIdx.x == 0) blk_count = 0;
+    // the tile's rows, the +y row and the +z plane (one warp per row)
+    for (int r = warp; r < HY * HZ; r += NW) {
+        const int hy = r % HY, hz = r / HY;
+        if (hy > ny || hz > nz || (hy == ny && hz == nz)) continue;
+        const uint32_t y = (uint32_t)(Y0 + hy) == L ? 0u : (uint32_t)(Y0 + hy);
+        const uint32_t z = (uint32_t)(Z0 + hz) == L ? 0u : (uint32_t)(Z0 + hz);
+        const int ce = (int)((y + z) & 1u);  // colour of the even-x sites
+        const uint32_t j = (L * (y + L * z) + (uint32_t)(X0 + lx0)) >> 1;
+        const int8_t ve = ex ? a.s[ce][j] : (int8_t)0, vo = ex ? a.s[ce ^ 1][j] : (int8_t)0;
+        const uint32_t E = __ballot_sync(kAll, ve != 0), O = __ballot_sync(kAll, vo != 0);
+        if (lane == 0) {
+            rowE[r] = E;
+            rowO[r] = O;
+        }
+    }
+    uint32_t hx = 0u;  // bit k: the spin after the last of the warp's row k
+    {
+        const uint32_t x = (uint32_t)(X0 + nx) == L ? 0u : (uint32_t)(X0 + nx);
+        for (int k = 0; k < rows; ++k)
+            hx |= (uint32_t)a.s[(x + (uint32_t)(Y0 + ly0 + k + Z0 + lz)) & 1u]
+                               [(zb + L * (uint32_t)k + x) >> 1] << k;
+    }
     __syncthreads();
+
+    // Active bonds, and every site's parent: the first site of its x-run.  Bonds that
+    // leave the tile go to its face words (even sites' word, odd sites' word).
+    {
+        const PhiloxGroups pg = philox_groups(t, a.replica, kSwBond << 1, a.rk);
+        const uint32_t may = a.never ? 0u : valid;
+        const uint32_t flipw = a.anti ? 0u : kAll;  // like spins satisfy a bond, or unlike ones
+        uint32_t fxw = 0u;
+#pragma unroll 2
+        for (int k = 0; k < rows; ++k) {
+            const int row = row0 + k, ly = ly0 + k, r = lz * HY + ly;
+            const uint32_t i0 = zb + L * (uint32_t)k + (uint32_t)(X0 + lx0);
+            const uint4 u0 = philox_at(pg, i0, a.rk), u1 = philox_at(pg, i0 + 1u, a.rk);
+            const uint32_t E = rowE[r], O = rowO[r];
+            const uint32_t x0 = __ballot_sync(kAll, u0.x <= a.thr) & may & (E ^ O ^ flipw);
+            uint32_t x1 = __ballot_sync(kAll, u1.x <= a.thr) & may &
+                          (O ^ ((E >> 1) | ((hx >> k & 1u) << last)) ^ flipw);
+            uint32_t y0 = __ballot_sync(kAll, u0.y <= a.thr) & may & (E ^ rowE[r + 1] ^ flipw);
+            uint32_t y1 = __ballot_sync(kAll, u1.y <= a.thr) & may & (O ^ rowO[r + 1] ^ flipw);
+            uint32_t z0 = __ballot_sync(kAll, u0.z <= a.thr) & may & (E ^ rowE[r + HY] ^ flipw);
+            uint32_t z1 = __ballot_sync(kAll, u1.z <= a.thr) & may & (O ^ rowO[r + HY] ^ flipw);
+            fxw |= (x1 >> last & 1u) << (row & 31);
+            x1 &= ~(1u << last);
+            if (ly + 1 == ny) {
+                if (lane < 2) fm[ROWS / 32 + 2 * lz + lane] = lane ? y1 : y0;
+                y0 = y1 = 0u;
+            }
+            if (lz + 1 == nz) {
+                if (lane < 2) fm[(ROWS + TX * TZ) / 32 + 2 * ly + lane] = lane ? z1 : z0;
+                z0 = z1 = 0u;
+            }
+            if (lane == 0) {
+                bx[0][row] = x0;
+                bx[1][row] = x1;
+                by[0][row] = y0;
+                by[1][row] = y1;
+                bz[0][row] = z0;
+                bz[1][row] = z1;
+            }
+            // run starts: the even site unless the bond from the previous lane's odd
+            // site is active, the odd site unless the pair's bond is
+            const uint32_t R0 = ~(x1 << 1), R1 = ~x0;
+            int rs0 = 2 * (31 - __clz(R0 & ((2u << lane) - 1u)));
+            const uint32_t m1 = R1 & below;
+            if (m1) rs0 = max(rs0, 2 * (31 - __clz(m1)) + 1);
+            const int rs1 = (x0 >> lane & 1u) ? rs0 : lx0 + 1;
+            *reinterpret_cast<uint2*>(&par[TX * row + lx0]) =
+                make_uint2((uint32_t)(TX * row + rs0), (uint32_t)(TX * row + rs1));
+        }
+        if (lane == 0 && fxw) atomicOr(&fm[row0 >> 5], fxw);
+    }
+    __syncthreads();
+
+    // place the sites of two masks (even, odd) of a row in the warp's list
+    auto put = [&](uint32_t m0, uint32_t m1, int row, unsigned& n) {
+        const unsigned n0 = __popc(m0);
+        if (m0 >> lane & 1u) list[warp][n + __popc(m0 & below)] = (uint16_t)(TX * row + lx0);
+        if (m1 >> lane & 1u)
+            list[warp][n + n0 + __popc(m1 & below)] = (uint16_t)(TX * row + lx0 + 1);
+        n += n0 + __popc(m1);
+    };
+    // the bonds w between the warp's row k and the one `step` rows on, without those
+    // whose two runs a bond further left has joined already (see sw_local2)
+    auto put_bonds = [&](const uint32_t (&w)[2][ROWS], int k, int step, unsigned& n) {
+        if (k >= rows) return;
+        const int row = row0 + k, next = min(row + step, ROWS - 1);
+        const uint32_t w0 = w[0][row], w1 = w[1][row];
+        const uint32_t r0 = bx[0][row] & bx[0][next], r1 = (bx[1][row] & bx[1][next]) << 1;
+        uint32_t c0 = 0u, c1 = 0u;
+#pragma unroll
+        for (int it = 0; it < 3; ++it) {
+            c1 = (w0 | c0) & r0;
+            c0 = (w1 | c1) << 1 & r1;
+        }
+        put(w0 & ~c0, w1 & ~c1, row, n);
+    };
+    // one union per listed bond, the first ny of them along y (see sw_local2)
+    volatile uint32_t* vp = par;
+    auto unite = [&](unsigned n, unsigned ny_) {
+        __syncwarp();
+        for (unsigned q = lane; q < n; q += 32) {
+            const uint32_t u = list[warp][q];
+            const uint32_t v = u + (uint32_t)(q < ny_ ? TX : TX * TY);
+            uint32_t ra = sfind(vp, u), rb = sfind(vp, v);
+            while (ra != rb) {
+                const uint32_t hi = max(ra, rb), lo = min(ra, rb);
+                const uint32_t old = atomicMin(par + hi, lo);
+                if (old == hi) break;
+                ra = sfind(vp, old);
+                rb = lo;
+            }
+        }
+        __syncwarp();
+    };
+    unsigned n = 0;
+    for (int k = 0; k < RPW; k += 2) put_bonds(by, k, 1, n);
+    unite(n, n);
+    n = 0;
+    for (int k = 1; k < RPW - 1; k += 2) put_bonds(by, k, 1, n);
+    unite(n, n);
+    __syncthreads();
+    n = 0;
+    put_bonds(by, RPW - 1, 1, n);
+    const unsigned along_y = n;
+    for (int k = 0; k < 4; ++k) put_bonds(bz, k, TY, n);
+    unite(n, along_y);
+    n = 0;
+    for (int k = 4; k < RPW; ++k) put_bonds(bz, k, TY, n);
+    unite(n, 0u);
+    __syncthreads();
+    // the run heads jump to their roots; every other site's label is read through
+    // its head
+    for (int k = 0; k < rows; k += 4) {
+        n = 0;
+        for (int q = k; q < k + 4 && q < rows; ++q)
+            put(~(bx[1][row0 + q] << 1) & valid, ~bx[0][row0 + q] & valid, row0 + q, n);
+        __syncwarp();
+        for (unsigned q = lane; q < n; q += 32) {
+            const uint32_t l = list[warp][q];
+            uint32_t p = vp[l];
+            while (true) {
+                const uint32_t g = vp[p];
+                if (g == p) break;
+                p = g;
+            }
+            vp[l] = p;
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+
+    // labels: the natural index of each site's tile root; tile roots are marked
+    // and appended to the update's list (one global atomic per block)
+    const uint32_t i00 = (uint32_t)X0 + L * ((uint32_t)Y0 + L * (uint32_t)Z0);
+    auto label = [&](uint32_t m) {
+        return i00 + (m & 63u) + L * ((m >> 6 & 15u) + L * (m >> 10));
+    };
+    uint32_t mine = 0u;  // bits 2 k, 2 k + 1: the lane's sites of row k are tile roots
+#pragma unroll 4
+    for (int k = 0; k < rows; ++k) {
+        if (!ex) continue;
+        const uint32_t l = (uint32_t)(TX * (row0 + k) + lx0);
+        const uint2 h = *reinterpret_cast<const uint2*>(&par[l]);
+        const uint32_t ra = par[h.x], rb = par[h.y];
+        const uint32_t root0 = ra == l, root1 = rb == l + 1;
+        mine |= (root0 | root1 << 1) << (2 * k);
+        *reinterpret_cast<uint2*>(a.lab + zb + L * (uint32_t)k + (uint32_t)(X0 + lx0)) =
+            make_uint2(label(ra) | (root0 ? kTileRoot : 0u), label(rb) | (root1 ? kTileRoot : 0u));
+    }
+    for (int w = threadIdx.x; w < WORDS; w += kSwThreads) a.face[tile * WORDS + w] = fm[w];
     const unsigned cnt = __popc(mine);
     unsigned incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const unsigned v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        const unsigned v = __shfl_up_sync(kAll, incl, o);
         if (lane >= o) incl += v;
     }
     unsigned wbase = 0;
     if (lane == 31) wbase = atomicAdd(&blk_count, incl);
-    wbase = __shfl_sync(0xFFFFFFFFu, wbase, 31);
+    wbase = __shfl_sync(kAll, wbase, 31);
     __syncthreads();
     if (threadIdx.x == 0) blk_base = atomicAdd(a.nroots, blk_count);
     __syncthreads();
     unsigned pos = blk_base + wbase + incl - cnt;
     for (uint32_t bits = mine; bits; bits &= bits - 1) {
         const int bit = __ffs(bits) - 1;
-        const int k = bit >> 1, e = bit & 1;
-        const int row = warp + NW * k;
-        const int ly = row % TY, lz = row / TY;
-        a.roots[pos++] = (uint32_t)(X0 + lx0 + e) +
-                         L * ((uint32_t)(Y0 + ly) + L * (uint32_t)(Z0 + lz));
+        a.roots[pos++] = zb + L * (uint32_t)(bit >> 1) + (uint32_t)(X0 + lx0 + (bit & 1));
     }
 }
 
@@ -759,15 +674,15 @@ __global__ void __launch_bounds__(256) sw_merge(const SwArgs a)
             lz = bit / TY;
         } else if (bit < TY * TZ + TX * TZ) {
             mu = 1;
-            // (2D: the even sites' word, then the odd sites')
+            // (per row the even sites' word, then the odd sites')
             const int k = bit - TY * TZ;
-            lx = D == 2 ? 2 * (k & 31) + (k >> 5) : k % TX;
+            lx = 2 * (k & 31) + (k >> 5 & 1);
             ly = ny - 1;
-            lz = D == 2 ? 0 : k / TX;
+            lz = k / TX;
         } else {
             mu = 2;
             const int k = bit - TY * TZ - TX * TZ;
-            lx = k % TX;
+            lx = 2 * (k & 31) + (k >> 5 & 1);
             ly = k / TX;
             lz = nz - 1;
         }
