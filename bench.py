@@ -71,7 +71,7 @@ WORKLOADS = {
                               desc="3D Ising, L=512, one bit per spin"),
     "ising2d_L8192_sw": dict(d=2, L=8192, n=1, beta=0.440687, storage="i8", bytes=16.0,
                              update=2, paper_flips_per_ns=1 / 4.62,
-                             kernels="sw_local, sw_merge, sw_resolve, sw_flip, measurement",
+                             kernels="sw_local2, sw_merge, sw_resolve, sw_flip, measurement",
                              desc="2D Ising ferromagnet J=1, L=8192, int8 spins, beta_c, "
                                   "Swendsen-Wang cluster updates (the paper's Table 1 "
                                   "cluster row)"),
@@ -390,11 +390,11 @@ def launch_shape(wl):
     """(kernel launches per sweep, name of the dominant kernel) of a workload."""
     d = wl["d"]
     if wl.get("update") == 2:
-        return 5, "sw_local<%d> .. sw_flip (Swendsen-Wang)" % d
+        return 5, "sw_local%d .. sw_flip (Swendsen-Wang)" % d
     if wl.get("multihit"):
         return 3, "ising_tile_kernel<%d,%d>" % (d, wl["tile"])
-    # the streaming paths: two colour passes and the one-block kernel that
-    # adds the measuring pass's partials
+    # the streaming paths: two colour passes and the kernel that adds the measuring
+    # pass's partials
     if wl["storage"] == "bits":
         return 3, "bits_stream<%d,0,0/1>" % d
     hb = 1 if wl.get("update") == 1 else 0
@@ -402,7 +402,7 @@ def launch_shape(wl):
         kern = "heis_pair" if (wl["L"] // 2) % 64 == 0 else "heis_stream"
         return 3, "%s<%d,%d,%d,0/1>" % (kern, d, wl.get("fast", 0), hb)
     if wl["storage"] == "angle":
-        return 3, "xy_stream<0,%d,0/1>" % hb
+        return 3, "xy_heatbath<0/1>" if hb else "xy_stream<0,0/1>"
     return 3, "i8_stream<%d,0,0,%d,0/1>" % (d, hb)
 
 

@@ -197,8 +197,11 @@ int sl_set_option(sl_lattice* lat, int option, int64_t value);
  * SM count and (d, L, n, storage, couplings, update rule, fast math); a
  * matching line is used without timing, and a new choice is appended.  The
  * chosen values are returned in *rows and *blocks_per_sm (either may be
- * NULL).  Lattices whose sweeps do not use the streaming kernels (slabs,
- * multi-hit, Swendsen-Wang, short rows, zero couplings) keep their options.
+ * NULL).  For continuous spins the automatic shape (both options 0) is timed
+ * too; where it is the fastest, this lattice runs it, and the values returned
+ * are the best of the others.  Lattices whose sweeps do not use the streaming
+ * kernels (slabs, multi-hit, Swendsen-Wang, short rows, zero couplings) keep
+ * their options.
  * Synchronises.
  */
 int sl_autotune(sl_lattice* lat, double beta, int trial_sweeps, const char* cache_path,

@@ -8,11 +8,11 @@
 //   sw_local2, sw_local3
 //               one CTA per tile (64 x 32 sites in 2D, 64 x 16 x 8 in 3D):
 //               loads the tile's spins and a one-site halo on its +x/+y/+z
-//               faces into shared memory (one warp per row, one lane per site
-//               pair), draws the bond uniforms, joins each row's x-runs of
+//               faces into shared memory (two words per row, by ballot, one lane
+//               per site pair), draws the bond uniforms, joins each row's x-runs of
 //               active bonds through warp ballots, then joins the runs along
 //               y and z by a lock-free union-find in shared memory (the
-//               larger root linked below the smaller by compare-and-swap),
+//               larger root linked below the smaller by an atomic minimum),
 //               which names every tile cluster by its smallest site (a y/z
 //               bond is skipped when the bond beside it already joins the
 //               same two runs), writes every site's label (the natural index
@@ -20,7 +20,7 @@
 //               one bit per active bond that leaves the tile, and appends
 //               its tile roots to a list;
 //   sw_merge    one thread per tile-face bond: unites the two labels of each
-//               active face bond in global memory (same hooking rule);
+//               active face bond in global memory (larger root below smaller);
 //               afterwards the root of every cluster is its smallest site;
 //   sw_resolve  one thread per listed tile root: follows the parents to the
 //               cluster root g and rewrites the tile root's word as g with
