@@ -1642,6 +1642,94 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
     store_partial(a.partials, mine);
 }
 
+// ----------------------------------------------------- Heisenberg, flat ----
+//
+// Metropolis sweeps of Heisenberg spins with a uniform coupling on rows that the
+// streaming kernels cannot take.  on_generic gives a block of 128 threads one row at a
+// time, of which the rows of a small lattice fill less than half, and computes 64-bit
+// indices for every neighbour; here a thread takes one colour index after another of
+// the whole array, 32 registers a thread.  Bound by issue: 3D L = 100 45 us a sweep and
+// now 17, L = 240 245 and 151, 2D L = 2002 64 and 42.  The arithmetic of a site is that
+// of on_generic, rounding for rounding; its heat-bath, whose roundings the compiler
+// chooses in each kernel, stays there.
+template <int D, bool FAST, bool MEAS>
+__global__ void __launch_bounds__(256) heis_flat(const OnArgs a, const FastDiv Wd,
+                                                 const FastDiv Ld)
+{
+    __shared__ double red[32];  // 4 per warp
+    const unsigned long long t64 = a.ctrl->t + a.toff;
+    const bool renorm =
+        a.renorm_every > 0 && (t64 + 1) % (unsigned long long)a.renorm_every == 0;
+    const int L = a.L, W = a.W, H = (int)a.H, P = D == 3 ? L * W : W;
+    const float J = a.J;
+    const PhiloxGroups pg =
+        philox_groups((uint32_t)t64, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
+    const float *vx = a.oth, *vy = a.oth + a.H, *vz = a.oth + 2 * a.H;
+    float *ux = a.own, *uy = a.own + a.H, *uz = a.own + 2 * a.H;
+    float pe = 0.f, pmx = 0.f, pmy = 0.f, pmz = 0.f;
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < H; j += gridDim.x * blockDim.x) {
+        const int row = (int)Wd.div((uint32_t)j), k = j - row * W;
+        const int z = D == 3 ? (int)Ld.div((uint32_t)row) : 0;
+        const int y = D == 3 ? row - z * L : row;
+        const int p = (y + z + a.c) & 1;
+        // the other x neighbour than j itself; -y, +y (, -z, +z)
+        const int je = p ? (k + 1 == W ? j + 1 - W : j + 1) : (k == 0 ? j + W - 1 : j - 1);
+        int nb[2 * D - 2];
+        if (D == 3) {
+            nb[0] = y == 0 ? j + (L - 1) * W : j - W;
+            nb[1] = y == L - 1 ? j - (L - 1) * W : j + W;
+        }
+        nb[2 * D - 4] = j < P ? j + H - P : j - P;
+        nb[2 * D - 3] = j + P < H ? j + P : j + P - H;
+        const float ox = __ldg(vx + j), oy = __ldg(vy + j), oz = __ldg(vz + j);
+        const float ex = __ldg(vx + je), ey = __ldg(vy + je), ez = __ldg(vz + je);
+        float hx = __fmaf_rn(J, p ? ex : ox, __fmul_rn(J, p ? ox : ex));
+        float hy = __fmaf_rn(J, p ? ey : oy, __fmul_rn(J, p ? oy : ey));
+        float hz = __fmaf_rn(J, p ? ez : oz, __fmul_rn(J, p ? oz : ez));
+#pragma unroll
+        for (int q = 0; q < 2 * D - 2; ++q) {
+            hx = __fmaf_rn(J, __ldg(vx + nb[q]), hx);
+            hy = __fmaf_rn(J, __ldg(vy + nb[q]), hy);
+            hz = __fmaf_rn(J, __ldg(vz + nb[q]), hz);
+        }
+        const uint4 r = philox_at(pg, (uint32_t)j, a.rk);
+        float sx = ux[j], sy = uy[j], sz = uz[j];
+        bool changed = false;
+        const float3 v = sphere_point<FAST>(r.y, r.z);
+        const float dE = -__fmaf_rn(__fsub_rn(v.z, sz), hz,
+                                    __fmaf_rn(__fsub_rn(v.x, sx), hx,
+                                              __fmul_rn(__fsub_rn(v.y, sy), hy)));
+        const float w = boltzmann<FAST>(__fmul_rn(-a.beta, dE));
+        if ((dE <= 0.f) | (u24(r.x) < w)) {
+            sx = v.x;
+            sy = v.y;
+            sz = v.z;
+            changed = true;
+        }
+        if (renorm) {
+            const float inv =
+                rsqrtf(__fmaf_rn(sz, sz, __fmaf_rn(sx, sx, __fmul_rn(sy, sy))));
+            sx = __fmul_rn(sx, inv);
+            sy = __fmul_rn(sy, inv);
+            sz = __fmul_rn(sz, inv);
+            changed = true;
+        }
+        if (changed) {
+            ux[j] = sx;
+            uy[j] = sy;
+            uz[j] = sz;
+        }
+        if (MEAS) {
+            pe -= sx * hx + sy * hy + sz * hz;
+            pmx += sx + ox;
+            pmy += sy + oy;
+            pmz += sz + oz;
+        }
+    }
+    if (!MEAS) return;
+    store_partial(a.partials, fp_partial(pe, pmx, pmy, pmz, red));
+}
+
 // Adds the partials a streaming measuring pass of nblocks blocks stored and
 // closes the pass (one block of kFinishThreads; FP64 in a fixed order).
 __global__ void __launch_bounds__(kFinishThreads) on_finish_kernel(const OnArgs a,
@@ -1849,6 +1937,12 @@ bool xy_flat_ok(const sl_lattice* h)
     return h->n == 2 && h->j_layout == SL_J_UNIFORM && h->kernel != 1;
 }
 
+bool heis_flat_ok(const sl_lattice* h)
+{
+    return h->n == 3 && h->j_layout == SL_J_UNIFORM && h->kernel != 1 &&
+           h->update != SL_UPDATE_HEATBATH;
+}
+
 bool on_stream_ok(const sl_lattice* h)
 {
     if (h->bonds[0][0] != nullptr || h->kernel == 1) return false;
@@ -1860,7 +1954,7 @@ bool on_stream_ok(const sl_lattice* h)
 
 bool on_streams(const sl_lattice* h) { return on_stream_ok(h) || (h->kernel == 4 && tile_ok(h)); }
 
-bool on_deferred(const sl_lattice* h) { return on_streams(h) || xy_flat_ok(h); }
+bool on_deferred(const sl_lattice* h) { return on_streams(h) || xy_flat_ok(h) || heis_flat_ok(h); }
 
 bool on_tile_ok(const sl_lattice* h) { return tile_ok(h); }
 
@@ -1906,6 +2000,21 @@ cudaError_t launch_xy_flat(const sl_lattice* h, const OnArgs& a, int var, cudaSt
     if (var == 2) xy_flat<D, EVEN, false, true><<<g, 256, 0, s>>>(a, cs, Wd, Ld);
     else if (var == 1) xy_flat<D, EVEN, true, false><<<g, 256, 0, s>>>(a, cs, Wd, Ld);
     else xy_flat<D, EVEN, false, false><<<g, 256, 0, s>>>(a, cs, Wd, Ld);
+    return a.measure ? launch_finish(h, a, (unsigned)g, s) : cudaGetLastError();
+}
+
+template <int D>
+cudaError_t launch_heis_flat(const sl_lattice* h, const OnArgs& a, int var, cudaStream_t s)
+{
+    const FastDiv Wd = make_fast_div((uint32_t)h->W), Ld = make_fast_div((uint32_t)h->L);
+    int g = grid_for(h->H, 256);
+    // (few FP64 sums, as for xy_flat)
+    if (a.measure && g > 4 * h->sms) g = 4 * h->sms;
+    auto run = [&](void (*k)(const OnArgs, const FastDiv, const FastDiv)) {
+        k<<<g, 256, 0, s>>>(a, Wd, Ld);
+    };
+    if (var == 1) run(a.measure ? heis_flat<D, true, true> : heis_flat<D, true, false>);
+    else run(a.measure ? heis_flat<D, false, true> : heis_flat<D, false, false>);
     return a.measure ? launch_finish(h, a, (unsigned)g, s) : cudaGetLastError();
 }
 
@@ -1964,8 +2073,11 @@ cudaError_t launch_on(const sl_lattice* h, OnArgs a, cudaStream_t s)
 #undef SPINMC_ON
         return a.measure ? launch_finish(h, a, (unsigned)grid, s) : cudaGetLastError();
     }
-    // XY sweeps with a uniform coupling (SL_OPT_KERNEL 1 asks for on_generic, which
-    // also takes float couplings, Heisenberg spins and the standalone measurement)
+    // sweeps with a uniform coupling (SL_OPT_KERNEL 1 asks for on_generic, which also
+    // takes float couplings, the heat-bath of Heisenberg spins and the standalone
+    // measurement)
+    if (a.update && heis_flat_ok(h))
+        return h->d == 2 ? launch_heis_flat<2>(h, a, var, s) : launch_heis_flat<3>(h, a, var, s);
     if (a.update && xy_flat_ok(h)) {
         if (h->d == 2)
             return h->W % 2 == 0 ? launch_xy_flat<2, true>(h, a, var, s)
