@@ -35,3 +35,17 @@ def test_pieces_give_the_chains_of_whole_packs(sm, d, samples, sides, temps):
                 assert got[1] == ref[1]
     b.close()
     w.close()
+
+
+def test_batches_of_different_packs_take_turns(sm):
+    """The kernel's shared-memory limit serves every batch of the process, whichever
+    was set up last."""
+    betas = np.geomspace(0.5, 3.0, 4)
+    a, b = (sm.Batch(2, [32] * 8, 4, betas, seed=2) for _ in range(2))
+    a.set_option(sm.SL_BOPT_PACK, 4)
+    b.set_option(sm.SL_BOPT_PACK, 1)
+    E = [np.asarray(x.run(3, 5, series=True).cpu()) for x in (a, b, a, b)]
+    np.testing.assert_array_equal(E[0], E[1])
+    np.testing.assert_array_equal(E[2], E[3])
+    a.close()
+    b.close()
