@@ -59,6 +59,14 @@ struct SweepFork {
     unsigned k, count;               // sweep being captured, sweeps of the run
 };
 
+// What a captured run of sweeps depends on: graphs are replayed while all of it is
+// the same.  Every field has its own place (cleared first: compared as bytes).
+struct GraphKey {
+    double beta;
+    uint64_t seed;
+    int kernel, rows, blocks_per_sm, shape_auto, update, fast_math, renorm_every, multihit, tile;
+};
+
 }  // namespace spinmc
 
 struct sl_lattice {
@@ -103,7 +111,7 @@ struct sl_lattice {
     int multihit, tile;      // k-fold multi-hit sweeps in tiles of side `tile` (0 = off)
     // cached graphs of 2^i sweeps, captured when a call first needs one
     cudaGraphExec_t graphs[spinmc::kGraphSizes];
-    uint64_t graph_key[4];
+    spinmc::GraphKey graph_key;
     void* owned_buf;
     // update workspace (Swendsen-Wang labels), caller-owned unless ws_owned
     void* ws;

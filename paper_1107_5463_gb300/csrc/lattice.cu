@@ -261,17 +261,22 @@ void drop_graphs(sl_lattice* h)
 // later call.
 void check_graph_key(sl_lattice* h, const SweepParams& p)
 {
-    uint64_t key[4];
-    std::memcpy(&key[0], &p.beta, 8);
-    key[1] = p.seed;
-    key[2] = ((uint64_t)h->kernel << 48) ^ ((uint64_t)h->rows << 32) ^
-             ((uint64_t)h->fast_math << 24) ^ ((uint64_t)h->update << 40) ^
-             (uint64_t)h->renorm_every;
-    key[3] = ((uint64_t)h->multihit << 16) ^ (uint64_t)h->tile ^
-             ((uint64_t)h->blocks_per_sm << 40) ^ ((uint64_t)h->shape_auto << 56);
-    if (std::memcmp(key, h->graph_key, sizeof key) == 0) return;
+    GraphKey key;
+    std::memset(&key, 0, sizeof key);
+    key.beta = p.beta;
+    key.seed = p.seed;
+    key.kernel = h->kernel;
+    key.rows = h->rows;
+    key.blocks_per_sm = h->blocks_per_sm;
+    key.shape_auto = h->shape_auto;
+    key.update = h->update;
+    key.fast_math = h->fast_math;
+    key.renorm_every = h->renorm_every;
+    key.multihit = h->multihit;
+    key.tile = h->tile;
+    if (std::memcmp(&key, &h->graph_key, sizeof key) == 0) return;
     drop_graphs(h);
-    std::memcpy(h->graph_key, key, sizeof key);
+    h->graph_key = key;
 }
 
 // Wait for the stream and check the error word; the control block comes back in
@@ -442,7 +447,7 @@ int create_lattice(int d, int L, int n, int j_layout, int storage, double J, con
     h->fork_res = SweepFork{};
     h->fork = nullptr;
     for (cudaGraphExec_t& g : h->graphs) g = nullptr;
-    std::memset(h->graph_key, 0, sizeof h->graph_key);
+    std::memset(&h->graph_key, 0, sizeof h->graph_key);
     h->next_colour = 0;
     h->ev = nullptr;
     h->owned_buf = owned;
