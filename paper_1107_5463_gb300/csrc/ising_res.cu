@@ -43,6 +43,7 @@ constexpr int kResSweeps = 1024;   // sweeps per launch
 constexpr int kResMaxBlocks = 256;
 constexpr int kResThreads = 1024;
 constexpr int kFlagStride = 8;     // flags 32 bytes apart: one L2 sector each
+constexpr int kResSmem = 216 * 1024;  // a block's dynamic part; its static arrays take 8.3 KB of 227
 constexpr unsigned kResWaitLimit = 1u << 21;  // polls of one word: about a second
 
 // In the upper half of the block partials (which the byte kernels' grids leave alone).
@@ -413,8 +414,7 @@ bool res_shape(const sl_lattice* h, ResShape* y)
     y->smem = 2 * (size_t)y->cstride + 4 * (size_t)h->d * y->jstride;
     const long long groups = (nown + 3) / 4;
     y->threads = groups >= kResThreads ? kResThreads : (int)((groups + 31) / 32 * 32);
-    // the static arrays take 8.3 KB of a block's 227 KB
-    if (y->smem > 216 * 1024) return false;
+    if (y->smem > (size_t)kResSmem) return false;
     if (G == 1) return true;
     // Several blocks finish with the one that owns most sites; the kernels in
     // global memory spread evenly but pay launches.  Microseconds a sweep, fitted to
@@ -475,8 +475,10 @@ cudaError_t i8_resident_sweeps(const sl_lattice* h, const SweepParams& p, int64_
     a.ctl = (ResCtl*)(h->partials + kI8Blocks);
     a.J = h->J;
     ResKernel k = pick_kernel(h, y.G > 1);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)y.smem);
+    // (one limit for every lattice: it is the kernel's, and another thread may launch it
+    // with another size between this call and the launch)
+    cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
     while (e == cudaSuccess && count > 0) {
         a.nsweeps = (int)(count < kResSweeps ? count : kResSweeps);
         void* args[] = {&a};

@@ -543,8 +543,10 @@ cudaError_t launch_walk_res(const WalkArgs& a, cudaStream_t s)
     const int fit = std::min(walk_block(KT), (int)((size_t)most / bytes));
     int per = (warps + sms - 1) / sms;
     if (per > fit) per = per <= 2 * fit ? (per + 1) / 2 : 1;
+    // (one limit whatever the number of walkers: it is the kernel's, and another thread
+    // may launch it with another size between this call and the launch)
     e = cudaFuncSetAttribute(walk_kernel<KT, WL, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(per * bytes));
+                             std::max(most, (int)(per * bytes)));
     if (e != cudaSuccess) return e;
     walk_kernel<KT, WL, SM>
         <<<(warps + per - 1) / per, 32 * per, per * bytes, s>>>(a, (uint32_t)bytes);
