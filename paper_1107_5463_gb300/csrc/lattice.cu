@@ -111,9 +111,12 @@ Layout make_layout(int d, int L, int n, int j_layout, int storage, int Lz = 0, b
     return y;
 }
 
-__global__ void set_series_kernel(Ctrl* c, long long base, double* E, double* m)
+// The next sweep's values go to series[0], whichever sweep that is: the index is the
+// device's, which runs ahead of the host's count where captured calls were replayed or
+// behind it where a launch failed.
+__global__ void set_series_kernel(Ctrl* c, double* E, double* m)
 {
-    c->series_base = base;
+    c->series_base = (long long)c->t;
     c->series_E = E;
     c->series_absm = m;
 }
@@ -520,7 +523,7 @@ cudaError_t set_sweep_index(const sl_lattice* h, int64_t t, cudaStream_t s)
 
 cudaError_t clear_series(const sl_lattice* h, cudaStream_t s)
 {
-    set_series_kernel<<<1, 1, 0, s>>>(h->ctrl, (long long)h->sweeps_done, nullptr, nullptr);
+    set_series_kernel<<<1, 1, 0, s>>>(h->ctrl, nullptr, nullptr);
     return cudaGetLastError();
 }
 
@@ -626,7 +629,7 @@ int sl_sweep_series(sl_lattice* h, double beta, int64_t nsweeps, uint64_t seed, 
         const int st = ising_table(h, beta, &p.tab);
         if (st != SL_OK) return st;
     }
-    set_series_kernel<<<1, 1, 0, h->stream>>>(h->ctrl, (long long)h->sweeps_done, dev_E, dev_absm);
+    set_series_kernel<<<1, 1, 0, h->stream>>>(h->ctrl, dev_E, dev_absm);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "series setup");
     int64_t left = nsweeps;
