@@ -59,8 +59,8 @@ struct SweepFork {
     unsigned k, count;               // sweep being captured, sweeps of the run
 };
 
-// What a captured run of sweeps depends on: graphs are replayed while all of it is
-// the same.  Every field has its own place (cleared first: compared as bytes).
+// What the kernels of a captured run of sweeps depend on: graphs are replayed while all
+// of it is the same.  Every field has its own place (cleared first: compared as bytes).
 struct GraphKey {
     double beta;
     uint64_t seed;
@@ -109,9 +109,11 @@ struct sl_lattice {
     int shape_auto;          // which measured them slower than the automatic shape: ignored
     int update;              // SL_UPDATE_METROPOLIS, _HEATBATH or _SW
     int multihit, tile;      // k-fold multi-hit sweeps in tiles of side `tile` (0 = off)
-    // cached graphs of 2^i sweeps, captured when a call first needs one
+    // graphs of 2^i sweeps (graph_sweeps, lattice.cu); graph_fresh bit i: the graph's
+    // arguments are those of the key
     cudaGraphExec_t graphs[spinmc::kGraphSizes];
     spinmc::GraphKey graph_key;
+    unsigned graph_fresh;
     void* owned_buf;
     // update workspace (Swendsen-Wang labels), caller-owned unless ws_owned
     void* ws;

@@ -215,10 +215,11 @@ cudaError_t fork_init(SweepFork* f)
     return e;
 }
 
-// Capture `count` sweeps into an executable graph on the private capture stream.
+// Capture `count` sweeps on the private capture stream into an executable graph, into
+// *out where there is one of this length (captured with other parameters: its kernels'
+// arguments are exchanged, which also leaves launches that are still running alone).
 int capture_sweeps(sl_lattice* h, const SweepParams& p, int count, cudaGraphExec_t* out)
 {
-    *out = nullptr;
     const bool forked = count > 1 && deferred_finish(h);
     cudaError_t e = forked ? fork_init(&h->fork_res) : cudaSuccess;
     if (e == cudaSuccess)
@@ -241,7 +242,13 @@ int capture_sweeps(sl_lattice* h, const SweepParams& p, int count, cudaGraphExec
         return st;
     }
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-    e = cudaGraphInstantiate(out, g, 0);
+    cudaGraphExecUpdateResultInfo info;
+    if (*out && cudaGraphExecUpdate(*out, g, &info) != cudaSuccess) {
+        cudaGetLastError();  // another kernel or shape: a new one
+        cudaGraphExecDestroy(*out);
+        *out = nullptr;
+    }
+    if (!*out) e = cudaGraphInstantiate(out, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
         *out = nullptr;
@@ -256,9 +263,10 @@ void drop_graphs(sl_lattice* h)
         if (g) cudaGraphExecDestroy(g);
         g = nullptr;
     }
+    h->graph_fresh = 0;
 }
 
-// Drop the graphs unless they were captured with the sweep parameters p and the
+// The graphs are stale unless they were captured with the sweep parameters p and the
 // options that shape the launches.  The kernels read the sweep index and the
 // series pointers from the device control block, so a capture serves every
 // later call.
@@ -278,8 +286,43 @@ void check_graph_key(sl_lattice* h, const SweepParams& p)
     key.multihit = h->multihit;
     key.tile = h->tile;
     if (std::memcmp(&key, &h->graph_key, sizeof key) == 0) return;
-    drop_graphs(h);
     h->graph_key = key;
+    h->graph_fresh = 0;
+}
+
+// nsweeps sweeps as replays of captured runs of 2^i sweeps: the powers of two that make
+// up the rest of a division by 32, then 32 at a time.
+//   To capture a sweep takes the host 2.4 us (Ising) to 3.5, to give a graph new
+// arguments 1, to make a graph 6 and to destroy one 5.5.  So a graph is kept when beta,
+// the seed or an option changes and takes the new arguments when its length is next
+// run, and the short runs come first, behind which the longer ones are captured.  (With
+// graphs dropped and made anew 16 sweeps with a new seed took 604 us in 3D XY, L = 100,
+// and now take 357, a repeated call 275; 63 sweeps of 2D bits, L = 1024, 1056, 399 and
+// 348; 63 of 2D bytes, L = 8192, 5030, 4371 and 4363.)
+//   Where a capture fails, its sweeps run as plain launches.
+int graph_sweeps(sl_lattice* h, const SweepParams& p, int64_t nsweeps)
+{
+    check_graph_key(h, p);
+    constexpr int top = kGraphSizes - 1;
+    for (int i = 0; i <= top; ++i) {
+        int64_t runs = i < top ? nsweeps >> i & 1 : nsweeps >> top;
+        if (runs == 0) continue;
+        if (!(h->graph_fresh >> i & 1u)) {
+            if (capture_sweeps(h, p, 1 << i, &h->graphs[i]) == SL_OK) h->graph_fresh |= 1u << i;
+            else cudaGetLastError();
+        }
+        for (; runs > 0; --runs) {
+            if (h->graph_fresh >> i & 1u) {
+                const cudaError_t e = cudaGraphLaunch(h->graphs[i], h->stream);
+                if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
+            } else {
+                const int st = model_sweeps(h, p, 1 << i, h->stream);
+                if (st != SL_OK) return st;
+            }
+            h->sweeps_done += 1LL << i;
+        }
+    }
+    return SL_OK;
 }
 
 // Wait for the stream and check the error word; the control block comes back in
@@ -451,6 +494,7 @@ int create_lattice(int d, int L, int n, int j_layout, int storage, double J, con
     h->fork = nullptr;
     for (cudaGraphExec_t& g : h->graphs) g = nullptr;
     std::memset(&h->graph_key, 0, sizeof h->graph_key);
+    h->graph_fresh = 0;
     h->next_colour = 0;
     h->ev = nullptr;
     h->owned_buf = owned;
@@ -638,23 +682,7 @@ int sl_sweep_series(sl_lattice* h, double beta, int64_t nsweeps, uint64_t seed, 
         if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
         left = 0;
     }
-    if (h->use_graph && left >= 2) {
-        // runs of 32 sweeps, then one each of the powers of two that make up the
-        // rest: a graph costs a launch, and inside one the finishing kernels run
-        // beside the next sweep
-        check_graph_key(h, p);
-        while (left > 0) {
-            int i = kGraphSizes - 1;
-            while ((1LL << i) > left) --i;
-            if (!h->graphs[i]) {
-                const int st = capture_sweeps(h, p, 1 << i, &h->graphs[i]);
-                if (st != SL_OK) return st;
-            }
-            e = cudaGraphLaunch(h->graphs[i], h->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
-            left -= 1LL << i;
-        }
-    }
+    if (h->use_graph && left >= 2) return graph_sweeps(h, p, left);
     if (left > 0) {
         const int st = model_sweeps(h, p, left, h->stream);
         if (st != SL_OK) return st;
