@@ -43,6 +43,7 @@ struct OnArgs {
     const float* Joth[3];
     int d, L, W, c;
     Segments seg;
+    int rows_mask;     // xy_heatbath: rows that a thread adds up before it folds them, less one
     long long H, N;
     uint32_t replica;
     RoundKeys rk;
@@ -537,7 +538,6 @@ __device__ __forceinline__ V3 shfl3_down(V3 v)
 template <int D, bool FAST, bool HB, bool MEAS>
 __global__ void __launch_bounds__(256, D == 2 && !HB ? 4 : 3) heis_stream(const OnArgs a)
 {
-    __shared__ double red[32];  // 4 per warp
     // Metropolis with accurate functions: the proposal's azimuth from the shared table
     constexpr bool TAB = !FAST && !HB;
     __shared__ float2 tab[TAB ? kTurnTab : 1];
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(256, D == 2 && !HB ? 4 : 3) heis_stream(const 
         v.z = __ldg(oz + i);
         return v;
     };
-    float pe = 0.f, pmx = 0.f, pmy = 0.f, pmz = 0.f;
+    LongSum sum[4] = {};  // E, M
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nitems;
          it += (long long)gridDim.x * blockDim.x) {
         const int k = (int)(it % W);
@@ -662,17 +662,17 @@ __global__ void __launch_bounds__(256, D == 2 && !HB ? 4 : 3) heis_stream(const 
                 }
             }
             if (MEAS) {
-                pe -= s.x * hx + s.y * hy + s.z * hz;
-                pmx += s.x + cur.x;
-                pmy += s.y + cur.y;
-                pmz += s.z + cur.z;
+                sum[0].add(-(s.x * hx + s.y * hy + s.z * hz));
+                sum[1].add(s.x + cur.x);
+                sum[2].add(s.y + cur.y);
+                sum[3].add(s.z + cur.z);
             }
             prev = cur;
             cur = nxt;
         }
     }
     if (!MEAS) return;
-    const Partial mine = fp_partial(pe, pmx, pmy, pmz, red);
+    const Partial mine = long_partial(sum, J);
     store_partial(a.partials, mine);
 }
 
@@ -689,7 +689,6 @@ struct P3 {
 template <int D, bool FAST, bool HB, bool MEAS>
 __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
 {
-    __shared__ double red[32];  // 4 per warp
     // Metropolis with accurate functions: the proposal's azimuth from the shared table
     constexpr bool TAB = !FAST && !HB;
     __shared__ float2 tab[TAB ? kTurnTab : 1];
@@ -732,7 +731,7 @@ __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
         v.z = __ldg(oz + i);
         return v;
     };
-    float pe = 0.f, pmx = 0.f, pmy = 0.f, pmz = 0.f;
+    LongSum sum[4] = {};  // E, M
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nitems;
          it += (long long)gridDim.x * blockDim.x) {
         const int k0 = 2 * (int)(it % WP);
@@ -850,18 +849,18 @@ __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
                 }
             }
             if (MEAS) {
-                pe -= s.x.x * hA.x + s.y.x * hA.y + s.z.x * hA.z + s.x.y * hB.x + s.y.y * hB.y +
-                      s.z.y * hB.z;
-                pmx += s.x.x + s.x.y + cur.x.x + cur.x.y;
-                pmy += s.y.x + s.y.y + cur.y.x + cur.y.y;
-                pmz += s.z.x + s.z.y + cur.z.x + cur.z.y;
+                sum[0].add(-(s.x.x * hA.x + s.y.x * hA.y + s.z.x * hA.z + s.x.y * hB.x +
+                             s.y.y * hB.y + s.z.y * hB.z));
+                sum[1].add(s.x.x + s.x.y + cur.x.x + cur.x.y);
+                sum[2].add(s.y.x + s.y.y + cur.y.x + cur.y.y);
+                sum[3].add(s.z.x + s.z.y + cur.z.x + cur.z.y);
             }
             prev = cur;
             cur = nxt;
         }
     }
     if (!MEAS) return;
-    const Partial mine = fp_partial(pe, pmx, pmy, pmz, red);
+    const Partial mine = long_partial(sum, J);
     store_partial(a.partials, mine);
 }
 
@@ -1162,7 +1161,6 @@ __global__ void __launch_bounds__(kTileThreads, 3) heis_tile3(const OnArgs a)
 template <bool FAST, bool MEAS>
 __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
 {
-    __shared__ double red[32];  // 4 per warp
     // Metropolis with accurate functions: sin and cos from the shared table
     constexpr bool TAB = !FAST;
     __shared__ float2 tab[TAB ? kTurnTab : 1];
@@ -1185,7 +1183,7 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
     const int lane = threadIdx.x & 31;
     const long long nitems = (long long)WP * nseg;
     const float J = a.J;
-    float pe = 0.f, pmx = 0.f, pmy = 0.f;
+    LongSum sum[3] = {};  // E, M
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nitems;
          it += (long long)gridDim.x * blockDim.x) {
         const int q = (int)(it % WP);
@@ -1283,16 +1281,16 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
                 if (ch) *reinterpret_cast<float2*>(a.own + j) = th;
             }
             if (MEAS) {
-                pe -= sx0 * hx0 + sy0 * hy0 + sx1 * hx1 + sy1 * hy1;
-                pmx += sx0 + sx1 + cur.c0 + cur.c1;
-                pmy += sy0 + sy1 + cur.s0 + cur.s1;
+                sum[0].add(-(sx0 * hx0 + sy0 * hy0 + sx1 * hx1 + sy1 * hy1));
+                sum[1].add(sx0 + sx1 + cur.c0 + cur.c1);
+                sum[2].add(sy0 + sy1 + cur.s0 + cur.s1);
             }
             prev = cur;
             cur = nxt;
         }
     }
     if (!MEAS) return;
-    const Partial mine = fp_partial(pe, pmx, pmy, 0.f, red);
+    const Partial mine = long_partial(sum, J);
     store_partial(a.partials, mine);
 }
 
@@ -1311,7 +1309,6 @@ constexpr int kHbList = 96;  // fewer than 32 waiting, then up to 64 from a row
 template <bool MEAS>
 __global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
 {
-    __shared__ double red[32];  // 4 per warp
     struct List {
         uint32_t j[kHbList], at[kHbList];
         float rho[kHbList], g[kHbList], cnum[kHbList], arg[kHbList];
@@ -1319,6 +1316,23 @@ __global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
     };
     __shared__ List lists[8];
     List& q = lists[threadIdx.x >> 5];
+    // what the rows so far add up to, each thread's own: registers are short here, and
+    // the latest rows, a.rows_mask + 1 at most, are still apart in `latest` (274 us a
+    // sweep at L = 4096; folded at every row 277, sums compensated in registers 281, plain
+    // sums of whole segments 272)
+    __shared__ LongSum sums[MEAS ? 3 : 1][MEAS ? 256 : 1];
+    auto fold = [&](float (&latest)[3]) {
+        if (!MEAS) return;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            LongSum v = sums[k][threadIdx.x];
+            v.add(latest[k]);
+            sums[k][threadIdx.x] = v;
+            latest[k] = 0.f;
+        }
+    };
+    if (MEAS)
+        for (int k = 0; k < 3; ++k) sums[k][threadIdx.x].s = sums[k][threadIdx.x].c = 0.f;
     const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
     const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
     const int L = a.L, W = a.W, nseg = a.seg.nseg;  // (L^2 <= 2^31: offsets fit in 32 bits)
@@ -1327,7 +1341,7 @@ __global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
     const uint32_t below = (1u << lane) - 1u;
     const long long nitems = (long long)WP * nseg;
     const float J = a.J;
-    float pe = 0.f, pmx = 0.f, pmy = 0.f;
+    float latest[3] = {0.f, 0.f, 0.f};  // E, M
     int nq = 0;  // sites waiting (the same in every lane)
     auto push = [&](bool wait, uint32_t j, uint32_t at, const VonMises& m, float hx, float hy) {
         const uint32_t b = __ballot_sync(0xFFFFFFFFu, wait);
@@ -1353,9 +1367,9 @@ __global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
         if (MEAS) {
             float sx, sy;
             sincos_turns(th, &sy, &sx);
-            pe -= sx * hx + sy * hy;
-            pmx += sx;
-            pmy += sy;
+            latest[0] -= sx * hx + sy * hy;
+            latest[1] += sx;
+            latest[2] += sy;
         }
     };
     // the next attempt of the last n waiting sites, one per lane
@@ -1447,19 +1461,23 @@ __global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
             if (a0) settle(j, von_mises_angle(v0, rnd.x), hx0, hy0);
             if (a1) settle(j + 1, von_mises_angle(v1, rnd.z), hx1, hy1);
             if (MEAS) {
-                pmx += cur.c0 + cur.c1;
-                pmy += cur.s0 + cur.s1;
+                latest[1] += cur.c0 + cur.c1;
+                latest[2] += cur.s0 + cur.s1;
             }
             push(!a0, j, 1u, v0, hx0, hy0);
             push(!a1, j + 1, 1u, v1, hx1, hy1);
             while (nq >= 32) serve(32);
+            if ((r & a.rows_mask) == a.rows_mask) fold(latest);
             prev = cur;
             cur = nxt;
         }
     }
     while (nq > 0) serve(nq < 32 ? nq : 32);
     if (!MEAS) return;
-    const Partial mine = fp_partial(pe, pmx, pmy, 0.f, red);
+    fold(latest);
+    LongSum sum[3];
+    for (int k = 0; k < 3; ++k) sum[k] = sums[k][threadIdx.x];
+    const Partial mine = long_partial(sum, J);
     store_partial(a.partials, mine);
 }
 
@@ -1883,6 +1901,7 @@ OnArgs make_args(const sl_lattice* h, int c)
     a.measure = c == 1;
     a.update = 1;
     a.seg = Segments{1, 1, 0};
+    a.rows_mask = 0;
     a.renorm_every = h->renorm_every;
     return a;
 }
@@ -2062,6 +2081,13 @@ cudaError_t launch_on(const sl_lattice* h, OnArgs a, cudaStream_t s)
             }
         } else {
             if (var == 2) {
+                // (a power of two up to 32, fewer on lattices with less than 1024 such
+                // runs of rows a multiprocessor)
+                int rows = 32;
+                while (rows > 1 &&
+                       (h->L % rows != 0 || lanes * (h->L / rows) < (long long)h->sms * 1024))
+                    rows >>= 1;
+                a.rows_mask = rows - 1;
                 if (a.measure) run(xy_heatbath<true>);
                 else run(xy_heatbath<false>);
             } else if (var == 1) {
