@@ -180,7 +180,9 @@ cudaError_t ising_i8_measure_advance(const sl_lattice* h, cudaStream_t s);
 
 // ---- Ising int8, lattices resident in shared memory (ising_res.cu) ----
 bool i8_resident_ok(const sl_lattice* h);
-cudaError_t i8_resident_sweeps(const sl_lattice* h, const SweepParams& p, int64_t count,
+// *left sweeps; counts down those it has launched, and leaves the rest to the other
+// kernels where its blocks cannot all be resident at once
+cudaError_t i8_resident_sweeps(const sl_lattice* h, const SweepParams& p, int64_t* left,
                                cudaStream_t s);
 cudaError_t i8_resident_clear(const sl_lattice* h, cudaStream_t s);  // once, at creation
 

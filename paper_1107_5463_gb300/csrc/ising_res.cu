@@ -445,11 +445,11 @@ bool i8_resident_ok(const sl_lattice* h)
     return res_shape(h, &y);
 }
 
-cudaError_t i8_resident_sweeps(const sl_lattice* h, const SweepParams& p, int64_t count,
+cudaError_t i8_resident_sweeps(const sl_lattice* h, const SweepParams& p, int64_t* left,
                                cudaStream_t s)
 {
     ResShape y;
-    if (!res_shape(h, &y)) return cudaErrorInvalidConfiguration;
+    if (!res_shape(h, &y)) return cudaSuccess;
     ResArgs a;
     for (int c = 0; c < 2; ++c) {
         a.s[c] = (int8_t*)h->spins[c];
@@ -479,15 +479,21 @@ cudaError_t i8_resident_sweeps(const sl_lattice* h, const SweepParams& p, int64_
     // with another size between this call and the launch)
     cudaError_t e =
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
-    while (e == cudaSuccess && count > 0) {
-        a.nsweeps = (int)(count < kResSweeps ? count : kResSweeps);
+    while (e == cudaSuccess && *left > 0) {
+        a.nsweeps = (int)(*left < kResSweeps ? *left : kResSweeps);
         void* args[] = {&a};
         if (y.G > 1)
             e = cudaLaunchCooperativeKernel((const void*)k, dim3(y.G), dim3(y.threads), args, y.smem,
                                             s);
         else
             e = cudaLaunchKernel((const void*)k, dim3(1), dim3(y.threads), args, y.smem, s);
-        count -= a.nsweeps;
+        if (e == cudaSuccess) *left -= a.nsweeps;
+    }
+    // Where the context has fewer multiprocessors than the device (a partition of it) the
+    // blocks do not all fit, and nothing was launched.
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        e = cudaSuccess;
     }
     return e;
 }

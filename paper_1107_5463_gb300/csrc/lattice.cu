@@ -678,16 +678,16 @@ int sl_sweep_series(sl_lattice* h, double beta, int64_t nsweeps, uint64_t seed, 
     if (e != cudaSuccess) return cuda_fail(e, "series setup");
     int64_t left = nsweeps;
     if (i8_resident_ok(h)) {
-        e = i8_resident_sweeps(h, p, nsweeps, h->stream);
+        e = i8_resident_sweeps(h, p, &left, h->stream);
+        h->sweeps_done += nsweeps - left;
         if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
-        left = 0;
     }
     if (h->use_graph && left >= 2) return graph_sweeps(h, p, left);
     if (left > 0) {
         const int st = model_sweeps(h, p, left, h->stream);
         if (st != SL_OK) return st;
+        h->sweeps_done += left;
     }
-    h->sweeps_done += nsweeps;
     return SL_OK;
 }
 
