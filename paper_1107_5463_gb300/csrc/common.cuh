@@ -104,13 +104,23 @@ enum Purpose : uint32_t { kSweep = 0, kInit = 1, kCoupling = 2, kExchange = 3 };
 // Device control block: one per lattice, inside the caller's buffer.
 struct Ctrl {
     unsigned long long t;      // index of the sweep in progress
-    long long series_base;     // sweep index written to series[0]
+    long long series_base;     // sweep index written to series[0]; -1: that of the next one closed
     double* series_E;          // per-sweep energy, or null
     double* series_absm;       // per-sweep |m|, or null
     unsigned int done;         // blocks finished in the measuring pass
     unsigned int error;        // bit 0: a bounded device-side wait ran out (sticky)
     double obs[4];             // E, Mx, My, Mz after the last measured pass
 };
+
+// Place in the series of the sweep with index t, which the caller closes.  A call's first
+// is its place 0 whatever its index, which runs ahead of the host's count where captured
+// calls were replayed and behind it where a launch failed.  (Read here, beside the next
+// sweep, and not when the series is set, where the read took up to 2 us of a short call.)
+__device__ __forceinline__ long long series_place(Ctrl* c, unsigned long long t)
+{
+    if (c->series_base < 0) c->series_base = (long long)t;
+    return (long long)t - c->series_base;
+}
 
 // Partial sums one block contributes to a measured pass.  Ising passes use
 // the integer members (exact), continuous spins the double members.

@@ -74,7 +74,7 @@ __device__ __forceinline__ void i8_finish(const I8Args& a, const Partial& tot)
     C->obs[2] = 0.0;
     C->obs[3] = 0.0;
     if (a.update || a.advance) {
-        const long long k = (long long)C->t + a.toff - C->series_base;
+        const long long k = series_place(C, C->t + a.toff);
         if (C->series_E) C->series_E[k] = E;
         // a slab records its own M (summed over slabs, |M| / N is |m|)
         if (C->series_absm) C->series_absm[k] = a.wrap ? fabs(M) / (double)a.N : M;

@@ -344,10 +344,14 @@ __global__ void __launch_bounds__(kResThreads, 1) i8_resident(const ResArgs a)
         if (flipsign) bond = -bond;
         const double E = -a.J * (double)bond;
         const double M = (double)(a.N - 2 * dn);
-        const long long k = (long long)t0 + s - a.ctrl->series_base;
+        // (as series_place; the last sweep's thread sets the base, to what makes no difference
+        // to the others)
+        const long long base = a.ctrl->series_base;
+        const long long k = (base < 0 ? 0LL : (long long)t0 - base) + s;
         if (a.ctrl->series_E) a.ctrl->series_E[k] = E;
         if (a.ctrl->series_absm) a.ctrl->series_absm[k] = fabs(M) / (double)a.N;
         if (s + 1 == a.nsweeps) {
+            if (base < 0) a.ctrl->series_base = (long long)t0;
             a.ctrl->obs[0] = E;
             a.ctrl->obs[1] = M;
             a.ctrl->obs[2] = 0.0;

@@ -909,7 +909,7 @@ __global__ void __launch_bounds__(256) sw_measure(const SwArgs a, Partial* parti
         C->obs[1] = M;
         C->obs[2] = 0.0;
         C->obs[3] = 0.0;
-        const long long k = (long long)C->t - C->series_base;
+        const long long k = series_place(C, C->t);
         if (C->series_E) C->series_E[k] = E;
         if (C->series_absm) C->series_absm[k] = fabs(M) / (double)a.N;
         C->t = C->t + 1;

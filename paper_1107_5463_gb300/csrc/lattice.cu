@@ -111,12 +111,9 @@ Layout make_layout(int d, int L, int n, int j_layout, int storage, int Lz = 0, b
     return y;
 }
 
-// The next sweep's values go to series[0], whichever sweep that is: the index is the
-// device's, which runs ahead of the host's count where captured calls were replayed or
-// behind it where a launch failed.
 __global__ void set_series_kernel(Ctrl* c, double* E, double* m)
 {
-    c->series_base = (long long)c->t;
+    c->series_base = -1;  // see series_place
     c->series_E = E;
     c->series_absm = m;
 }

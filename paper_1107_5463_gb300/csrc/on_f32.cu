@@ -338,7 +338,7 @@ __device__ __forceinline__ void on_finish(const OnArgs& a, const Partial& tot)
     C->obs[2] = tot.f[2];
     C->obs[3] = tot.f[3];
     if (a.update) {
-        const long long k = (long long)C->t + a.toff - C->series_base;
+        const long long k = series_place(C, C->t + a.toff);
         const double m = sqrt(tot.f[1] * tot.f[1] + tot.f[2] * tot.f[2] + tot.f[3] * tot.f[3]);
         if (C->series_E) C->series_E[k] = tot.f[0];
         if (C->series_absm) C->series_absm[k] = m / (double)a.N;
