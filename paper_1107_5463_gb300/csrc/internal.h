@@ -179,7 +179,7 @@ cudaError_t ising_i8_measure(const sl_lattice* h, cudaStream_t s);
 cudaError_t ising_i8_measure_advance(const sl_lattice* h, cudaStream_t s);
 
 // ---- Ising int8, lattices resident in shared memory (ising_res.cu) ----
-bool i8_resident_ok(const sl_lattice* h);
+bool i8_resident_ok(const sl_lattice* h, int64_t sweeps);  // for a call of so many
 // *left sweeps; counts down those it has launched, and leaves the rest to the other
 // kernels where its blocks cannot all be resident at once
 cudaError_t i8_resident_sweeps(const sl_lattice* h, const SweepParams& p, int64_t* left,

@@ -396,8 +396,9 @@ struct ResShape {
 
 int up16(long long x) { return (int)((x + 15) / 16 * 16); }
 
-// The split of a lattice over the multiprocessors, or false if it does not fit.
-bool res_shape(const sl_lattice* h, ResShape* y)
+// The split of a lattice over the multiprocessors for calls of `sweeps` sweeps, or false
+// if it does not fit or the other kernels are faster.
+bool res_shape(const sl_lattice* h, int64_t sweeps, ResShape* y)
 {
     if (h->N > (1LL << 28)) return false;  // offsets are 32-bit; far above the capacity
     const int P = (int)h->P;
@@ -430,15 +431,27 @@ bool res_shape(const sl_lattice* h, ResShape* y)
     const double site = d3 ? (al ? (np == 1 ? 0.37e-3 : 0.29e-3) : (np == 1 ? 0.95e-3 : 0.43e-3))
                            : (al ? 0.20e-3 : 0.27e-3);
     const bool bonds = h->j_layout == SL_J_BONDS;
-    const double other = h->W % 16 == 0 ? (d3 ? 1.4e-6 : 1.05e-6)           // i8_stream
-                         : bonds        ? 9.0e-6                             // i8_generic
-                                        : (d3 ? (al ? 1.9e-6 : 2.5e-6) : (al ? 1.4e-6 : 1.85e-6));
-    return 1.2 + own * site < 4.6 + (double)h->N * other;
+    const bool stream = h->W % 16 == 0;  // else i8_flat, or with bonds i8_generic
+    const double other = stream  ? (d3 ? 1.4e-6 : (bonds ? 1.2e-6 : 1.05e-6))
+                         : bonds ? 9.2e-6
+                                 : (d3 ? (al ? 1.9e-6 : 2.5e-6) : (al ? 1.4e-6 : 1.85e-6));
+    const double here = 1.2 + own * site;
+    const double there = (bonds && !stream ? 10.2 : 4.6) + (double)h->N * other;
+    if (here >= there) return false;
+    // A call also moves the spins to shared memory and back and meets its neighbours'
+    // blocks at the end (4.4 us more than a graph, 1.2 more than the launches of a single
+    // sweep), and puts the signs of its couplings together, so that short calls of large
+    // lattices are faster on the other kernels.  (+-1 bonds, 3D L = 128: 24.7 us for one
+    // sweep and 18.6, 68.9 and 67.7 for eight, 82.0 and 86.2 for ten; 2D L = 2048: 24.8
+    // and 20.6 for one, 38.8 and 43.1 for three; without bonds 3D L = 128 24.4 and 22.5
+    // for two, 35.2 and 36.9 for four.  `here` is some 13% above what such lattices take.)
+    const double load = bonds ? own * 2 * h->d * 0.055e-3 : 0.0;
+    return (double)sweeps * (there - 0.87 * here) > (sweeps == 1 ? 1.2 : 4.4) + load;
 }
 
 }  // namespace
 
-bool i8_resident_ok(const sl_lattice* h)
+bool i8_resident_ok(const sl_lattice* h, int64_t sweeps)
 {
     if (h->storage != SL_STORE_I8 || h->slab || h->multihit > 0 || h->kernel != 0 ||
         h->update == SL_UPDATE_SW || h->bonds_have_zero || h->z0 != 0)
@@ -446,14 +459,14 @@ bool i8_resident_ok(const sl_lattice* h)
     // rows and grid caps given by the user shape the streaming kernel
     if ((h->rows > 0 || h->blocks_per_sm > 0) && !h->shape_tuned) return false;
     ResShape y;
-    return res_shape(h, &y);
+    return res_shape(h, sweeps, &y);
 }
 
 cudaError_t i8_resident_sweeps(const sl_lattice* h, const SweepParams& p, int64_t* left,
                                cudaStream_t s)
 {
     ResShape y;
-    if (!res_shape(h, &y)) return cudaSuccess;
+    if (!res_shape(h, *left, &y)) return cudaSuccess;
     ResArgs a;
     for (int c = 0; c < 2; ++c) {
         a.s[c] = (int8_t*)h->spins[c];

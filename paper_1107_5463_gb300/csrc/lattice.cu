@@ -674,7 +674,7 @@ int sl_sweep_series(sl_lattice* h, double beta, int64_t nsweeps, uint64_t seed, 
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "series setup");
     int64_t left = nsweeps;
-    if (i8_resident_ok(h)) {
+    if (i8_resident_ok(h, left)) {
         e = i8_resident_sweeps(h, p, &left, h->stream);
         h->sweeps_done += nsweeps - left;
         if (e != cudaSuccess) return cuda_fail(e, "sweep launch");
