@@ -329,6 +329,8 @@ __global__ void __launch_bounds__(kResThreads, 1) i8_resident(const ResArgs a)
     }
     // close the launch's sweeps: E = -J (2d H - 2 v) over the H colour-1 sites
     const bool flipsign = a.tab.sigma_neg && !HB;
+    // (series_place; a thread that reads it after the last sweep's has set it finds the same)
+    const long long set = a.ctrl->series_base, first = set < 0 ? (long long)t0 : set;
     for (int s = tid; s < a.nsweeps; s += T) {
         long long v, dn;
         if (MULTI) {
@@ -344,14 +346,11 @@ __global__ void __launch_bounds__(kResThreads, 1) i8_resident(const ResArgs a)
         if (flipsign) bond = -bond;
         const double E = -a.J * (double)bond;
         const double M = (double)(a.N - 2 * dn);
-        // (as series_place; the last sweep's thread sets the base, to what makes no difference
-        // to the others)
-        const long long base = a.ctrl->series_base;
-        const long long k = (base < 0 ? 0LL : (long long)t0 - base) + s;
+        const long long k = (long long)t0 + s - first;
         if (a.ctrl->series_E) a.ctrl->series_E[k] = E;
         if (a.ctrl->series_absm) a.ctrl->series_absm[k] = fabs(M) / (double)a.N;
         if (s + 1 == a.nsweeps) {
-            if (base < 0) a.ctrl->series_base = (long long)t0;
+            a.ctrl->series_base = first;
             a.ctrl->obs[0] = E;
             a.ctrl->obs[1] = M;
             a.ctrl->obs[2] = 0.0;
