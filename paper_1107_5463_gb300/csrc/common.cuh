@@ -291,21 +291,45 @@ __device__ __forceinline__ Partial fp_partial(float e, float mx, float my, float
     return p;
 }
 
-// FP32 sum of a thread over a segment of any length, with what each addition rounds off
-// carried into the next (Kahan): its error stays that of the terms themselves, where a
-// plain sum's grows with the number of sites, 512 rows to 4e-6 of a uniform lattice's M.
-// (Per sweep, plain sums and these: 3D Heisenberg L = 256 143.9 and 145.2 us, on single
-// columns 179.4 and 183.3, L = 128 23.9 and 23.7, 2D L = 2048 35.5 and 36.0; 2D XY L =
-// 4096 91.9 and 92.7, L = 1408 19.9 and 19.6.)
+// FP32 sum of a thread over a segment of any length, with what the additions round off
+// added up beside it, so that it errs by some 2^-40 of the terms' sizes however many there
+// are; a plain sum's error grows with them, over 512 rows to 4e-6 of a uniform lattice's M.
+// The sum starts at a bias above all it can reach: what x - (t - s) gives is then exactly
+// what was lost, as s is the larger one (without it that takes six additions for three).
+// (Per sweep, plain sums and these: 3D Heisenberg L = 256 143.8 and 145.1 us, on single
+// columns 179.2 and 183.4, L = 128 24.0 and 23.8, 2D L = 2048 35.4 and 35.9; 2D XY L =
+// 4096 91.9 and 92.9, L = 1408 20.0 and 19.9.)
 struct __align__(8) LongSum {
-    float s, c;
+    float s, lost;
     __device__ __forceinline__ void add(float x)
     {
-        const float y = __fsub_rn(x, c), t = __fadd_rn(s, y);
-        c = __fsub_rn(__fsub_rn(t, s), y);
+        const float t = __fadd_rn(s, x);
+        lost = __fadd_rn(lost, __fsub_rn(x, __fsub_rn(t, s)));
         s = t;
     }
 };
+
+// the exponent of J, between those of 2^-127 and 2^100
+__device__ __forceinline__ int coupling_exponent(float J)
+{
+    return min((int)(__float_as_uint(J) >> 23 & 255u), 227) - 127;
+}
+
+// the biases of the energy (k = 0; terms up to 24 |J|) and of M's components (up to 4)
+__device__ __forceinline__ float sum_bias(int k, float J)
+{
+    return __uint_as_float((uint32_t)(127 + (k == 0 ? 17 + coupling_exponent(J) : 14)) << 23);
+}
+
+template <int N>
+__device__ __forceinline__ void start_sums(LongSum (&v)[N], float J)
+{
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        v[k].s = sum_bias(k, J);
+        v[k].lost = 0.f;
+    }
+}
 
 // (sum, what rounding took from it) of two such pairs
 __device__ __forceinline__ float2 add_pairs(float2 a, float2 b)
@@ -331,13 +355,13 @@ __device__ __forceinline__ Partial long_partial(const LongSum (&v)[N], float J)
     __shared__ float2 warps[8][4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool up = (lane & 16) != 0, odd = (lane & 8) != 0;
-    // the exponent of J, between those of 2^-127 and 2^126
-    const int ej = min((int)(__float_as_uint(J) >> 23 & 255u), 253) - 127;
+    const int ej = coupling_exponent(J);
     const float scale = __uint_as_float((uint32_t)(127 - ej) << 23);
     float2 f[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        f[k] = k < N ? make_float2(v[k % N].s, -v[k % N].c) : make_float2(0.f, 0.f);
+        f[k] = k < N ? make_float2(v[k % N].s - sum_bias(k, J), v[k % N].lost)
+                     : make_float2(0.f, 0.f);
     f[0].x *= scale;
     f[0].y *= scale;
     const float2 a = add_pairs(up ? f[2] : f[0], shfl_xor_pair(up ? f[0] : f[2], 16));

@@ -564,7 +564,8 @@ __global__ void __launch_bounds__(256, D == 2 && !HB ? 4 : 3) heis_stream(const 
         v.z = __ldg(oz + i);
         return v;
     };
-    LongSum sum[4] = {};  // E, M
+    LongSum sum[4];  // E, M
+    start_sums(sum, J);
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nitems;
          it += (long long)gridDim.x * blockDim.x) {
         const int k = (int)(it % W);
@@ -731,7 +732,8 @@ __global__ void __launch_bounds__(256, D == 2 ? 3 : 2) heis_pair(const OnArgs a)
         v.z = __ldg(oz + i);
         return v;
     };
-    LongSum sum[4] = {};  // E, M
+    LongSum sum[4];  // E, M
+    start_sums(sum, J);
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nitems;
          it += (long long)gridDim.x * blockDim.x) {
         const int k0 = 2 * (int)(it % WP);
@@ -1183,7 +1185,8 @@ __global__ void __launch_bounds__(256) xy_stream(const OnArgs a)
     const int lane = threadIdx.x & 31;
     const long long nitems = (long long)WP * nseg;
     const float J = a.J;
-    LongSum sum[3] = {};  // E, M
+    LongSum sum[3];  // E, M
+    start_sums(sum, J);
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < nitems;
          it += (long long)gridDim.x * blockDim.x) {
         const int q = (int)(it % WP);
@@ -1331,8 +1334,6 @@ __global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
             latest[k] = 0.f;
         }
     };
-    if (MEAS)
-        for (int k = 0; k < 3; ++k) sums[k][threadIdx.x].s = sums[k][threadIdx.x].c = 0.f;
     const uint32_t t = (uint32_t)a.ctrl->t + a.toff;
     const PhiloxGroups pg = philox_groups(t, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
     const int L = a.L, W = a.W, nseg = a.seg.nseg;  // (L^2 <= 2^31: offsets fit in 32 bits)
@@ -1342,6 +1343,11 @@ __global__ void __launch_bounds__(256) xy_heatbath(const OnArgs a)
     const long long nitems = (long long)WP * nseg;
     const float J = a.J;
     float latest[3] = {0.f, 0.f, 0.f};  // E, M
+    if (MEAS) {
+        LongSum v[3];
+        start_sums(v, J);
+        for (int k = 0; k < 3; ++k) sums[k][threadIdx.x] = v[k];
+    }
     int nq = 0;  // sites waiting (the same in every lane)
     auto push = [&](bool wait, uint32_t j, uint32_t at, const VonMises& m, float hx, float hy) {
         const uint32_t b = __ballot_sync(0xFFFFFFFFu, wait);

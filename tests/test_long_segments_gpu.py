@@ -64,3 +64,18 @@ def test_xy(sm, L, opts):
     want = magnetisation(sm, 2, L, 2, s0, [o for o in opts if o[0] != "ROWS"] + [("ROWS", 1)])
     assert torch.equal(got[1], want[1])
     assert abs(got[0] - want[0]) <= 1e-7 * want[0]
+
+
+@pytest.mark.parametrize("d,L,n", [(3, 64, 3), (3, 128, 3), (2, 1408, 2)])
+def test_couplings_of_any_size(sm, d, L, n):
+    """At beta = 0 every move is accepted whatever J, and a power of two in J goes through
+    every product and sum unchanged, as long as none leaves FP32's range: E / J is the same
+    number.  (Above 2^100 the energy's bias stays where it is; plain sums' 1e-6 then.)"""
+    E = {}
+    for k in (0, 100, -100, 112):
+        lat = sm.Lattice(d, L, n=n, J=2.0 ** k, seed=4)
+        E[k] = lat.sweep_series(0.0, 2, 8)[0].cpu().numpy() * 2.0 ** -k
+        lat.close()
+    np.testing.assert_array_equal(E[100], E[0])
+    np.testing.assert_array_equal(E[-100], E[0])
+    np.testing.assert_allclose(E[112], E[0], rtol=0, atol=1e-6 * 2 * d * L ** d)
