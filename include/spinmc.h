@@ -502,8 +502,8 @@ int sl_walkers_get_spins(sl_walkers* w, int walker, int8_t* dst);
 
 /* Checkpoint load.  sl_walkers_set_spins writes one walker's configuration
  * (natural order int8 +-1, host or device, N entries) and sets the walker's
- * level to that of the configuration (k = (E + 2N) / 4); SL_EINVAL if the
- * level lies outside the walker's window.  sl_walkers_write sets S, H (host,
+ * level to that of the configuration (k = (E + 2N) / 4); SL_EINVAL, and the
+ * walker stays as it was, if the level lies outside the walker's window.  sl_walkers_write sets S, H (host,
  * [walker][kmax], as sl_walkers_read returns them), stages and visited-level
  * masks; any pointer may be NULL to keep that array.
  * sl_walkers_set_sweeps_done sets the next sweep index.  Restoring all of

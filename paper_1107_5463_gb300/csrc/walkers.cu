@@ -439,26 +439,36 @@ __global__ void walk_gather_kernel(const uint32_t* spins, long long N, int walke
         nat[i] = ((col[i] >> (walker & 31)) & 1u) ? (int8_t)-1 : (int8_t)1;
 }
 
-// Writes one walker's bit of every site word from a natural-order +-1
-// configuration (1 = down; the other walkers' bits are kept) and sets the
-// walker's level to k = (E + 2N) / 4 of that configuration (one block).
-__global__ void __launch_bounds__(256) walk_scatter_kernel(uint32_t* spins, const int8_t* nat,
+// Works out the level k = (E + 2N) / 4 of a natural-order +-1 configuration, leaves it in
+// the first word of nat and, if it lies in [klo, khi], writes the walker's bit of every
+// site word (1 = down; the other walkers' bits are kept) and its level.  A walker never
+// stands outside its window: walk_kernel indexes shared memory by its level (one block).
+__global__ void __launch_bounds__(256) walk_scatter_kernel(uint32_t* spins, int8_t* nat,
                                                            long long N, int L, int log2L,
-                                                           int walker, int32_t* level)
+                                                           int walker, int klo, int khi,
+                                                           int32_t* level)
 {
     __shared__ long long red[32];
+    __shared__ int32_t k;
     uint32_t* col = spins + (size_t)(walker >> 5) * (size_t)N;
     const uint32_t bit = 1u << (walker & 31);
     long long bond = 0;
     for (long long i = threadIdx.x; i < N; i += blockDim.x) {
-        col[i] = (col[i] & ~bit) | (nat[i] < 0 ? bit : 0u);
         const int x = (int)(i & (L - 1)), y = (int)(i >> log2L);
         const long long xp = (long long)y * L + ((x + 1) & (L - 1));
         const long long yp = (long long)((y + 1) & (L - 1)) * L + x;
         bond += (long long)nat[i] * (nat[xp] + nat[yp]);
     }
     const long long tot = block_sum(bond, red);
-    if (threadIdx.x == 0) level[walker] = (int32_t)((-tot + 2 * N) / 4);
+    if (threadIdx.x == 0) k = (int32_t)((-tot + 2 * N) / 4);
+    __syncthreads();
+    if (k >= klo && k <= khi) {
+        for (long long i = threadIdx.x; i < N; i += blockDim.x)
+            col[i] = (col[i] & ~bit) | (nat[i] < 0 ? bit : 0u);
+        if (threadIdx.x == 0) level[walker] = k;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) *reinterpret_cast<int32_t*>(nat) = k;
 }
 
 struct WalkLayout {
@@ -850,18 +860,19 @@ int sl_walkers_set_spins(sl_walkers* w, int walker, const int8_t* src)
     if (walker < 0 || walker >= w->nwalk) return fail(SL_EINVAL, "walker %d out of range", walker);
     int8_t* nat = (int8_t*)(w->base + w->y.off_nat);
     int32_t* level = (int32_t*)(w->base + w->y.off_level);
+    const int win = walker / w->wpw;
     cudaError_t e = cudaMemcpyAsync(nat, src, (size_t)w->N, cudaMemcpyDefault, w->stream);
     if (e == cudaSuccess) {
-        walk_scatter_kernel<<<1, 256, 0, w->stream>>>((uint32_t*)(w->base + w->y.off_spins), nat,
-                                                       w->N, w->L, w->log2L, walker, level);
+        walk_scatter_kernel<<<1, 256, 0, w->stream>>>(
+            (uint32_t*)(w->base + w->y.off_spins), nat, w->N, w->L, w->log2L, walker,
+            w->klo_host[win], w->khi_host[win], level);
         e = cudaGetLastError();
     }
     int32_t k = -1;
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&k, level + walker, sizeof k, cudaMemcpyDeviceToHost, w->stream);
+        e = cudaMemcpyAsync(&k, nat, sizeof k, cudaMemcpyDeviceToHost, w->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(w->stream);
     if (e != cudaSuccess) return cuda_fail(e, "sl_walkers_set_spins");
-    const int win = walker / w->wpw;
     if (k < w->klo_host[win] || k > w->khi_host[win])
         return fail(SL_EINVAL, "walker %d: the configuration's level %d lies outside its window "
                                "[%d, %d]", walker, k, w->klo_host[win], w->khi_host[win]);
