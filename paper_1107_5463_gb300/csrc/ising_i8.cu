@@ -57,7 +57,6 @@ struct I8Args {
     int measure;  // accumulate E and M and finish the pass
     int update;   // 0: standalone measurement (no moves, no sweep advance)
     int advance;  // a measurement that closes a sweep: write the series, t + 1
-    int defer;    // i8_stream: add the block totals into the accumulator for i8_finish_kernel
     int Lz;       // planes along the slowest axis (L, or the slab's planes)
     int wrap;     // 1: periodic along the slowest axis; 0: halo planes at -1 and Lz
     int par;      // parity of the first plane's global index
@@ -522,24 +521,18 @@ __global__ void __launch_bounds__(128) i8_stream(const I8Args a)
     const long long na_after = s_na + 2 * D * s_flip - 2 * s_flipna;
     long long bond = (long long)(2 * D) * (long long)nsite - 2 * na_after;
     if (JNEG && !HB) bond = -bond;
-    Partial mine;
-    mine.i0 = block_sum(bond, red);
-    mine.i1 = block_sum((long long)down, red);
-    mine.f[0] = mine.f[1] = mine.f[2] = mine.f[3] = 0.0;
-    if (a.defer) {
-        // integer totals: the order of the additions does not matter, so
-        // every block adds its own into the pass's accumulator
-        if (threadIdx.x == 0) {
-            Partial* acc = a.partials + kMaxBlocks;
-            atomicAdd(reinterpret_cast<unsigned long long*>(&acc->i0), (unsigned long long)mine.i0);
-            atomicAdd(reinterpret_cast<unsigned long long*>(&acc->i1), (unsigned long long)mine.i1);
-        }
-        return;
+    const long long b = block_sum(bond, red);
+    const long long dn = block_sum((long long)down, red);
+    // integer totals: the order of the additions does not matter, so every block
+    // adds its own into the pass's accumulator, for i8_finish_kernel
+    if (threadIdx.x == 0) {
+        Partial* acc = a.partials + kMaxBlocks;
+        atomicAdd(reinterpret_cast<unsigned long long*>(&acc->i0), (unsigned long long)b);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&acc->i1), (unsigned long long)dn);
     }
-    finish_pass<false>(a.ctrl, a.partials, mine, [&](const Partial& tot) { i8_finish(a, tot); });
 }
 
-// Closes an i8_stream measuring pass from the totals its blocks added into
+// Closes an i8_stream or i8_flat measuring pass from the totals its blocks added into
 // the accumulator after the block partials, and clears the accumulator for
 // the next pass (one thread; the kernel boundary orders it after the pass).
 __global__ void i8_finish_kernel(const I8Args a)
@@ -722,7 +715,6 @@ I8Args make_args(const sl_lattice* h, int c)
     a.measure = c == 1;
     a.update = 1;
     a.advance = 0;
-    a.defer = 0;
     a.Lz = h->Lz;
     a.wrap = !h->slab;
     a.par = h->z0 & 1;
@@ -796,7 +788,6 @@ cudaError_t launch_pass(const sl_lattice* h, I8Args a, cudaStream_t s, bool stre
             grid = h->sms * h->blocks_per_sm;
         const bool bonds = a.Jown[0] != nullptr;
         const bool jneg = a.tab.sigma_neg != 0;
-        a.defer = a.measure;
         // slabs have uniform couplings: their instantiations have BONDS = 0
 #define SPINMC_LAUNCH(D, B, N, HB)                                                        \
     do {                                                                                  \
@@ -822,7 +813,7 @@ cudaError_t launch_pass(const sl_lattice* h, I8Args a, cudaStream_t s, bool stre
             else { if (jneg) SPINMC_LAUNCH(3, 0, 1, 0); else SPINMC_LAUNCH(3, 0, 0, 0); }
         }
 #undef SPINMC_LAUNCH
-        if (a.defer) return launch_finish(h, a, s);
+        if (a.measure) return launch_finish(h, a, s);
     } else {
         int grid = grid_for((h->H + 3) >> 2, 256);
         if (a.measure && grid > kI8Blocks) grid = kI8Blocks;

@@ -1520,7 +1520,7 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
     const float J = a.J;
     const PhiloxGroups pg =
         philox_groups((uint32_t)a.ctrl->t + a.toff, a.replica, (kSweep << 1) | (uint32_t)a.c, a.rk);
-    const int ncalls = (H + 1) / 2;
+    const int ncalls = H / 2;  // (L is even, and so is H)
     float pe = 0.f, pmx = 0.f, pmy = 0.f;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < ncalls; q += gridDim.x * blockDim.x) {
         const int j0 = 2 * q;
@@ -1530,7 +1530,6 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
         int y = D == 3 ? row - z * L : row;
         // neighbour vectors of the two sites: -x, +x, -y, +y (, -z, +z)
         float2 v[2][2 * D], own_col[2];
-        const bool second = EVEN || j0 + 1 < H;
         if (EVEN) {
             const int p = (y + z + a.c) & 1;
             const float4* c4 = reinterpret_cast<const float4*>(cs);
@@ -1557,7 +1556,7 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
         } else {
 #pragma unroll
             for (int b = 0; b < 2; ++b) {
-                const int j = b && second ? j0 + 1 : j0;
+                const int j = j0 + b;
                 const int p = (y + z + a.c) & 1;
                 own_col[b] = __ldg(cs + j);
                 const float2 e = __ldg(cs + (p ? (k + 1 == W ? j + 1 - W : j + 1)
@@ -1570,7 +1569,7 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
                 }
                 v[b][2 * D - 2] = __ldg(cs + (j < P ? j + H - P : j - P));
                 v[b][2 * D - 1] = __ldg(cs + (j + P < H ? j + P : j + P - H));
-                if (second && ++k == W) {  // the second site opens the next row
+                if (++k == W) {  // the second site opens the next row
                     k = 0;
                     if (++y == L && D == 3) {
                         y = 0;
@@ -1596,13 +1595,13 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
             th[1] = o.y;
         } else {
             th[0] = a.own[j0];
-            th[1] = second ? a.own[j0 + 1] : th[0];
+            th[1] = a.own[j0 + 1];
         }
         bool changed[2] = {false, false};
         if (HB) {
             const VonMises m0 = von_mises_setup(hx[0], hy[0], a.beta);
             const VonMises m1 = von_mises_setup(hx[1], hy[1], a.beta);
-            bool p0 = true, p1 = second;
+            bool p0 = true, p1 = true;
             uint32_t acc0 = 0u, acc1 = 0u;
             for (int at = 0; at < kVonMisesAttempts && (p0 || p1); ++at) {
                 const uint4 rnd = philox4x32_10(
@@ -1619,9 +1618,9 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
                 }
             }
             if (!p0) th[0] = von_mises_angle(m0, acc0);
-            if (second && !p1) th[1] = von_mises_angle(m1, acc1);
+            if (!p1) th[1] = von_mises_angle(m1, acc1);
             changed[0] = !p0;
-            changed[1] = second && !p1;
+            changed[1] = !p1;
 #pragma unroll
             for (int b = 0; b < 2; ++b) sincos_angle<FAST>(th[b], &sy[b], &sx[b]);
         } else {
@@ -1648,17 +1647,15 @@ __global__ void __launch_bounds__(256) xy_flat(const OnArgs a, const float2* cs,
                 *reinterpret_cast<float2*>(a.own + j0) = make_float2(th[0], th[1]);
         } else {
             if (changed[0]) a.own[j0] = th[0];
-            if (second && changed[1]) a.own[j0 + 1] = th[1];
+            if (changed[1]) a.own[j0 + 1] = th[1];
         }
         if (a.measure) {
             pe -= sx[0] * hx[0] + sy[0] * hy[0];
             pmx += sx[0] + own_col[0].x;
             pmy += sy[0] + own_col[0].y;
-            if (second) {
-                pe -= sx[1] * hx[1] + sy[1] * hy[1];
-                pmx += sx[1] + own_col[1].x;
-                pmy += sy[1] + own_col[1].y;
-            }
+            pe -= sx[1] * hx[1] + sy[1] * hy[1];
+            pmx += sx[1] + own_col[1].x;
+            pmy += sy[1] + own_col[1].y;
         }
     }
     if (!a.measure) return;
