@@ -201,7 +201,9 @@ int sl_set_option(sl_lattice* lat, int option, int64_t value);
  * too; where it is the fastest, this lattice runs it, and the values returned
  * are the best of the others.  Lattices whose sweeps do not use the streaming
  * kernels (slabs, multi-hit, Swendsen-Wang, short rows, zero couplings) keep
- * their options.
+ * their options.  Byte lattices that fit the device's shared memory are tuned
+ * for the calls that stream them all the same (short ones of large lattices);
+ * their other calls run without regard to the choice.
  * Synchronises.
  */
 int sl_autotune(sl_lattice* lat, double beta, int trial_sweeps, const char* cache_path,

@@ -222,7 +222,7 @@ extern "C" int sl_autotune(sl_lattice* h, double beta, int trial_sweeps, const c
     // Segments in whole waves, which the automatic shape deals out for continuous
     // spins, are mostly the faster choice: then they run, and the caller still learns
     // the best of the shapes that the options can name (3D Heisenberg L = 256: 166 us
-    // and 143).
+    // and 145).
     int automatic = 0;
     for (int kern : kernels) {
         if (h->n == 1 || kern < 0 || kern == 4 || e != cudaSuccess || st != SL_OK) continue;

@@ -323,7 +323,7 @@ int graph_sweeps(sl_lattice* h, const SweepParams& p, int64_t nsweeps)
 }
 
 // Wait for the stream and check the error word; the control block comes back in
-// the same trip (one copy of 88 bytes in place of a synchronisation and a copy
+// the same trip (one copy of 72 bytes in place of a synchronisation and a copy
 // each for the error word and the observables, some 10 us apiece).
 int sync_and_check(sl_lattice* h, Ctrl* out = nullptr)
 {
@@ -580,9 +580,9 @@ Segments pick_segments(const sl_lattice* h, long long cols, int threads, const v
     // what a block pays to start (half a row to fill its window, 3.5 where it
     // also fills the sine table) and, as blocks do not end together, some 15% of
     // a segment.  Power-of-two segments left the last wave up to three quarters
-    // empty: per sweep 3D Heisenberg L = 256 166 us, now 143 (k = 2; 155, 144,
+    // empty: per sweep 3D Heisenberg L = 256 166 us, these 143 (k = 2; 155, 144,
     // 147 for k = 1, 3, 4), L = 128 55 and 23; 2D XY L = 4096 105 and 92 (k = 1),
-    // L = 2048 46 and 30.  Ising kernels keep equal segments of 2^i rows: the row
+    // L = 2048 46 and 30 (before sums kept what rounding takes: LongSum).  Ising kernels keep equal segments of 2^i rows: the row
     // loop's end must be the same for a whole warp, or its addresses and keys
     // leave the uniform registers (64 registers a thread became 78, and L = 16384
     // 247 us a sweep became 255).

@@ -24,8 +24,8 @@
 //         FP64 weights ln W (u < exp(lnW(k) - lnW(k')) 2^32 as an exact
 //         integer test); H counts the level after every attempt.
 //   WL:   accept iff D >= 0 or u < exp(D 2^-32) 2^32, D = S(k) - S(k'): an
-//         FP32 exp2 decides unless u lies within 2^-14 (relative) of the
-//         threshold, where FP64 exp decides; after every attempt
+//         FP32 exp2 decides unless u 2^-32 lies within 2^-16 of exp(D 2^-32),
+//         where FP64 exp decides; after every attempt
 //         S(k) += 2^(32 - stage), H(k) += 1, level k is marked visited;
 //         after every sweep a walker whose visited levels all have
 //         H(k) * nvisited * 100 >= flat_percent * sum H moves to the next
