@@ -1,8 +1,8 @@
 """Calls of few sweeps on byte lattices that fit the chip's shared memory.  Loading a
 large one, above all its couplings, takes longer than a sweep, so such calls run on the
 streaming kernel; the choice by the length of the call changes no chain, and a call of
-one sweep takes no longer than on the streaming kernel (a tenth is allowed for what two
-timings differ by)."""
+one sweep takes no longer than on the streaming kernel (15% is allowed: equal launches
+back to back can differ by a step of 2 us a call; the load took 20 to 33%)."""
 import time
 
 import numpy as np
@@ -56,4 +56,4 @@ def test_single_sweeps_cost_no_more_than_streaming(sm, d, L):
                 took[k].append(time.perf_counter() - t0)
     for lat in lats:
         lat.close()
-    assert min(took[0]) < 1.1 * min(took[1])
+    assert min(took[0]) < 1.15 * min(took[1])
