@@ -59,6 +59,10 @@ def libraries():
     import __graft_entry__
     __graft_entry__.build()
     from paper_1107_5463_gb300 import build
+    objects = {os.path.basename(s)[:-3]: os.path.join(build.OUT, os.path.basename(s)[:-3] + ".o")
+               for s in build._sources()}
+    if not all(os.path.exists(o) for o in objects.values()):
+        build.build(force=True)
     os.makedirs(OUT, exist_ok=True)
     base = [build.nvcc()] + build.ARCH
 
@@ -74,8 +78,7 @@ def libraries():
     libs = {}
     for name, define in (("ising_res", "-DcudaLaunchCooperativeKernel=standin_launch"),
                          ("lattice", "-DcudaStreamBeginCapture=standin_capture")):
-        objs = [os.path.join(build.OUT, os.path.basename(s)[:-3] + ".o") for s in build._sources()
-                if os.path.basename(s) != name + ".cu"]
+        objs = [o for s, o in objects.items() if s != name]
         objs += [standin, obj(os.path.join(build.CSRC, name + ".cu"), name, [define])]
         libs[name] = os.path.join(OUT, "libspinmc_refused_%s.so" % name)
         subprocess.run(base + ["-shared", "-o", libs[name]] + objs + ["-cudart", "static"],
